@@ -595,10 +595,18 @@ int chunk_for_kind(int kind)
     return kind_is_mixed(kind) ? CHUNK_F32 : CHUNK_F64;
 }
 
-// Work per (primitive pair, charge) of a class with L = l_A + l_B: the flop model that splits the
-// SMs between the concurrent class sweeps until qmmm_autotune measures the real costs.
-double class_weight(int L, bool grad)
+// Work per (primitive pair, charge) of a class with L = l_A + l_B: the model that splits the SMs
+// between the concurrent class sweeps until qmmm_autotune measures the real costs.  FP64: the
+// FP64 instructions of the harmonic kernels (the solid harmonics' recursion, one multiply-add per
+// harmonic and sum, Boys function and displacement; a fifth of the steps with the Gaussian terms);
+// mixed: the flop model of the Hermite recursion and its contractions.
+double class_weight(int L, int kind)
 {
+    const bool grad = kind_is_grad(kind);
+    if (!kind_is_mixed(kind)) {
+        const double n = (L + 1) * (L + 1), near = nherm(L) - n + 30, walk = L < 2 ? 0.0 : 2.6 * L * L + 1.5 * L - 6.0;
+        return grad ? 41 + 8 * L + walk + 2 * n + 3 * L * L + 0.4 * near : 15 + 2 * L + walk + n + 0.2 * near;
+    }
     auto c4 = [](int n) { return n >= 4 ? (double)n * (n - 1) * (n - 2) * (n - 3) / 24.0 : 0.0; };
     auto c3 = [](int n) { return n >= 3 ? (double)n * (n - 1) * (n - 2) / 6.0 : 0.0; };
     return grad ? 75 + 3 * L + 2 * c4(L + 5) + 14 * c3(L + 3) : 40 + 3 * L + 2 * c4(L + 4) + 2 * c3(L + 3);
@@ -613,7 +621,7 @@ int sweep_kind(const qmmm_handle *h, bool grad)
 void reset_tuning(qmmm_handle *h, int kind)
 {
     for (int c = 0; c < NCLASS; ++c) {
-        h->cls_cost[kind][c] = class_weight(la_of_class(c) + lb_of_class(c), kind_is_grad(kind));
+        h->cls_cost[kind][c] = class_weight(la_of_class(c) + lb_of_class(c), kind);
         h->cls_variant[kind][c] = 0;
         h->cls_ms[kind][c] = 0.0;
     }

@@ -29,9 +29,7 @@ constexpr double HALF_SQRT_PI = 0.88622692545275801365;
 // Boys tables (rows T_k = k * step; columns m = 0..NCOL-2, last column e^{-T_k})
 constexpr double BOYS_STEP = 0.1;
 constexpr double BOYS_INV_STEP = 10.0;
-constexpr double BOYS_TMAX_D = 60.0;          // FP64 table range; above: asymptotic branch, where
-                                              // e^{-T} < 1e-26 is below FP64 resolution of F_m, m <= 8
-constexpr int BOYS_NROW_D = 601;
+constexpr int BOYS_NROW_D = 601;              // FP64 table range T <= 60, above every harm_tmax (harm.cuh)
 constexpr int BOYS_NCOL_D = 17;               // host table: orders 0..15 + exp column
 constexpr int BOYS_TAYLOR_D = 7;              // terms of the FP64 Taylor expansion
 constexpr int BOYS_ROW_D = 8;                 // device row for order M: F_{M+j}(T_k) / j!, j = 0..6,
@@ -85,46 +83,6 @@ __host__ __device__ constexpr int class_of(int la, int lb) { return la * (la + 1
 // ------------------------------------------------------------------------------------------
 // Boys function
 // ------------------------------------------------------------------------------------------
-// F_m(T), m = 0..M.  tab holds one table per order M (BOYS_NROW_D rows of BOYS_ROW_D): for
-// T < BOYS_TMAX_D a 7-term Taylor expansion about the nearest T_k with the 1/j! folded into the
-// table (Horner with one FMA per term), then the stable downward recursion; above, F_0 from its
-// asymptotic form and the upward recursion, which is exact there up to e^{-T}.
-template <int M>
-__device__ __forceinline__ void boys_f64(double T, double (&F)[M + 1], const double *__restrict__ tab)
-{
-    if (T < BOYS_TMAX_D) {
-        const int k = __double2int_rn(T * BOYS_INV_STEP);
-        const double x = (double)k * BOYS_STEP - T;  // -(T - T_k)
-        const double2 *row =
-            reinterpret_cast<const double2 *>(tab + ((size_t)M * BOYS_NROW_D + k) * BOYS_ROW_D);
-        const double2 c01 = __ldg(row), c23 = __ldg(row + 1), c45 = __ldg(row + 2), c6e = __ldg(row + 3);
-        double f = fma(c6e.x, x, c45.y);
-        f = fma(f, x, c45.x);
-        f = fma(f, x, c23.y);
-        f = fma(f, x, c23.x);
-        f = fma(f, x, c01.y);
-        f = fma(f, x, c01.x);
-        F[M] = f;
-        if (M > 0) {
-            // e^{-T} = e^{-T_k} e^{x}, |x| <= 0.05: 8-term Taylor of e^x
-            double ex = 1.0 + x * (1.0 + x * (0.5 + x * (1.0 / 6.0 + x * (1.0 / 24.0 + x * (1.0 / 120.0 +
-                        x * (1.0 / 720.0 + x * (1.0 / 5040.0)))))));
-            const double e = c6e.y * ex;
-            const double T2 = 2.0 * T;
-#pragma unroll
-            for (int m = M; m > 0; --m) F[m - 1] = (T2 * F[m] + e) * (1.0 / (2 * m - 1));
-        }
-    } else {
-        const double rs = rsqrt(T);
-        F[0] = HALF_SQRT_PI * rs;
-        if (M > 0) {
-            const double inv2T = 0.5 * rs * rs;
-#pragma unroll
-            for (int m = 0; m < M; ++m) F[m + 1] = ((2 * m + 1) * inv2T) * F[m];
-        }
-    }
-}
-
 // rho * (X^2 + Y^2 + Z^2) as an unevaluated sum Th + Tl: squares split exactly with FMA and the
 // three-term sum and the product by rho carried with two-sum / two-product error terms, so T is
 // accurate to about one FP32 rounding of T itself (the per-charge rounding error of r^2 is what
@@ -194,45 +152,6 @@ __device__ __forceinline__ void boys_f32(float T, float (&F)[M + 1], const float
 #pragma unroll
             for (int m = 0; m < M; ++m) F[m + 1] = fmaf((float)(2 * m + 1), F[m], -e) * inv2T;
         }
-    }
-}
-
-// ------------------------------------------------------------------------------------------
-// Hermite R tensors, in place: on entry Fn[n] = pref * (-2 rho)^n F_n(T) for n = 0..L;
-// on exit R[hidx(t,u,v)] = pref * R_tuv for t+u+v <= L.  Each level n is built from level n+1
-// in decreasing total order, so entries of order k only read orders k-1 and k-2 that still
-// hold level n+1 values.
-// ------------------------------------------------------------------------------------------
-template <int L, typename T>
-__device__ __forceinline__ void hermite_R(T (&R)[nherm(L)], const T (&Fn)[L + 1], T X, T Y, T Z)
-{
-    R[0] = Fn[L];
-#pragma unroll
-    for (int n = L - 1; n >= 0; --n) {
-#pragma unroll
-        for (int k = L - n; k >= 1; --k) {
-#pragma unroll
-            for (int t = k; t >= 0; --t) {
-#pragma unroll
-                for (int u = k - t; u >= 0; --u) {
-                    const int v = k - t - u;
-                    if (t > 0) {
-                        T r = X * R[hidx(t - 1, u, v)];
-                        if (t > 1) r += (T)(t - 1) * R[hidx(t - 2, u, v)];
-                        R[hidx(t, u, v)] = r;
-                    } else if (u > 0) {
-                        T r = Y * R[hidx(t, u - 1, v)];
-                        if (u > 1) r += (T)(u - 1) * R[hidx(t, u - 2, v)];
-                        R[hidx(t, u, v)] = r;
-                    } else {
-                        T r = Z * R[hidx(t, u, v - 1)];
-                        if (v > 1) r += (T)(v - 1) * R[hidx(t, u, v - 2)];
-                        R[hidx(t, u, v)] = r;
-                    }
-                }
-            }
-        }
-        R[0] = Fn[n];
     }
 }
 

@@ -246,8 +246,11 @@ __host__ __device__ constexpr int cl_variant(int L, int v, int field)
     return (L >= 0 && L <= 6) ? T[L][v][field] : 0;
 }
 
-// Hermite R tensors as hermite_R, with every loop of constant trip count (bounds as guards) so
-// that the nest unrolls completely and R stays in registers.
+// Hermite R tensors of the mixed sweeps, in place: on entry Fn[n] = pref (-2 rho)^n F_n(T) for
+// n = 0..L; on exit R[hidx(t,u,v)] = pref R_tuv for t+u+v <= L.  Each level n is built from level
+// n+1 in decreasing total order, so entries of order k only read orders k-1 and k-2 that still
+// hold level n+1 values.  Every loop has a constant trip count (bounds as guards) so that the nest
+// unrolls completely and R stays in registers.
 template <int L, typename T>
 __device__ __forceinline__ void hermite_R_u(T (&R)[nherm(L)], const T (&Fn)[L + 1], T X, T Y, T Z)
 {

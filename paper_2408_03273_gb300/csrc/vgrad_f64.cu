@@ -6,17 +6,29 @@
 // with g_ab the density element (plus its mirror) times the pair prefactor and
 //   E'^{ij}_t = dE^{ij}_t / dX_AB = 2a E^{i+1,j}_t - i E^{i-1,j}_t - (a/p) E^{ij}_{t-1}.
 // Moving A shifts P by a/p, so with e_a = sum D0_tuv R_{tuv + 1_a} and d_a = sum Da_tuv R_tuv
-// (R recomputed up to L+1 for every charge, never stored):
+// (recomputed for every charge, never stored):
 //   dI/dA_a = d_a + (a/p) e_a,   dI/dB_a = -d_a + (b/p) e_a,   dI/dC_a = -e_a,
-// and E contains -q_C I.  The d_a enter only through sum_C q_C d_a(C) = sum Da_tuv S_tuv with
-// S_tuv = sum_C q_C R_tuv, so up to L = 4 the sweep accumulates S (NH terms per charge instead
-// of the 3 NH of the three contractions) and Da is formed and contracted once per pair after it
-// (contract_dA); for L >= 5 the three contractions stay in the loop (see CSUM).
+// and E contains -q_C I.  The d_a enter only through sum_C q_C d_a(C) = sum Da_tuv W_tuv with
+// W_tuv = sum_C q_C R_tuv, so the sweep accumulates the charge sums and Da is formed and contracted
+// once per pair after it (contract_dA).
+//
+// Bound: the FP64 pipe, 2 lanes per clock and SM, 85-91% busy, with 7-8% of the issue slots used: the
+// kernel's time is its count of FP64 instructions.  So the tensors R are never formed: D0 and W are
+// kept as solid-harmonic components (harm.cuh), per charge one recursion of (L+1)^2 harmonics, one
+// multiply-add per harmonic for the value, the charge sum and each gradient component (these with
+// the coefficients N of the differentiated harmonics, one order lower).  FP64 instructions per
+// (warp, charge) on a 60-atom active site, setup included: (s,s) 30, (p,p) 77, (d,s) 87, (d,p) 141,
+// (d,d) 262.  Coefficients and sums of the high classes spill to local memory ((f,f): 4.7 KB
+// stores), which the idle load pipe carries.  Adjoint sweep against the Hermite recursion with its
+// contractions: active site 78.3 -> 60.9 ms, a 150-atom site with f shells 412 -> 242 ms, a QM
+// water 1.35 -> 0.82 ms (untuned handles).
+//
 // Per-pair sums over charges stay in registers; per-charge sums over the
 // 32 primitive pairs of a tile use a warp butterfly and go to shared-memory accumulators that
 // are flushed to global memory once per block.
 #include <algorithm>
 
+#include "harm.cuh"
 #include "pp_tile.cuh"
 
 namespace qmmm {
@@ -37,7 +49,7 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
             const double *__restrict__ boys, const double *__restrict__ dm, double *__restrict__ gqm,
             double *__restrict__ gchg, int *err)
 {
-    constexpr int L = LA + LB, NH = nherm(L), NH1 = nherm(L + 1);
+    constexpr int L = LA + LB, NH = nherm(L), NG = nhgrad(L) + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t bar;
     {
@@ -58,78 +70,59 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
     for (int tile = blockIdx.x * nwarp + warp; tile < ntile; tile += gridDim.x * nwarp) {
         const PPLane pl = load_pp(bd, pp_begin + tile * 32 + lane, pp_end);
         const double aop = pl.a * pl.ip, bop = pl.b * pl.ip;
-        double D0[NH];
-        // L <= 4: S_tuv = sum_C q_C R_tuv(P - C), contracted with the centre-A derivative
-        // coefficients once per pair after the charge sweep.  L >= 5 (f shells with d or f): S
-        // would be read and written every charge from a register file already full, so there
-        // the derivative coefficients are contracted per charge (only read in the loop).
-        constexpr bool CSUM = L <= 4;
-        double S[CSUM ? NH : 1], Dx[CSUM ? 1 : NH], Dy[CSUM ? 1 : NH], Dz[CSUM ? 1 : NH];
-        if constexpr (CSUM) {
+        // the density-folded Hermite coefficients as harmonic ones, their gradients, and the charge
+        // sums S (harm.cuh); unit: the unit of the harmonic factors
+        const double unit = HALF_SQRT_PI * sqrt(pl.ip);
+        double M[NH], Nx[NG], Ny[NG], Nz[NG], S[NH];
+        {
+            double D0[NH];
             fold_density<LA, LB>(pl, bd, dm, D0);
 #pragma unroll
-            for (int k = 0; k < NH; ++k) S[k] = 0.0;
-        } else {
-            fold_density_dA<LA, LB, true>(pl, bd, dm, Dx, Dy, Dz, D0);
+            for (int k = 0; k < NH; ++k) D0[k] *= unit;
+            harm_fold<L>(D0, M);
+            harm_grad<L>(M, Nx, Ny, Nz);
         }
+#pragma unroll
+        for (int k = 0; k < NH; ++k) S[k] = 0.0;
 
-        double sex = 0, sey = 0, sez = 0, sdx = 0, sdy = 0, sdz = 0;
+        double sex = 0, sey = 0, sez = 0;
         for (int c = 0; c < rg.ncls; ++c) {
             const int lo = max(__ldg(rg.cls_off + c), ch_begin) - ch_begin;
             const int hi = min(__ldg(rg.cls_off + c + 1), ch_end) - ch_begin;
             if (lo >= hi) continue;
             const double kap = __ldg(rg.cls_kappa + c);
-            const double t = kap > 0.0 ? kap / (pl.p + kap) : 1.0;
-            const double rho = pl.p * t, m2rho = -2.0 * rho, sq = sqrt(t);
+            const double rho = kap > 0.0 ? pl.p * (kap / (pl.p + kap)) : pl.p;
+            const double c0 = sqrt(rho) / HALF_SQRT_PI;
+            const double rfar = harm_tmax(L + 1) / rho;
             for (int j = lo; j < hi; ++j) {
                 const double4_32a ch = chg[j];
                 const double X = pl.P[0] - ch.x, Y = pl.P[1] - ch.y, Z = pl.P[2] - ch.z;
-                const double T = rho * (X * X + Y * Y + Z * Z);
-                double F[L + 2];
-                boys_f64<L + 1>(T, F, boys);
-                double Fn[L + 2];
-                double sc = sq;
-#pragma unroll
-                for (int n = 0; n <= L + 1; ++n) {
-                    Fn[n] = sc * F[n];
-                    sc *= m2rho;
-                }
-                double R[NH1];
-                hermite_R<L + 1, double>(R, Fn, X, Y, Z);
-                double e0 = 0, ex = 0, ey = 0, ez = 0, dx = 0, dy = 0, dz = 0;
+                const double r2 = X * X + Y * Y + Z * Z;
+                const bool far = harm_far(r2, rfar);
+                double e0, ex, ey, ez;
                 const double q = ch.w;
+                if (__all_sync(FULL, far)) {
+                    double F[L + 1];
+                    const double y = harm_rsqrt(r2), y2 = y * y;
+                    F[0] = y;
 #pragma unroll
-                for (int t = 0; t <= L; ++t)
-#pragma unroll
-                    for (int u = 0; u <= L - t; ++u)
-#pragma unroll
-                        for (int w = 0; w <= L - t - u; ++w) {
-                            const int k = hidx(t, u, w);
-                            e0 += D0[k] * R[k];
-                            ex += D0[k] * R[hidx(t + 1, u, w)];
-                            ey += D0[k] * R[hidx(t, u + 1, w)];
-                            ez += D0[k] * R[hidx(t, u, w + 1)];
-                            if constexpr (CSUM) {
-                                S[k] += q * R[k];
-                            } else {
-                                dx += Dx[k] * R[k];
-                                dy += Dy[k] * R[k];
-                                dz += Dz[k] * R[k];
-                            }
-                        }
-                sex += q * ex; sey += q * ey; sez += q * ez;
-                if constexpr (!CSUM) {
-                    sdx += q * dx; sdy += q * dy; sdz += q * dz;
+                    for (int l = 1; l <= L; ++l) F[l] = F[l - 1] * y2;
+                    harm_eval<L, false>(M, Nx, Ny, Nz, F, 0.0, 0.0, y2, X, Y, Z, r2, q, S, e0, ex, ey, ez);
+                } else {
+                    double F[L + 2], E0;
+                    boys_hat<L + 1>(far, r2, rho, c0, F, E0, boys);
+                    harm_eval<L, true>(M, Nx, Ny, Nz, F, E0, rho, 0.0, X, Y, Z, r2, q, S, e0, ex, ey, ez);
                 }
-                // per-charge sums over the 32 primitive pairs of (dE/dC_x, dE/dC_y, dE/dC_z, dE/dq) =
-                // (q e_x, q e_y, q e_z, -e0): halve the four values twice (each lane keeps one
-                // component summed over 4 lanes), then a 3-step butterfly; lane 8c ends with
-                // component c.  6 FP64 additions instead of 4 full warp sums (20).
+                sex += q * ex; sey += q * ey; sez += q * ez;
+                // per-charge sums over the 32 primitive pairs of (e_x, e_y, e_z, e_0), whose
+                // factors (q, q, q, -1) in (dE/dC, dE/dq) are applied when the block's sums leave:
+                // halve the four values twice (each lane keeps one component summed over 4
+                // lanes), then a 3-step butterfly; lane 8c ends with component c.  6 FP64
+                // additions instead of 4 full warp sums (20).
                 {
-                    const double v0 = q * ex, v1 = q * ey, v2 = q * ez, v3 = -e0;
                     const bool up = lane & 16;
-                    double k0 = up ? v2 : v0, k1 = up ? v3 : v1;
-                    const double s0 = up ? v0 : v2, s1 = up ? v1 : v3;
+                    double k0 = up ? ez : ex, k1 = up ? e0 : ey;
+                    const double s0 = up ? ex : ez, s1 = up ? ey : e0;
                     k0 += __shfl_xor_sync(FULL, s0, 16);
                     k1 += __shfl_xor_sync(FULL, s1, 16);
                     const bool up8 = lane & 8;
@@ -142,16 +135,17 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
                 }
             }
         }
-        if constexpr (CSUM) {
-            double sd[3];
-            contract_dA<LA, LB>(pl, bd, dm, S, sd);
-            sdx = sd[0];
-            sdy = sd[1];
-            sdz = sd[2];
+        double sd[3];
+        {
+            double W[NH];
+            harm_unfold<L>(S, W);
+#pragma unroll
+            for (int k = 0; k < NH; ++k) W[k] *= unit;
+            contract_dA<LA, LB>(pl, bd, dm, W, sd);
         }
         // dE/dA = -(sd + a/p se), dE/dB = sd - b/p se
-        double g[6] = {-(sdx + aop * sex), -(sdy + aop * sey), -(sdz + aop * sez),
-                       sdx - bop * sex, sdy - bop * sey, sdz - bop * sez};
+        double g[6] = {-(sd[0] + aop * sex), -(sd[1] + aop * sey), -(sd[2] + aop * sez),
+                       sd[0] - bop * sex, sd[1] - bop * sey, sd[2] - bop * sez};
         bool take[5], head;
         seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
 #pragma unroll
@@ -166,7 +160,7 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
     }
     __syncthreads();
     for (int k = threadIdx.x; k < 4 * nch; k += blockDim.x) {
-        const double v = acc[k];
+        const double v = (k & 3) < 3 ? chg[k >> 2].w * acc[k] : -acc[k];
         if (v != 0.0) atomicAdd(gchg + 4 * (size_t)ch_begin + k, v);
     }
 }

@@ -5,15 +5,19 @@
 //
 // A warp owns 32 primitive pairs of one angular class; the block stages a chunk of region-I
 // charges (x, y, z, q) into shared memory with one TMA bulk copy, every lane sweeps all of them
-// (shared-memory broadcast) and accumulates the Hermite sums W_tuv = sum_C q_C s_C R_tuv in
-// registers.  Charges are grouped by Gaussian width so that rho and sqrt(kappa/(p+kappa)) are
-// computed once per (primitive pair, width class).  The E-contraction runs once per primitive
-// pair; primitive pairs of a shell pair are summed by a segmented warp-shuffle reduction and the
-// head lane adds the block into V (and its mirror).  A shell pair spans at most two tiles when
-// it has at most 32 primitive pairs, so at most two additions reach any element: the result does
-// not depend on scheduling.
+// (shared-memory broadcast) and accumulates W_tuv = sum_C q_C s_C R_tuv in registers, as
+// solid-harmonic components (harm.cuh).  The bound is the FP64 pipe (90% busy, 8% of the issue
+// slots used), so the kernel's time is its count of FP64 instructions: per (warp, charge) 13 for
+// (s,s), 38 (d,s), 106 (d,d) on a 60-atom active site.  V sweep against the Hermite recursion:
+// active site 33.5 -> 24.4 ms, a 150-atom site with f shells 147 -> 104 ms, a QM water 0.43 ->
+// 0.33 ms (untuned handles).  Charges are grouped by Gaussian width so that rho is formed once per
+// (primitive pair, width class).  The E-contraction runs once per primitive pair; primitive pairs
+// of a shell pair are summed by a segmented warp-shuffle reduction and the head lane adds the block
+// into V (and its mirror).  A shell pair spans at most two tiles when it has at most 32 primitive
+// pairs, so at most two additions reach any element: the result does not depend on scheduling.
 #include <algorithm>
 
+#include "harm.cuh"
 #include "pp_tile.cuh"
 
 namespace qmmm {
@@ -52,42 +56,40 @@ k_vpot_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, in
     const int ntile = (pp_end - pp_begin + 31) >> 5;
     for (int tile = blockIdx.x * nwarp + warp; tile < ntile; tile += gridDim.x * nwarp) {
         const PPLane pl = load_pp(bd, pp_begin + tile * 32 + lane, pp_end);
-        double W[NH];
+        double S[NH];  // harmonic sums (harm.cuh)
 #pragma unroll
-        for (int k = 0; k < NH; ++k) W[k] = 0.0;
+        for (int k = 0; k < NH; ++k) S[k] = 0.0;
 
         for (int c = 0; c < rg.ncls; ++c) {
             const int lo = max(__ldg(rg.cls_off + c), ch_begin) - ch_begin;
             const int hi = min(__ldg(rg.cls_off + c + 1), ch_end) - ch_begin;
             if (lo >= hi) continue;
             const double kap = __ldg(rg.cls_kappa + c);
-            const double t = kap > 0.0 ? kap / (pl.p + kap) : 1.0;
-            const double rho = pl.p * t, m2rho = -2.0 * rho, sq = sqrt(t);
+            const double rho = kap > 0.0 ? pl.p * (kap / (pl.p + kap)) : pl.p;
+            const double c0 = sqrt(rho) / HALF_SQRT_PI;
+            const double rfar = harm_tmax(L) / rho;
             for (int j = lo; j < hi; ++j) {
                 const double4_32a ch = chg[j];
                 const double X = pl.P[0] - ch.x, Y = pl.P[1] - ch.y, Z = pl.P[2] - ch.z;
-                const double T = rho * (X * X + Y * Y + Z * Z);
-                double F[L + 1];
-                boys_f64<L>(T, F, boys);
-                double Fn[L + 1];
-                double sc = ch.w * sq;
-#pragma unroll
-                for (int n = 0; n <= L; ++n) {
-                    Fn[n] = sc * F[n];
-                    sc *= m2rho;
+                const double r2 = X * X + Y * Y + Z * Z;
+                const bool far = harm_far(r2, rfar);
+                if (__all_sync(FULL, far)) {
+                    harm_add_far<L>(S, ch.w, X, Y, Z, r2);
+                } else {
+                    double F[L + 1], E0;
+                    boys_hat<L>(far, r2, rho, c0, F, E0, boys);
+                    harm_add<L, true>(S, F, E0, rho, ch.w, X, Y, Z, r2);
                 }
-                double R[NH];
-                hermite_R<L, double>(R, Fn, X, Y, Z);
-#pragma unroll
-                for (int k = 0; k < NH; ++k) W[k] += R[k];
             }
         }
+        double W[NH];
+        harm_unfold<L>(S, W);
 
         double Ex[LA + 1][LB + 1][L + 1], Ey[LA + 1][LB + 1][L + 1], Ez[LA + 1][LB + 1][L + 1];
         hermite_E<LA, LB, double>(Ex, pl.P[0] - pl.A[0], pl.P[0] - pl.B[0], 0.5 * pl.ip);
         hermite_E<LA, LB, double>(Ey, pl.P[1] - pl.A[1], pl.P[1] - pl.B[1], 0.5 * pl.ip);
         hermite_E<LA, LB, double>(Ez, pl.P[2] - pl.A[2], pl.P[2] - pl.B[2], 0.5 * pl.ip);
-        const double coef = -TWO_PI * pl.ip * pl.cab;
+        const double coef = -TWO_PI * pl.ip * pl.cab * HALF_SQRT_PI * sqrt(pl.ip);
 
         bool take[5], head;
         seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
