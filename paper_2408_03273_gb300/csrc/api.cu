@@ -670,35 +670,76 @@ bool split_sms(const qmmm_handle *h, int kind, const int *variant, int *share, i
     return true;
 }
 
-// Launch the sweep of every non-empty angular class concurrently: each class on its own stream,
-// forked from and joined back into the handle's stream, its grid capped at its share of the SMs
-// (so small classes do not leave most SMs idle while they run alone).  With maxsl > 1 (sweeps
-// over nch charges; V sweeps then write slice s of a class into partial matrix s) every class
-// picks its own charge slices (class_slices), and a class with fewer tiles than its share of the
-// SMs may take up to maxsl times its tile count in blocks.
-template <typename F>
-int run_classes(qmmm_handle *h, int kind, F launch, int nslice = 1, int maxsl = 1, int nch = 0, bool join = true)
+// Most charge slices of a class sweep.
+constexpr int MAX_SLICES = 16;
+
+// Per-pair work of a sweep outside its charge loop, in charges of loop work: the Hermite and
+// density algebra, FP64 in both precisions (against an FP32 charge loop on the mixed path).
+double setup_charges(int L, int kind)
 {
-    int share[NCLASS];
-    if (!split_sms(h, kind, h->cls_variant[kind], share, nslice == 1 ? maxsl : 1)) return QMMM_OK;
-    CUDA_TRY(cudaEventRecord(h->fork, h->stream));
-    // the charge-lane sweeps (mixed adjoint) size their own fine-grained grids and are launched
-    // highest class first (their blocks are the longest), so that the short low-l blocks fill the tail
+    if (kind_is_mixed(kind)) return 64.0;
+    return kind_is_grad(kind) ? 3.0 + 1.5 * L * L : 3.0 + 0.6 * L * L;
+}
+
+// How the classes of a sweep over nch charges are cut into blocks: charge slices per class, launch
+// order and warps per block.
+struct Cut {
+    int ns[NCLASS], order[NCLASS], threads[NCLASS];
+    int most = 1;  // slices of the most sliced class
+};
+Cut cut_classes(const qmmm_handle *h, int kind, int nch)
+{
+    Cut k;
+    int tiles[NCLASS];
+    double w[NCLASS], setup[NCLASS];
+    for (int c = 0; c < NCLASS; ++c) {
+        tiles[c] = (h->class_off[c + 1] - h->class_off[c] + 31) / 32;
+        w[c] = std::max(h->cls_cost[kind][c], 1e-30);
+        setup[c] = setup_charges(la_of_class(c) + lb_of_class(c), kind);
+    }
+    const size_t n2 = (size_t)h->nao * h->nao;
+    fine_slices(NCLASS, tiles, w, setup, nch, h->nsm, kind_is_grad(kind) ? MAX_SLICES : vpot_slice_cap(n2, MAX_SLICES),
+                k.ns);
+    slice_order(NCLASS, tiles, w, k.ns, k.order);
+    long long warps = 0;
+    for (int c = 0; c < NCLASS; ++c) {
+        warps += (long long)tiles[c] * k.ns[c];
+        k.most = std::max(k.most, k.ns[c]);
+    }
+    // few warps in all: four to a block, one per SM sub-partition (each has its own FP64 pipe)
+    for (int c = 0; c < NCLASS; ++c) {
+        k.threads[c] = variant_threads(kind, c, h->cls_variant[kind][c]);
+        if (warps <= 4LL * h->nsm) k.threads[c] = 128;
+    }
+    return k;
+}
+
+// Launch the sweep of every non-empty angular class concurrently, each class on its own stream,
+// forked from and joined back into the handle's stream.  A class is cut into blocks of one tile per
+// warp and one charge slice (cut_classes; V sweeps write slice s of a class into partial matrix s)
+// and the classes are launched in order of falling block time, so that the block scheduler packs
+// the blocks onto the SMs as they fall free, whatever a class really costs.  (One block per SM of a
+// class's share, the shares from the work model, left SMs idle once a class finished early.
+// Untuned FP64 adjoint / V / mixed V: 60-atom site 60.9 -> 45.0 / 24.4 -> 19.8 / 1.86 -> 1.29 ms,
+// 150-atom site 242 -> 194 / 104 -> 85 / 8.0 -> 5.6 ms, QM water adjoint 0.82 -> 0.53 ms.)
+// The mixed adjoint (charge lanes) sizes its own grids, highest class first.
+template <typename F>
+int run_classes(qmmm_handle *h, int kind, F launch, int nch = 0, bool join = true)
+{
+    if (h->n_pp == 0) return QMMM_OK;
     const bool cl = kind == SW_VGRAD_F32;
+    const Cut k = cut_classes(h, kind, nch);
+    int share[NCLASS];
+    split_sms(h, kind, h->cls_variant[kind], share);
+    CUDA_TRY(cudaEventRecord(h->fork, h->stream));
     for (int i = 0; i < NCLASS; ++i) {
-        const int c = cl ? NCLASS - 1 - i : i;
+        const int c = cl ? NCLASS - 1 - i : k.order[i];
         const int p0 = h->class_off[c], p1 = h->class_off[c + 1];
         if (p1 <= p0) continue;
-        int sh = share[c], ns = nslice;
-        if (nslice == 1 && maxsl > 1) {
-            const int nwarp = variant_threads(kind, c, h->cls_variant[kind][c]) / 32;
-            // per-pair setup in charges of sweep work: FP64 Hermite/density setup against an FP64
-            // charge loop (~1%), or against an FP32 one (several percent)
-            const double setup = kind_is_mixed(kind) ? 64.0 : 16.0;
-            class_slices((p1 - p0 + 31) / 32, nwarp, sh, nch, maxsl, setup, &sh, &ns);
-        }
         CUDA_TRY(cudaStreamWaitEvent(h->side[c], h->fork, 0));
-        CUDA_TRY(launch(c, p0, p1, sh, h->cls_variant[kind][c], ns, h->side[c]));
+        const int nwarp = k.threads[c] / 32, blocks = ((p1 - p0 + 31) / 32 + nwarp - 1) / nwarp;
+        CUDA_TRY(launch(c, p0, p1, cl ? share[c] : blocks, cl ? h->cls_variant[kind][c] : k.threads[c], cl ? 1 : k.ns[c],
+                        h->side[c]));
         CUDA_TRY(cudaEventRecord(h->join[c], h->side[c]));
     }
     if (join)
@@ -733,22 +774,6 @@ int fork_classes(qmmm_handle *h, F launch)
     return QMMM_OK;
 }
 
-// Charge slices of a sweep: when the classes together ask for fewer than half the SMs (a small
-// QM region: few 32-pair tiles), the charge chunk is split over up to 8 block rows so that the
-// work spreads over more SMs (at least 64 charges per slice).
-int sweep_slices(const qmmm_handle *h, int kind, int nch)
-{
-    int share[NCLASS];
-    if (!split_sms(h, kind, h->cls_variant[kind], share)) return 1;
-    int blocks = 0;
-    for (int c = 0; c < NCLASS; ++c) blocks += share[c];
-    int ns = blocks > 0 ? h->nsm / blocks : 1;
-    ns = std::min(ns, std::min(8, nch / 64));
-    return std::max(ns, 1);
-}
-
-// One class sweep of the given kind over region-I charges [c0, c1), split into nslice block rows;
-// V kernels write slice s into V + s * vstride.
 // Scratch of the charge-lane adjoint sweep for every class that takes it (allocated on first use).
 int ensure_cl(qmmm_handle *h)
 {
@@ -767,21 +792,24 @@ int ensure_cl(qmmm_handle *h)
     return QMMM_OK;
 }
 
-cudaError_t launch_sweep(const qmmm_handle *h, int kind, int cls, int p0, int p1, int c0, int c1, int share,
-                         int variant, int nslice, size_t vstride, const double *ddm, double *V, double *gqm,
+// One class sweep of the given kind over region-I charges [c0, c1): nblk blocks of `threads` threads
+// in each of nslice block rows (the mixed adjoint: its variant in place of `threads`); V kernels
+// write slice s into V + s * vstride.
+cudaError_t launch_sweep(const qmmm_handle *h, int kind, int cls, int p0, int p1, int c0, int c1, int nblk,
+                         int threads, int nslice, size_t vstride, const double *ddm, double *V, double *gqm,
                          double *gchg, cudaStream_t cs)
 {
     const BasisDev b = h->basis();
     const RegionDev r = h->region();
     switch (kind) {
     case SW_VPOT_F64:
-        return launch_vpot_f64(b, r, cls, p0, p1, c0, c1, h->boys64.p, V, h->err.p, share, variant, nslice, vstride,
+        return launch_vpot_f64(b, r, cls, p0, p1, c0, c1, h->boys64.p, V, h->err.p, nblk, threads, nslice, vstride,
                                cs);
     case SW_VPOT_F32:
-        return launch_vpot_f32(b, r, cls, p0, p1, c0, c1, h->boys32.p, V, h->err.p, share, variant, nslice, vstride,
+        return launch_vpot_f32(b, r, cls, p0, p1, c0, c1, h->boys32.p, V, h->err.p, nblk, threads, nslice, vstride,
                                cs);
     case SW_VGRAD_F64:
-        return launch_vgrad_f64(b, r, cls, p0, p1, c0, c1, h->boys64.p, ddm, gqm, gchg, h->err.p, share, variant,
+        return launch_vgrad_f64(b, r, cls, p0, p1, c0, c1, h->boys64.p, ddm, gqm, gchg, h->err.p, nblk, threads,
                                 nslice, cs);
     case SW_VGRAD_F32: {
         ClScratch cl;
@@ -789,7 +817,7 @@ cudaError_t launch_sweep(const qmmm_handle *h, int kind, int cls, int p0, int p1
             cl.rec = h->cl_rec.p + h->cl_rec_off[cls];
             cl.psum = h->cl_psum.p + h->cl_psum_off[cls];
         }
-        return launch_vgrad_f32(b, r, cls, p0, p1, c0, c1, h->boys32.p, ddm, gqm, gchg, h->err.p, share, variant,
+        return launch_vgrad_f32(b, r, cls, p0, p1, c0, c1, h->boys32.p, ddm, gqm, gchg, h->err.p, nblk, threads,
                                 nslice, cl, cs);
     }
     default: return cudaErrorInvalidValue;
@@ -824,17 +852,16 @@ int time_best(qmmm_handle *h, cudaEvent_t e0, cudaEvent_t e1, F run, float *ms)
 int tune_launch(qmmm_handle *h, int kind, int cls, int share, int variant)
 {
     const int c1 = std::min(h->nI, std::min(chunk_for_kind(kind), TUNE_CHARGES));
-    auto one = [&](int c, int p0, int p1, int s, int v, int ns, cudaStream_t cs) {
-        return launch_sweep(h, kind, c, p0, p1, 0, c1, s, v, ns, 0, h->tune_dm.p, h->tune_V.p, h->tune_gqm.p,
+    auto one = [&](int c, int p0, int p1, int nblk, int threads, int ns, cudaStream_t cs) {
+        return launch_sweep(h, kind, c, p0, p1, 0, c1, nblk, threads, ns, 0, h->tune_dm.p, h->tune_V.p, h->tune_gqm.p,
                             h->tune_gchg.p, cs);
     };
     if (cls < 0) {
         // the slices of the real sweep (V slices all add into the one scratch matrix here)
-        const int maxsl = kind_is_grad(kind) ? std::max(1, std::min(8, c1 / 128))
-                                             : vpot_max_slices(c1, (size_t)h->nao * h->nao);
-        return run_classes(h, kind, one, 1, maxsl, c1);
+        return run_classes(h, kind, one, c1);
     }
-    CUDA_TRY(one(cls, h->class_off[cls], h->class_off[cls + 1], share, variant, 1, h->stream));
+    CUDA_TRY(one(cls, h->class_off[cls], h->class_off[cls + 1], share,
+                 kind == SW_VGRAD_F32 ? variant : variant_threads(kind, cls, variant), 1, h->stream));
     return QMMM_OK;
 }
 
@@ -1290,11 +1317,7 @@ static int vpot_prep(qmmm_handle *h, bool slices, double **Vdst, int *nbuf)
     *nbuf = 1;
     if (!slices) return QMMM_OK;
     const int kind = sweep_kind(h, false), ch = chunk_for_kind(kind);
-    const int ns = sweep_slices(h, kind, std::min(h->nI, ch));
-    // otherwise per-class charge slices (class_slices), as many as the per-slice partial
-    // matrices' memory allows
-    const int maxsl = ns > 1 ? 1 : vpot_max_slices(std::min(h->nI, ch), n2);
-    *nbuf = std::max(ns, maxsl);
+    for (int c0 = 0; c0 < h->nI; c0 += ch) *nbuf = std::max(*nbuf, cut_classes(h, kind, std::min(ch, h->nI - c0)).most);
     if (*nbuf > 1) {  // per-slice partial V, summed in a fixed order afterwards
         if ((rc = h->Vslices.ensure((size_t)*nbuf * n2))) return rc;
         CUDA_TRY(cudaMemsetAsync(h->Vslices.p, 0, (size_t)*nbuf * n2 * sizeof(double), st));
@@ -1309,17 +1332,15 @@ static int vpot_sweep(qmmm_handle *h, double *Vdst, int nbuf)
     int rc;
     const int kind = sweep_kind(h, false), ch = chunk_for_kind(kind);
     const size_t n2 = (size_t)h->nao * h->nao;
-    const int ns = sweep_slices(h, kind, std::min(h->nI, ch));
-    const int maxsl = ns > 1 ? 1 : vpot_max_slices(std::min(h->nI, ch), n2);
     for (int c0 = 0; c0 < h->nI; c0 += ch) {
         const int c1 = std::min(h->nI, c0 + ch);
         rc = run_classes(
             h, kind,
-            [&](int cls, int p0, int p1, int share, int variant, int nsl, cudaStream_t cs) {
-                return launch_sweep(h, kind, cls, p0, p1, c0, c1, share, variant, nsl, nbuf > 1 ? n2 : 0, nullptr,
+            [&](int cls, int p0, int p1, int nblk, int threads, int nsl, cudaStream_t cs) {
+                return launch_sweep(h, kind, cls, p0, p1, c0, c1, nblk, threads, nsl, nbuf > 1 ? n2 : 0, nullptr,
                                     Vdst, nullptr, nullptr, cs);
             },
-            ns, maxsl, c1 - c0);
+            c1 - c0);
         if (rc) return rc;
     }
     return QMMM_OK;
@@ -1461,16 +1482,15 @@ static int forces_sweep(qmmm_handle *h, const double *ddm)
     int rc;
     const int kind = sweep_kind(h, true), ch = chunk_for_kind(kind);
     if (kind == SW_VGRAD_F32 && (rc = ensure_cl(h))) return rc;
-    const int ns = sweep_slices(h, kind, std::min(h->nI, ch));
     for (int c0 = 0; c0 < h->nI; c0 += ch) {
         const int c1 = std::min(h->nI, c0 + ch);
         rc = run_classes(
             h, kind,
-            [&](int cls, int p0, int p1, int share, int variant, int nsl, cudaStream_t cs) {
-                return launch_sweep(h, kind, cls, p0, p1, c0, c1, share, variant, nsl, 0, ddm, nullptr, h->gqm.p,
+            [&](int cls, int p0, int p1, int nblk, int threads, int nsl, cudaStream_t cs) {
+                return launch_sweep(h, kind, cls, p0, p1, c0, c1, nblk, threads, nsl, 0, ddm, nullptr, h->gqm.p,
                                     h->gchg.p, cs);
             },
-            ns, std::max(1, std::min(8, (c1 - c0) / 128)), c1 - c0, false);
+            c1 - c0, false);
         if (rc) return rc;
     }
     return QMMM_OK;

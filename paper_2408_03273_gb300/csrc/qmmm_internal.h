@@ -45,17 +45,18 @@ struct RegionDev {
 struct qmmm_handle_impl;
 
 // launchers (defined in the .cu files); all return a cudaError_t of the last launch
-// Region-I sweeps.  `nsm` caps the grid (the class's share of the SMs); `variant` picks the block
-// shape: 0 = 256 threads, 1 = the class's wide block (sweep_wide_threads), where one exists;
-// `nslice` splits the charge chunk over that many block rows (small systems), the V kernels then
-// writing slice s into V + s * vstride.
+// Region-I sweeps.  A launch has `nblk` blocks of `threads` threads per charge slice (at most 256, or
+// the class's wide block, sweep_wide_threads, where one exists); its warps take the class's tiles in
+// turn.  `nslice` splits the charge chunk over that many block rows, the V kernels then writing
+// slice s into V + s * vstride.  The mixed adjoint (launch_vgrad_f32) sizes its own grid; `variant`
+// picks its charges per lane (cl_variant).
 // dst[k] = sum_s src[s*n + k], s < nslice, in order (the V slices)
 cudaError_t launch_sum_slices_d(const double *src, int nslice, size_t n, double *dst, cudaStream_t st);
 cudaError_t launch_vpot_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
-                            int ch_begin, int ch_end, const double *boys, double *V, int *err, int nsm, int variant,
+                            int ch_begin, int ch_end, const double *boys, double *V, int *err, int nblk, int threads,
                             int nslice, size_t vstride, cudaStream_t st);
 cudaError_t launch_vpot_f32(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
-                            int ch_begin, int ch_end, const float *boys, double *V, int *err, int nsm, int variant,
+                            int ch_begin, int ch_end, const float *boys, double *V, int *err, int nblk, int threads,
                             int nslice, size_t vstride, cudaStream_t st);
 // One frame's share of a class's mixed V sweep: its basis, region I and V, the primitive pairs
 // [pp_begin, pp_end) and region-I charges [ch_begin, ch_end) in ns slices of gx blocks each, its
@@ -73,7 +74,7 @@ cudaError_t launch_vpot_f32_jobs(int cls, const VJob *jobs, int njob, int nblk, 
                                  int *err, int variant, cudaStream_t st);
 cudaError_t launch_vgrad_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                              int ch_begin, int ch_end, const double *boys, const double *dm, double *gqm,
-                             double *gchg /* n*4: dC xyz, dq */, int *err, int nsm, int variant, int nslice,
+                             double *gchg /* n*4: dC xyz, dq */, int *err, int nblk, int threads, int nslice,
                              cudaStream_t st);
 // Scratch of one class's charge-lane adjoint sweep (mixed path): pair
 // records (cl_rec_floats(L) floats per primitive pair) and per-pair charge sums (6 doubles).

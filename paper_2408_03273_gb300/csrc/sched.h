@@ -16,6 +16,13 @@ inline int vpot_max_slices(int nch, size_t n2)
     return std::max(1, std::min({8, nch / 128, (int)std::min<size_t>(cap, 8)}));
 }
 
+// Most partial V matrices of a sliced sweep: 512 MB of them.
+inline int vpot_slice_cap(size_t n2, int most)
+{
+    const size_t cap = ((size_t)512 << 20) / std::max<size_t>(1, n2 * sizeof(double));
+    return std::max(1, (int)std::min<size_t>(cap, (size_t)most));
+}
+
 // Charge slices of one class.  The warps of a class sweep take whole 32-pair tiles, so
 // the class finishes when its busiest warp does, after ceil(tiles / warps) tiles: a high-l class
 // with 1.2 tiles per warp on average runs as long as with 2.  Splitting the charges over ns block
@@ -37,6 +44,38 @@ inline void class_slices(int tiles, int nwarp, int share, int nch, int maxsl, do
             *ns = s;
         }
     }
+}
+
+// Charge slices of class sweeps whose grids are one block per nwarp tiles and slice, launched in
+// order of falling block time (slice_order) so that the block scheduler packs them onto the SMs.
+// ideal: the sweep's time if it were spread evenly over nsm SMs of 8 warps.  A class is sliced so
+// that one of its blocks takes at most a quarter of that (the last blocks then leave little idle),
+// down to max(32, setup) charges per slice (setup: the work per pair that every slice repeats, in
+// charges) and to at most maxsl slices.  w: work per tile and charge.
+inline void fine_slices(int n, const int *tiles, const double *w, const double *setup, int nch, int nsm, int maxsl,
+                        int *ns)
+{
+    double work = 0.0;
+    for (int c = 0; c < n; ++c) work += tiles[c] * w[c];
+    const double ideal = work / (8.0 * nsm);  // per charge
+    for (int c = 0; c < n; ++c) {
+        ns[c] = 1;
+        if (tiles[c] <= 0) continue;
+        const double want = 4.0 * w[c] / ideal;
+        const int most = (int)(nch / (setup[c] > 32.0 ? setup[c] : 32.0));
+        ns[c] = std::max(1, std::min({want < 1e6 ? (int)(want + 0.999) : 1000000, most, maxsl}));
+    }
+}
+
+// Class indices in order of falling block time w / ns (empty classes last).
+inline void slice_order(int n, const int *tiles, const double *w, const int *ns, int *order)
+{
+    double t[64];
+    for (int c = 0; c < n; ++c) {
+        order[c] = c;
+        t[c] = tiles[c] > 0 ? w[c] / ns[c] : -1.0;
+    }
+    std::stable_sort(order, order + n, [&](int a, int b) { return t[a] > t[b]; });
 }
 
 // Shares of nsm SMs for n classes in proportion to their weights w (SM-time: primitive pairs x

@@ -37,7 +37,7 @@ template <int LA, int LB>
 struct VgradF64 {
     static cudaError_t run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
                            int ch_end, const double *boys, const double *dm, double *gqm, double *gchg, int *err,
-                           int nsm, int variant, int nslice,
+                           int nblk, int threads, int nslice,
                            cudaStream_t st);
 };
 
@@ -168,7 +168,7 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
 template <int LA, int LB, int NT>
 static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
                              int ch_end, const double *boys, const double *dm, double *gqm, double *gchg, int *err,
-                             int nsm, int nslice, cudaStream_t st)
+                             int nblk, int threads, int nslice, cudaStream_t st)
 {
     const int nper = (ch_end - ch_begin + nslice - 1) / nslice;  // charges per slice
     const size_t smem = std::max((size_t)nper * (sizeof(double4_32a) + 4 * sizeof(double)), SWEEP_SMEM_MIN);
@@ -179,11 +179,7 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const int ntile = (pp_end - pp_begin + 31) / 32;
-    int grid = (ntile + NT / 32 - 1) / (NT / 32);
-    if (grid > nsm) grid = nsm;
-    if (grid < 1) return cudaSuccess;
-    k_vgrad_f64<LA, LB, NT><<<dim3(grid, nslice), NT, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
+        k_vgrad_f64<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
                                                                   dm, gqm, gchg, err);
     return cudaGetLastError();
 }
@@ -192,15 +188,15 @@ template <int LA, int LB>
 cudaError_t VgradF64<LA, LB>::run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
                                   int ch_end, const double *boys, const double *dm, double *gqm, double *gchg,
                                   int *err,
-                                  int nsm, int variant, int nslice,
+                                  int nblk, int threads, int nslice,
                                   cudaStream_t st)
 {
     constexpr int W = sweep_wide_threads(SW_VGRAD_F64, class_of(LA, LB));
     if constexpr (W > 0)
-        if (variant == 1)
-            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nsm,
+        if (threads == W)
+            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nblk, threads,
                                         nslice, st);
-    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nsm,
+    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nblk, threads,
                                   nslice, st);
 }
 
@@ -210,11 +206,10 @@ template struct VgradF64<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_C
 
 cudaError_t launch_vgrad_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                              int ch_begin, int ch_end, const double *boys, const double *dm, double *gqm,
-                             double *gchg, int *err, int nsm, int variant, int nslice, cudaStream_t st)
+                             double *gchg, int *err, int nblk, int threads, int nslice, cudaStream_t st)
 {
     if (pp_end <= pp_begin || ch_end <= ch_begin) return cudaSuccess;
-    return dispatch_class<VgradF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nsm,
-                                    variant, nslice, st);
+    return dispatch_class<VgradF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nblk, threads, nslice, st);
 }
 
 #endif

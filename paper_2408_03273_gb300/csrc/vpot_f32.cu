@@ -16,7 +16,7 @@ namespace qmmm {
 template <int LA, int LB>
 struct VpotF32 {
     static cudaError_t run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                           int ch_end, const float *boys, double *V, int *err, int nsm, int variant, int nslice,
+                           int ch_end, const float *boys, double *V, int *err, int nblk, int threads, int nslice,
                            size_t vstride,
                            cudaStream_t st);
     static cudaError_t run_jobs(const VJob *jobs, int njob, int nblk, int maxch, const float *boys, int *err,
@@ -169,7 +169,7 @@ inline unsigned boys32_bytes() { return (unsigned)(BOYS_TAB_F * sizeof(float)); 
 
 template <int LA, int LB, int NT>
 static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                             int ch_end, const float *boys, double *V, int *err, int nsm, int nslice,
+                             int ch_end, const float *boys, double *V, int *err, int nblk, int threads, int nslice,
                              size_t vstride, cudaStream_t st)
 {
     const unsigned tb = boys32_bytes();
@@ -182,11 +182,7 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const int ntile = (pp_end - pp_begin + 31) / 32;
-    int grid = (ntile + NT / 32 - 1) / (NT / 32);
-    if (grid > nsm) grid = nsm;
-    if (grid < 1) return cudaSuccess;
-    VJob one{};
+        VJob one{};
     one.bd = bd;
     one.rg = rg;
     one.V = V;
@@ -194,9 +190,9 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
     one.pp_end = pp_end;
     one.ch_begin = ch_begin;
     one.ch_end = ch_end;
-    one.gx = grid;
+    one.gx = nblk;
     one.ns = nslice;
-    k_vpot_f32<LA, LB, NT><<<dim3(grid, nslice), NT, smem, st>>>(one, nullptr, 0, boys + (size_t)(LA + LB) * BOYS_TAB_F,
+    k_vpot_f32<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(one, nullptr, 0, boys + (size_t)(LA + LB) * BOYS_TAB_F,
                                                                  tb, vstride, err);
     return cudaGetLastError();
 }
@@ -224,16 +220,16 @@ static cudaError_t launch_nt_jobs(const VJob *jobs, int njob, int nblk, int maxc
 
 template <int LA, int LB>
 cudaError_t VpotF32<LA, LB>::run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                                 int ch_end, const float *boys, double *V, int *err, int nsm, int variant,
+                                 int ch_end, const float *boys, double *V, int *err, int nblk, int threads,
                                  int nslice, size_t vstride,
                                  cudaStream_t st)
 {
     constexpr int W = sweep_wide_threads(SW_VPOT_F32, class_of(LA, LB));
     if constexpr (W > 0)
-        if (variant == 1)
-            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nsm, nslice,
+        if (threads == W)
+            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice,
                                         vstride, st);
-    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nsm, nslice, vstride, st);
+    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice, vstride, st);
 }
 
 template <int LA, int LB>
@@ -251,12 +247,12 @@ template struct VpotF32<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_CL
 #else  // the dispatcher
 
 cudaError_t launch_vpot_f32(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
-                            int ch_begin, int ch_end, const float *boys, double *V, int *err, int nsm, int variant,
+                            int ch_begin, int ch_end, const float *boys, double *V, int *err, int nblk, int threads,
                             int nslice, size_t vstride,
                             cudaStream_t st)
 {
     if (pp_end <= pp_begin || ch_end <= ch_begin) return cudaSuccess;
-    return dispatch_class<VpotF32>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nsm, variant,
+    return dispatch_class<VpotF32>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads,
                                    nslice, vstride, st);
 }
 

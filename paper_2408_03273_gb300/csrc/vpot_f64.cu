@@ -25,7 +25,7 @@ namespace qmmm {
 template <int LA, int LB>
 struct VpotF64 {
     static cudaError_t run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                           int ch_end, const double *boys, double *V, int *err, int nsm, int variant, int nslice,
+                           int ch_end, const double *boys, double *V, int *err, int nblk, int threads, int nslice,
                            size_t vstride,
                            cudaStream_t st);
 };
@@ -122,7 +122,7 @@ k_vpot_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, in
 
 template <int LA, int LB, int NT>
 static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                             int ch_end, const double *boys, double *V, int *err, int nsm, int nslice,
+                             int ch_end, const double *boys, double *V, int *err, int nblk, int threads, int nslice,
                              size_t vstride, cudaStream_t st)
 {
     const int per = (ch_end - ch_begin + nslice - 1) / nslice;
@@ -134,27 +134,23 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const int ntile = (pp_end - pp_begin + 31) / 32;
-    int grid = (ntile + NT / 32 - 1) / (NT / 32);
-    if (grid > nsm) grid = nsm;
-    if (grid < 1) return cudaSuccess;
-    k_vpot_f64<LA, LB, NT><<<dim3(grid, nslice), NT, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
+        k_vpot_f64<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
                                                                  V, vstride, err);
     return cudaGetLastError();
 }
 
 template <int LA, int LB>
 cudaError_t VpotF64<LA, LB>::run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                                 int ch_end, const double *boys, double *V, int *err, int nsm, int variant,
+                                 int ch_end, const double *boys, double *V, int *err, int nblk, int threads,
                                  int nslice, size_t vstride,
                                  cudaStream_t st)
 {
     constexpr int W = sweep_wide_threads(SW_VPOT_F64, class_of(LA, LB));
     if constexpr (W > 0)
-        if (variant == 1)
-            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nsm, nslice,
+        if (threads == W)
+            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice,
                                         vstride, st);
-    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nsm, nslice, vstride, st);
+    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice, vstride, st);
 }
 
 template struct VpotF64<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_CLASS)>;
@@ -162,12 +158,12 @@ template struct VpotF64<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_CL
 #else  // the dispatcher
 
 cudaError_t launch_vpot_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
-                            int ch_begin, int ch_end, const double *boys, double *V, int *err, int nsm,
-                            int variant, int nslice, size_t vstride,
+                            int ch_begin, int ch_end, const double *boys, double *V, int *err, int nblk,
+                            int threads, int nslice, size_t vstride,
                             cudaStream_t st)
 {
     if (pp_end <= pp_begin || ch_end <= ch_begin) return cudaSuccess;
-    return dispatch_class<VpotF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nsm, variant,
+    return dispatch_class<VpotF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads,
                                    nslice, vstride, st);
 }
 
