@@ -185,7 +185,7 @@ struct qmmm_handle {
     int tuned_mask = 0, tuned_nI = 0;
     DBuf<double> tune_V, tune_dm, tune_gqm, tune_gchg;  // autotuner scratch
     DBuf<double> oct, oct_bins, oct_err;                  // octupole error estimate
-    DBuf<double> qmq_P, qmq_u, qmq_g, qmq_E, qmq_F;       // QM-QM periodic images
+    DBuf<double> qmq_ws, qmq_u, qmq_g, qmq_E, qmq_F;       // QM-QM periodic images
     DBuf<double> Vslices;                                 // per-slice partial V (small systems)
     EwaldBuf ew;
     int nblk_mm = 1;
@@ -302,7 +302,7 @@ struct qmmm_handle {
         Adf.release(); Azdf.release(); gSdf.release(); atom_phdf.release(); mm_filt.release(); qm_filt.release();
         tune_V.release(); tune_dm.release(); tune_gqm.release(); tune_gchg.release();
         oct.release(); oct_bins.release(); oct_err.release();
-        qmq_P.release(); qmq_u.release(); qmq_g.release(); qmq_E.release(); qmq_F.release();
+        qmq_ws.release(); qmq_u.release(); qmq_g.release(); qmq_E.release(); qmq_F.release();
         Vslices.release(); centre_d.release(); cl_rec.release(); cl_psum.release();
     }
 };
@@ -1586,7 +1586,7 @@ int qmmm_qm_images(qmmm_handle *h, const double *dmat, double *E, double *dE_dRq
     const double *ddm;
     const size_t n2 = (size_t)h->nao * h->nao, na = (size_t)h->natm;
     if ((rc = stage_input(h, dmat, n2, h->dm, &ddm))) return rc;
-    if ((rc = h->qmq_P.ensure(na * na * 20)) || (rc = h->qmq_u.ensure(na * 20)) || (rc = h->qmq_g.ensure(na * 3)) ||
+    if ((rc = h->qmq_ws.ensure(qm_images_scratch(h->ewald(), h->nsm))) || (rc = h->qmq_u.ensure(na * 20)) || (rc = h->qmq_g.ensure(na * 3)) ||
         (rc = h->qmq_E.ensure(1)))
         return rc;
     double *Fd = nullptr;
@@ -1597,7 +1597,7 @@ int qmmm_qm_images(qmmm_handle *h, const double *dmat, double *E, double *dE_dRq
     }
     // Mulliken multipoles at this density, then the image tensors, energy, potentials, gradient
     if ((rc = compute_multipoles(h, ddm, nullptr, 0))) return rc;
-    CUDA_TRY(launch_qm_images(h->ewald(), h->gfac.p, h->mult.p, h->qmq_P.p, h->qmq_E.p, h->qmq_u.p, h->qmq_g.p, st));
+    CUDA_TRY(launch_qm_images(h->ewald(), h->gfac.p, h->mult.p, h->qmq_ws.p, h->nsm, h->qmq_E.p, h->qmq_u.p, h->qmq_g.p, st));
     // the multipoles move with the basis (Pulay) and depend on gamma (Fock): the moment kernels
     // with the image potential in place of the MM one
     const BasisDev b = h->basis();

@@ -1637,56 +1637,123 @@ cudaError_t launch_octupole_error(const EwaldDev &e0, const double *oct, const d
 
 // ---------------------------------------------------------------------------------------------
 // QM-QM periodic images (Eq. 5 in the Ewald form of Eq. 6)
-//   P_ji = sum_{L != 0} T(R_j - R_i + L) (20 Taylor components), by Ewald: erfc real space over
-//   images within the Ewald cutoff, reciprocal sum over the half space (2 g(G) weights), self
-//   terms -2 kappa/sqrt(pi) and +(2/3) kappa^3/sqrt(pi) delta_ab for i = j, minus the L = 0 point
-//   tensor for i != j (the reference-cell pair belongs to the QM calculation).
 //   E = 1/2 sum_{j,i} [Q_j Q_i P + 2 mu_j.Q_i P_a + 2 theta_j:Q_i P_ab - 2 mu_j mu_i : P_ab]
-//       - pi/(2 V kappa^2) (sum Q)^2.
+//       - pi/(2 V kappa^2) (sum Q)^2,   P = sum_{L != 0} T(R_j - R_i + L) (Taylor components) by Ewald:
+// erfc real space over images within the Ewald cutoff, reciprocal sum over the half space (2 g(G)
+// weights), self terms -2 kappa/sqrt(pi) and +(2/3) kappa^3/sqrt(pi) delta_ab for i = j, minus the
+// L = 0 point tensor for i != j (the reference-cell pair belongs to the QM calculation).
+//
+// The reciprocal part factorises over the atoms.  With a_n(G) = sum_j e^{iG.R_j} x (Q_j, i G.mu_j,
+// -1/2 G.theta_j.G) for n = 0, 1, 2 it is 1/2 sum_G 2g(G) [|a_0 + a_1|^2 + 2 Re(a_0* a_2)], so the
+// potential conjugate to a monopole is that of the field a_0 + a_1 + a_2, to a dipole of a_0 + a_1
+// and to a quadrupole of a_0: two passes over (atom, G) (k_image_fields, k_image_recip) instead of
+// one over (atom, atom, G) with a sincos and 20 tensor components each.  60 atoms, kmax 16: 18.7 ->
+// 0.33 ms for the call's image part, within rounding of the pair sum.
 // ---------------------------------------------------------------------------------------------
-__constant__ int c_p2[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
-__constant__ int c_p3[10][3] = {{0, 0, 0}, {0, 0, 1}, {0, 0, 2}, {0, 1, 1}, {0, 1, 2},
-                                {0, 2, 2}, {1, 1, 1}, {1, 1, 2}, {1, 2, 2}, {2, 2, 2}};
-
-// one block per ordered pair (i = blockIdx.x, j = blockIdx.y); P[(j*natm + i)*20 + c]
-__global__ void __launch_bounds__(128) k_qmqm_pairs(EwaldDev e, const double *gfac, double *P)
+// 2g(G) (a_0, a_0 + a_1, a_0 + a_1 + a_2) on the dense box; ph: the atoms' phase rows
+constexpr int IMF_NT = 64;
+__global__ void __launch_bounds__(IMF_NT) k_image_fields(EwaldDev e, const double *gfac, const double *mult,
+                                                         const double2 *ph, double2 *f)
 {
-    __shared__ double scratch[4 * 20];
-    const int i = blockIdx.x, j = blockIdx.y;
-    const double d0[3] = {e.qm_xyz[3 * j] - e.qm_xyz[3 * i], e.qm_xyz[3 * j + 1] - e.qm_xyz[3 * i + 1],
-                          e.qm_xyz[3 * j + 2] - e.qm_xyz[3 * i + 2]};
-    double acc[20];
-#pragma unroll
-    for (int c = 0; c < 20; ++c) acc[c] = 0.0;
     const int kx = e.kmax[0], ky = e.kmax[1], kz = e.kmax[2];
     const int NY = 2 * ky + 1, NZ = 2 * kz + 1, n = (kx + 1) * NY * NZ;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const double w = gfac[k];
-        if (w == 0.0) continue;
-        const double G[3] = {TWO_PI * (k / (NY * NZ)) / e.box[0], TWO_PI * ((k / NZ) % NY - ky) / e.box[1],
-                             TWO_PI * (k % NZ - kz) / e.box[2]};
-        double sn, cs;
-        sincos(G[0] * d0[0] + G[1] * d0[1] + G[2] * d0[2], &sn, &cs);
-        acc[0] += w * cs;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) acc[1 + a] -= w * G[a] * sn;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) acc[4 + c] -= 0.5 * w * G[c_p2[c][0]] * G[c_p2[c][1]] * cs;
-#pragma unroll
-        for (int c = 0; c < 10; ++c)
-            acc[10 + c] += w * G[c_p3[c][0]] * G[c_p3[c][1]] * G[c_p3[c][2]] * sn * (1.0 / 6.0);
+    const int k = blockIdx.x * IMF_NT + threadIdx.x;
+    if (k >= n) return;
+    const double g = gfac[k];
+    const int nx = k / (NY * NZ), iy = (k / NZ) % NY, iz = k % NZ;
+    const double Gx = TWO_PI * nx / e.box[0], Gy = TWO_PI * (iy - ky) / e.box[1], Gz = TWO_PI * (iz - kz) / e.box[2];
+    const double xx = 0.5 * Gx * Gx, yy = 0.5 * Gy * Gy, zz = 0.5 * Gz * Gz, xy = Gx * Gy, xz = Gx * Gz, yz = Gy * Gz;
+    double2 a0 = make_double2(0.0, 0.0), a1 = a0, a2 = a0;
+    for (int j = 0; g != 0.0 && j < e.natm; ++j) {
+        const double *M = mult + 10 * (size_t)j;
+        const double2 *pj = ph + (size_t)j * 3 * PHR_MAXN;
+        const double2 p = cmul(cmul(__ldg(pj + nx), __ldg(pj + PHR_MAXN + iy)), __ldg(pj + 2 * PHR_MAXN + iz));
+        const double q = M[0], d = Gx * M[1] + Gy * M[2] + Gz * M[3];
+        const double t = xx * M[4] + xy * M[5] + xz * M[6] + yy * M[7] + yz * M[8] + zz * M[9];
+        a0.x += q * p.x;
+        a0.y += q * p.y;
+        a1.x -= d * p.y;
+        a1.y += d * p.x;
+        a2.x -= t * p.x;
+        a2.y -= t * p.y;
     }
-    if (threadIdx.x == 0) {
-        double T[20];
-        const double rc2 = e.ewald_rc * e.ewald_rc;
-        double n0[3];
+    f[k] = make_double2(g * a0.x, g * a0.y);
+    f[(size_t)n + k] = make_double2(g * (a0.x + a1.x), g * (a0.y + a1.y));
+    f[2 * (size_t)n + k] = make_double2(g * (a0.x + a1.x + a2.x), g * (a0.y + a1.y + a2.y));
+}
+
+// Reciprocal part of the image potentials (10 components) and of the gradient at fixed multipoles
+// (3): grid (natm, nslice), part[(j nslice + slice) 13 + c], as k_phi_recip
+__global__ void __launch_bounds__(256) k_image_recip(EwaldDev e, const double2 *f, const double *mult,
+                                                     const double2 *ph, double *part)
+{
+    __shared__ double scratch[8 * 13];
+    const int j = blockIdx.x, sl = blockIdx.y, ns = gridDim.y;
+    const int kx = e.kmax[0], ky = e.kmax[1], kz = e.kmax[2];
+    const int NY = 2 * ky + 1, NZ = 2 * kz + 1, n = (kx + 1) * NY * NZ;
+    const double2 *pj = ph + (size_t)j * 3 * PHR_MAXN;
+    double M[10];
 #pragma unroll
-        for (int x = 0; x < 3; ++x) n0[x] = rint(d0[x] / e.box[x]);
+    for (int c = 0; c < 10; ++c) M[c] = mult[10 * (size_t)j + c];
+    const double bx = TWO_PI / e.box[0], by = TWO_PI / e.box[1], bz = TWO_PI / e.box[2];
+    const int per = (n + ns - 1) / ns, k0 = sl * per, k1 = min(n, k0 + per);
+    double acc[13];
+#pragma unroll
+    for (int c = 0; c < 13; ++c) acc[c] = 0.0;
+    for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+        const double2 f0 = f[k], f1 = f[(size_t)n + k], f2 = f[2 * (size_t)n + k];
+        const int nx = k / (NY * NZ), iy = (k / NZ) % NY, iz = k % NZ;
+        const double Gx = bx * nx, Gy = by * (iy - ky), Gz = bz * (iz - kz);
+        const double2 p = cmul(cmul(__ldg(pj + nx), __ldg(pj + PHR_MAXN + iy)), __ldg(pj + 2 * PHR_MAXN + iz));
+        // conj(f) exp(i G.R_j)
+        const double r0 = f0.x * p.x + f0.y * p.y, i0 = f0.x * p.y - f0.y * p.x;
+        const double r1 = f1.x * p.x + f1.y * p.y, i1 = f1.x * p.y - f1.y * p.x;
+        const double r2 = f2.x * p.x + f2.y * p.y, i2 = f2.x * p.y - f2.y * p.x;
+        const double hx = Gx * r0, hy = Gy * r0;
+        acc[0] += r2;
+        acc[1] -= Gx * i1; acc[2] -= Gy * i1; acc[3] -= Gz * i1;
+        acc[4] -= Gx * hx; acc[5] -= Gy * hx; acc[6] -= Gz * hx;  // -1/2 applied at the end
+        acc[7] -= Gy * hy; acc[8] -= Gz * hy; acc[9] -= Gz * Gz * r0;
+        const double d = Gx * M[1] + Gy * M[2] + Gz * M[3];
+        const double t = Gx * (0.5 * Gx * M[4] + Gy * M[5] + Gz * M[6]) + Gy * (0.5 * Gy * M[7] + Gz * M[8]) +
+                         0.5 * Gz * Gz * M[9];
+        const double w = t * i0 - d * r1 - M[0] * i2;
+        acc[10] += Gx * w; acc[11] += Gy * w; acc[12] += Gz * w;
+    }
+#pragma unroll
+    for (int c = 4; c < 10; ++c) acc[c] *= 0.5;
+    block_reduce_store<13>(acc, part + ((size_t)j * ns + sl) * 13, scratch);
+}
+
+// One block per atom: real-space images and reference-cell pairs with every atom, self terms, the
+// reciprocal parts and the background; image potentials u (20-stride like phi, components 10..19
+// zero), gradient at fixed multipoles and the atom's share 1/2 sum M.u of the energy (E is
+// quadratic in the multipoles).
+constexpr int IMR_NT = 64;
+__global__ void __launch_bounds__(IMR_NT) k_image_real(EwaldDev e, const double *M, const double *part, int ns, double bg,
+                                                       double *u20, double *grad, double *Eatom)
+{
+    __shared__ double scratch[IMR_NT / 32 * 14], out[14];
+    const int k = blockIdx.x;
+    const double Qk = M[10 * k], *mk = M + 10 * k + 1, *tk = M + 10 * k + 4;
+    const double rc2 = e.ewald_rc * e.ewald_rc;
+    double v[14];  // 10 potential, 3 gradient components, sum of charges
+#pragma unroll
+    for (int c = 0; c < 14; ++c) v[c] = 0.0;
+    for (int o = threadIdx.x; o < e.natm; o += IMR_NT) {
+        double P[20], T[20], d0[3], n0[3];
+#pragma unroll
+        for (int c = 0; c < 20; ++c) P[c] = 0.0;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            d0[x] = e.qm_xyz[3 * k + x] - e.qm_xyz[3 * o + x];
+            n0[x] = rint(d0[x] / e.box[x]);
+        }
         for (int a = -e.img[0] - 1; a <= e.img[0] + 1; ++a)
             for (int b = -e.img[1] - 1; b <= e.img[1] + 1; ++b)
                 for (int c = -e.img[2] - 1; c <= e.img[2] + 1; ++c) {
                     const double L[3] = {(n0[0] + a) * e.box[0], (n0[1] + b) * e.box[1], (n0[2] + c) * e.box[2]};
-                    if (i == j && L[0] == 0.0 && L[1] == 0.0 && L[2] == 0.0) continue;
+                    if (k == o && L[0] == 0.0 && L[1] == 0.0 && L[2] == 0.0) continue;
                     const double x = d0[0] - L[0], y = d0[1] - L[1], z = d0[2] - L[2];
                     const double r2 = x * x + y * y + z * z;
                     if (r2 >= rc2) continue;
@@ -1694,143 +1761,97 @@ __global__ void __launch_bounds__(128) k_qmqm_pairs(EwaldDev e, const double *gf
                     screened_radial(r2, e.alpha, f, g1, g2, g3);
                     radial_tensor(f, g1, g2, g3, x, y, z, T, 3);
 #pragma unroll
-                    for (int k = 0; k < 20; ++k) acc[k] += T[k];
+                    for (int i = 0; i < 20; ++i) P[i] += T[i];
                 }
-        if (i == j) {
+        if (k == o) {
             const double k1 = 2.0 * e.alpha / 1.7724538509055160273, k3 = k1 * e.alpha * e.alpha / 3.0;
-            acc[0] -= k1;
-            acc[4] += k3;
-            acc[7] += k3;
-            acc[9] += k3;
+            P[0] -= k1;
+            P[4] += k3;
+            P[7] += k3;
+            P[9] += k3;
         } else {
             double f, g1, g2, g3;
             point_radial(d0[0] * d0[0] + d0[1] * d0[1] + d0[2] * d0[2], f, g1, g2, g3);
             radial_tensor(f, g1, g2, g3, d0[0], d0[1], d0[2], T, 3);
 #pragma unroll
-            for (int k = 0; k < 20; ++k) acc[k] -= T[k];
+            for (int i = 0; i < 20; ++i) P[i] -= T[i];
         }
-    }
-    block_reduce_store<20>(acc, P + ((size_t)j * gridDim.x + i) * 20, scratch);
-}
-
-// Energy, image potentials u (dE/dM per stored component / W10, 20-stride like phi) and the
-// gradient at fixed multipoles, from the pair tensors.  One block; each atom's sums in a fixed order.
-__global__ void k_qmqm_contract(int natm, const double *P, const double *M, double bg, double *E, double *u20,
-                                double *grad)
-{
-    __shared__ double ws[32];
-    double esum = 0.0;
-    for (int k = threadIdx.x; k < natm; k += blockDim.x) {
-        double uk[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0}, gk[3] = {0.0, 0.0, 0.0};
-        for (int o = 0; o < natm; ++o) {
-            // (j, i) = (k, o): first slot is k
-            for (int pass = 0; pass < 2; ++pass) {
-                const int j = pass == 0 ? k : o, i = pass == 0 ? o : k;
-                const double *p = P + ((size_t)j * natm + i) * 20;
-                double Pab[3][3], thj[3][3];
-                for (int c = 0; c < 6; ++c) {
-                    const int a = c_p2[c][0], b = c_p2[c][1];
-                    Pab[a][b] = Pab[b][a] = p[4 + c];
-                    thj[a][b] = thj[b][a] = M[10 * j + 4 + c];
-                }
-                const double Qj = M[10 * j], Qi = M[10 * i];
-                const double *mj = M + 10 * j + 1, *mi = M + 10 * i + 1;
-                if (pass == 0) {
-                    // the pair energy, counted once per ordered pair
-                    double e2 = Qj * Qi * p[0];
-                    for (int a = 0; a < 3; ++a) e2 += 2.0 * mj[a] * Qi * p[1 + a];
-                    for (int a = 0; a < 3; ++a)
-                        for (int b = 0; b < 3; ++b)
-                            e2 += 2.0 * thj[a][b] * Qi * Pab[a][b] - 2.0 * mj[a] * mi[b] * Pab[a][b];
-                    esum += 0.5 * e2;
-                    // k in the first slot
-                    uk[0] += 0.5 * Qi * p[0];
-                    for (int a = 0; a < 3; ++a) {
-                        double t = 2.0 * Qi * p[1 + a];
-                        for (int b = 0; b < 3; ++b) t -= 2.0 * mi[b] * Pab[a][b];
-                        uk[1 + a] += 0.5 * t;
-                    }
-                    for (int c = 0; c < 6; ++c) uk[4 + c] += Qi * p[4 + c];
-                    // gradient: d/dR_j of e(j, i) with R_i fixed, for i != j
-                    if (i != j)
-                        for (int c = 0; c < 3; ++c) {
-                            double g = Qj * Qi * p[1 + c];
-                            for (int a = 0; a < 3; ++a) g += 4.0 * mj[a] * Qi * Pab[a][c];
-                            for (int a = 0; a < 3; ++a)
-                                for (int b = 0; b < 3; ++b) {
-                                    // P_abc from the 10 stored components
-                                    int s3[3] = {a, b, c};
-                                    // sort the three indices
-                                    if (s3[0] > s3[1]) { int t = s3[0]; s3[0] = s3[1]; s3[1] = t; }
-                                    if (s3[1] > s3[2]) { int t = s3[1]; s3[1] = s3[2]; s3[2] = t; }
-                                    if (s3[0] > s3[1]) { int t = s3[0]; s3[0] = s3[1]; s3[1] = t; }
-                                    int idx = 0;
-                                    for (int q = 0; q < 10; ++q)
-                                        if (c_p3[q][0] == s3[0] && c_p3[q][1] == s3[1] && c_p3[q][2] == s3[2]) idx = q;
-                                    g += (6.0 * thj[a][b] * Qi - 6.0 * mj[a] * mi[b]) * p[10 + idx];
-                                }
-                            gk[c] += 0.5 * g;
-                        }
-                } else {
-                    // k in the second slot of e(j = o, i = k)
-                    double t = Qj * p[0];
-                    for (int a = 0; a < 3; ++a) t += 2.0 * mj[a] * p[1 + a];
-                    for (int a = 0; a < 3; ++a)
-                        for (int b = 0; b < 3; ++b) t += 2.0 * thj[a][b] * Pab[a][b];
-                    uk[0] += 0.5 * t;
-                    for (int b = 0; b < 3; ++b) {
-                        double s2 = 0.0;
-                        for (int a = 0; a < 3; ++a) s2 -= 2.0 * mj[a] * Pab[a][b];
-                        uk[1 + b] += 0.5 * s2;
-                    }
-                    // gradient: d/dR_i of e(j, i) = -d/dd
-                    if (i != j)
-                        for (int c = 0; c < 3; ++c) {
-                            double g = Qj * Qi * p[1 + c];
-                            for (int a = 0; a < 3; ++a) g += 4.0 * mj[a] * Qi * Pab[a][c];
-                            for (int a = 0; a < 3; ++a)
-                                for (int b = 0; b < 3; ++b) {
-                                    int s3[3] = {a, b, c};
-                                    if (s3[0] > s3[1]) { int t2 = s3[0]; s3[0] = s3[1]; s3[1] = t2; }
-                                    if (s3[1] > s3[2]) { int t2 = s3[1]; s3[1] = s3[2]; s3[2] = t2; }
-                                    if (s3[0] > s3[1]) { int t2 = s3[0]; s3[0] = s3[1]; s3[1] = t2; }
-                                    int idx = 0;
-                                    for (int q = 0; q < 10; ++q)
-                                        if (c_p3[q][0] == s3[0] && c_p3[q][1] == s3[1] && c_p3[q][2] == s3[2]) idx = q;
-                                    g += (6.0 * thj[a][b] * Qi - 6.0 * mj[a] * mi[b]) * p[10 + idx];
-                                }
-                            gk[c] -= 0.5 * g;
-                        }
-                }
+        const double Qo = M[10 * o], *mo = M + 10 * o + 1, *to = M + 10 * o + 4;
+        v[13] += Qo;
+        // both slots of the ordered pair at once (P_a and P_abc are odd in the displacement)
+        const double p2[3][3] = {{P[4], P[5], P[6]}, {P[5], P[7], P[8]}, {P[6], P[8], P[9]}};
+        v[0] += Qo * P[0] - (mo[0] * P[1] + mo[1] * P[2] + mo[2] * P[3]) + to[0] * P[4] + to[3] * P[7] + to[5] * P[9] +
+                2.0 * (to[1] * P[5] + to[2] * P[6] + to[4] * P[8]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            v[1 + a] += Qo * P[1 + a] - 2.0 * (mo[0] * p2[a][0] + mo[1] * p2[a][1] + mo[2] * p2[a][2]);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) v[4 + c] += Qo * P[4 + c];
+        if (k != o) {
+            // (theta_k Q_o + theta_o Q_k)_ab - mu_k,a mu_o,b - mu_k,b mu_o,a, against 3 P_abc
+            const double s[6] = {tk[0] * Qo + to[0] * Qk - 2.0 * mk[0] * mo[0],
+                                 2.0 * (tk[1] * Qo + to[1] * Qk - mk[0] * mo[1] - mk[1] * mo[0]),
+                                 2.0 * (tk[2] * Qo + to[2] * Qk - mk[0] * mo[2] - mk[2] * mo[0]),
+                                 tk[3] * Qo + to[3] * Qk - 2.0 * mk[1] * mo[1],
+                                 2.0 * (tk[4] * Qo + to[4] * Qk - mk[1] * mo[2] - mk[2] * mo[1]),
+                                 tk[5] * Qo + to[5] * Qk - 2.0 * mk[2] * mo[2]};
+            // P_abc with (ab) = xx xy xz yy yz zz, per c
+            const double p3[3][6] = {{P[10], P[11], P[12], P[13], P[14], P[15]},
+                                     {P[11], P[13], P[14], P[16], P[17], P[18]},
+                                     {P[12], P[14], P[15], P[17], P[18], P[19]}};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                double g = Qk * Qo * P[1 + c], h = 0.0;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) g += 2.0 * (mk[a] * Qo - mo[a] * Qk) * p2[a][c];
+#pragma unroll
+                for (int i = 0; i < 6; ++i) h += s[i] * p3[c][i];
+                v[10 + c] += g + 3.0 * h;
             }
         }
-        double qsum = 0.0;
-        for (int o = 0; o < natm; ++o) qsum += M[10 * o];
-        uk[0] += 2.0 * bg * qsum;
-        for (int c = 0; c < 10; ++c) u20[20 * k + c] = uk[c];
-        for (int c = 10; c < 20; ++c) u20[20 * k + c] = 0.0;
-        for (int c = 0; c < 3; ++c) grad[3 * k + c] = gk[c];
     }
-    esum = warp_sum(esum);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = esum;
+    block_reduce_store<14>(v, out, scratch);
+    if (threadIdx.x < 13) {
+        const int c = threadIdx.x;
+        double s = out[c];
+        for (int i = 0; i < ns; ++i) s += part[((size_t)k * ns + i) * 13 + c];
+        if (c == 0) s += 2.0 * bg * out[13];
+        out[c] = s;
+        if (c < 10) u20[20 * k + c] = s;
+        else grad[3 * k + c - 10] = s;
+    }
+    if (threadIdx.x >= 32 && threadIdx.x < 42) u20[20 * k + threadIdx.x - 22] = 0.0;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t = 0.0, qsum = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w];
-        for (int o = 0; o < natm; ++o) qsum += M[10 * o];
-        E[0] = t + bg * qsum * qsum;
+        double s = 0.0;
+#pragma unroll
+        for (int c = 0; c < 10; ++c) s += 0.5 * w10(c) * M[10 * k + c] * out[c];
+        Eatom[k] = s;
     }
 }
 
-cudaError_t launch_qm_images(const EwaldDev &e, const double *gfac, const double *mult, double *P, double *E,
+// doubles of scratch of launch_qm_images: three fields, the atoms' phase rows, the reciprocal parts
+// per slice, the atoms' energies
+size_t qm_images_scratch(const EwaldDev &e, int nsm)
+{
+    const size_t na = (size_t)e.natm;
+    return 6 * (size_t)ewald_dense_size(e) + na * 6 * PHR_MAXN + na * ewald_recip_nslice(e, nsm) * 13 + na;
+}
+
+cudaError_t launch_qm_images(const EwaldDev &e, const double *gfac, const double *mult, double *scratch, int nsm, double *E,
                              double *u20, double *grad, cudaStream_t st)
 {
     if (e.natm <= 0) return cudaSuccess;
-    k_qmqm_pairs<<<dim3(e.natm, e.natm), 128, 0, st>>>(e, gfac, P);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
+    const size_t na = (size_t)e.natm, n = (size_t)ewald_dense_size(e);
+    const int ns = ewald_recip_nslice(e, nsm);
+    double2 *f = (double2 *)scratch, *ph = f + 3 * n;
+    double *part = (double *)(ph + na * 3 * PHR_MAXN), *Eatom = part + na * ns * 13;
+    k_atom_phases<<<e.natm, 128, 0, st>>>(e, ph, nullptr);
+    k_image_fields<<<(int)((n + IMF_NT - 1) / IMF_NT), IMF_NT, 0, st>>>(e, gfac, mult, ph, f);
+    k_image_recip<<<dim3(e.natm, ns), 256, 0, st>>>(e, f, mult, ph, part);
     const double V = e.box[0] * e.box[1] * e.box[2];
-    k_qmqm_contract<<<1, 256, 0, st>>>(e.natm, P, mult, -PI / (2.0 * V * e.alpha * e.alpha), E, u20, grad);
+    k_image_real<<<e.natm, IMR_NT, 0, st>>>(e, mult, part, ns, -PI / (2.0 * V * e.alpha * e.alpha), u20, grad, Eatom);
+    k_sum1<<<1, 1024, 0, st>>>(Eatom, e.natm, 1, E);
     return cudaGetLastError();
 }
 
