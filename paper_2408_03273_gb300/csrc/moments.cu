@@ -2,502 +2,429 @@
 // them: Mulliken charge/dipole/quadrupole (SI, "Multipolar Ewald"), the region-II Fock term of
 // Eqs. 11-14 and the multipole Pulay gradient of Eq. 15.
 //
-// Multipoles and the Fock term: one lane per primitive pair.  With the Pulay gradient: two kernels
-// per angular class, one thread per (primitive pair, Cartesian component of shell A) for everything
-// about centre A and one per (primitive pair, component of shell B) for centre B, so each thread
-// keeps one row (column) of the 1-D moment tables in registers with static indexing.
-// In one direction the moment about a centre K is
-//   <i| (x-K)^e |j> = sum_t E^{ij}_t M^e_t,  M^0 = (1), M^1 = (X_PK, 1),
-//   M^2 = (X_PK^2 + 1/(2p), 2 X_PK, 2)   (times sqrt(pi/p), folded into the prefactor).
-// With the local potential polynomial W_k(r) = sum_c w_c v_k,c O_c(r - R_k) of atom k
-// (w = 1, or 2 for the off-diagonal theta components), the multipole energy is
-// E_II = sum_k Z_k v_k,0 - sum_{mu in k, nu} gamma_{nu mu} <mu|W_k|nu>, hence
-//   F_{mu nu} = -1/2 (<mu|W_{k(mu)}|nu> + <mu|W_{k(nu)}|nu>),
-// and moving the centre B of nu by d changes <mu|W_k|nu> by <mu|W_k|d nu/dB> with
-// d g_b/dB_x = 2b g_{b+1x} - b_x g_{b-1x}; moving atom k (mu and the operator) gives minus that.
+// Everything goes through the Hermite expansion of the pair density g_a g_b = sum E^x_t E^y_u E^z_v
+// Lambda_tuv: a polynomial of order n about any centre only sees t + u + v <= n (in one direction
+// int Lambda_t (x-K)^e = M^e_t,  M^0 = (1), M^1 = (X_PK, 1), M^2 = (X_PK^2 + h, 2 X_PK, 2),
+// M^3 = (X_PK^3 + 3 h X_PK, 3 X_PK^2 + 3 h, 6 X_PK, 6),  h = 1/(2p)), so
+//   * the multipoles of both atoms follow from D_tuv = sum_ab gamma_ab E^x_t E^y_u E^z_v, ten sums per
+//     pair (twenty for octupoles), by a change of basis once per pair;
+//   * with the local potential polynomial W_k(r) = sum_c w_c v_k,c O_c(r - R_k) of atom k (w = 1, or
+//     2 for the off-diagonal theta components) and H^k_tuv = int Lambda_tuv W_k, the Fock element
+//     F_{mu nu} = -1/2 (<mu|W_{k(mu)}|nu> + <mu|W_{k(nu)}|nu>) is -1/2 sum E E E (H^A + H^B)_tuv;
+//   * E_II = sum_k Z_k v_k,0 - sum_{mu in k, nu} gamma_{nu mu} <mu|W_k|nu> moves with the basis: moving B
+//     by d moves P by b/p and changes E by -dE/dX_AB, and <a|W_A|b> only depends on B - A, so
+//       dE_II/dA = -dE_II/dB = sum_tuv D_tuv (b/p H^A - a/p H^B)_{tuv + 1_d} - sum_tuv D'_d,tuv (H^A + H^B)_tuv,
+//       dE^{ij}_t/dX_AB = (b/p) E^{ij}_{t-1} - 2b E^{i,j+1}_t + j E^{i,j-1}_t.
+// The sums over the Cartesian components cost 20 FP64 instructions per component for the
+// multipoles, 20 for the Fock term and 50 for the gradient, where forming ten operator integrals
+// about each centre took about 80, 20 and 350.  The kernels are bound by the FP64 pipe (2 lanes per
+// clock and SM), on small systems by one warp's chain of FP64 instructions.  qmmm_ewald (multipoles)
+// on a QM water 0.25 -> 0.12 ms, on a 60-atom site 0.58 -> 0.33 ms, on a 150-atom site with f shells
+// 2.9 -> 1.3 ms; the multipoles with their gradient in qmmm_forces on the 150-atom site, 14.5 -> 9.5 ms
+// for everything outside the sweep.
+// A density that is not symmetric counts gamma_{nu mu} for mu's atom, as the definitions have it: the
+// difference to the transpose is carried in sums of its own, formed only where it is not zero.
 #include "pp_tile.cuh"
 
 namespace qmmm {
 
-__constant__ int c_opx[10] = {0, 1, 0, 0, 2, 1, 1, 0, 0, 0};
-__constant__ int c_opy[10] = {0, 0, 1, 0, 0, 1, 0, 2, 1, 0};
-__constant__ int c_opz[10] = {0, 0, 0, 1, 0, 0, 1, 0, 1, 2};
-__constant__ double c_w10[10] = {1, 1, 1, 1, 1, 2, 2, 1, 2, 1};
-
-// One thread per primitive pair with the full 1-D moment tables (multipoles and the Fock term:
-// the tables are small there, and one Hermite setup per pair serves all components).
-template <int LA, int LB>
-__global__ void __launch_bounds__(128)
-k_moments(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm, const double *__restrict__ phi,
-          double *__restrict__ mult, double *__restrict__ F, double *__restrict__ gqm, int mode)
-{
-    constexpr int L = LA + LB, NA = ncart(LA), NB = ncart(LB);
-    constexpr int I = LA + 1, J = LB + 1;
-    const int lane = threadIdx.x & 31;
-    const int i = pp_begin + (blockIdx.x * blockDim.x + threadIdx.x);
-    if (pp_begin + (int)((blockIdx.x * blockDim.x + (threadIdx.x & ~31))) >= pp_end) return;  // whole warp out
-    const PPLane pl = load_pp(bd, i, pp_end);
-    const bool mirror = pl.sp.shA != pl.sp.shB;
-    const bool pulay = (mode & MOM_PULAY) && pl.atomA != pl.atomB;
-
-    // 1-D moment tables about centre A (atom of shell A) and centre B, per direction
-    double SA[3][I + 1][J + 1][3], SB[3][I + 1][J + 1][3];
-    {
-        double E[I + 1][J + 1][I + J + 1];
-        const double h = 0.5 * pl.ip;
-#pragma unroll 1
-        for (int d = 0; d < 3; ++d) {
-            hermite_E<I, J, double>(E, pl.P[d] - pl.A[d], pl.P[d] - pl.B[d], h);
-            const double XA = pl.P[d] - pl.A[d], XB = pl.P[d] - pl.B[d];
-#pragma unroll
-            for (int a = 0; a <= I; ++a)
-#pragma unroll
-                for (int b = 0; b <= J; ++b) {
-                    const double e0 = E[a][b][0], e1 = (a + b >= 1) ? E[a][b][1] : 0.0,
-                                 e2 = (a + b >= 2) ? E[a][b][2] : 0.0;
-                    SA[d][a][b][0] = e0;
-                    SA[d][a][b][1] = XA * e0 + e1;
-                    SA[d][a][b][2] = (XA * XA + h) * e0 + 2.0 * XA * e1 + 2.0 * e2;
-                    SB[d][a][b][0] = e0;
-                    SB[d][a][b][1] = XB * e0 + e1;
-                    SB[d][a][b][2] = (XB * XB + h) * e0 + 2.0 * XB * e1 + 2.0 * e2;
-                }
-        }
-    }
-    const double spp = PI * pl.ip;
-    const double coef = pl.active ? pl.cab * spp * sqrt(spp) : 0.0;
-    double wA[10], wB[10];
-#pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        wA[k] = c_w10[k] * phi[20 * pl.atomA + k];
-        wB[k] = c_w10[k] * phi[20 * pl.atomB + k];
-    }
-
-    bool take[5], head;
-    seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-
-    double mA[10], mB[10], g[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int k = 0; k < 10; ++k) mA[k] = mB[k] = 0.0;
-
-#pragma unroll 1
-    for (int ia = 0; ia < NA; ++ia) {
-#pragma unroll 1
-        for (int ib = 0; ib < NB; ++ib) {
-            const int ax = cart_lx(LA, ia), ay = cart_ly(LA, ia), az = cart_lz(LA, ia);
-            const int bx = cart_lx(LB, ib), by = cart_ly(LB, ib), bz = cart_lz(LB, ib);
-            const size_t r = pl.sp.aoA + ia, c = pl.sp.aoB + ib;
-            double g_ba = 0.0, g_ab = 0.0;
-            if (pl.active && (mode & (MOM_MULT | MOM_PULAY))) {
-                g_ba = dm[c * bd.nao + r];
-                g_ab = dm[r * bd.nao + c];
-            }
-            double fA = 0.0, fB = 0.0;
-#pragma unroll
-            for (int op = 0; op < 10; ++op) {
-                const int ox = c_opx[op], oy = c_opy[op], oz = c_opz[op];
-                const double sa = SA[0][ax][bx][ox] * SA[1][ay][by][oy] * SA[2][az][bz][oz];
-                const double sb = SB[0][ax][bx][ox] * SB[1][ay][by][oy] * SB[2][az][bz][oz];
-                mA[op] -= g_ba * sa;
-                mB[op] -= g_ab * sb;
-                fA += wA[op] * sa;
-                fB += wB[op] * sb;
-                if (pulay) {
-                    // G1: d/dB of <a|W_A|b>;  G2: d/dA of <a|W_B|b>
-                    const double dBx = 2.0 * pl.b * SA[0][ax][bx + 1][ox] - (bx > 0 ? bx * SA[0][ax][bx - 1][ox] : 0.0);
-                    const double dBy = 2.0 * pl.b * SA[1][ay][by + 1][oy] - (by > 0 ? by * SA[1][ay][by - 1][oy] : 0.0);
-                    const double dBz = 2.0 * pl.b * SA[2][az][bz + 1][oz] - (bz > 0 ? bz * SA[2][az][bz - 1][oz] : 0.0);
-                    const double dAx = 2.0 * pl.a * SB[0][ax + 1][bx][ox] - (ax > 0 ? ax * SB[0][ax - 1][bx][ox] : 0.0);
-                    const double dAy = 2.0 * pl.a * SB[1][ay + 1][by][oy] - (ay > 0 ? ay * SB[1][ay - 1][by][oy] : 0.0);
-                    const double dAz = 2.0 * pl.a * SB[2][az + 1][bz][oz] - (az > 0 ? az * SB[2][az - 1][bz][oz] : 0.0);
-                    const double ga = g_ba * wA[op], gb = g_ab * wB[op];
-                    const double sAy = SA[1][ay][by][oy], sAz = SA[2][az][bz][oz], sAx = SA[0][ax][bx][ox];
-                    const double sBy = SB[1][ay][by][oy], sBz = SB[2][az][bz][oz], sBx = SB[0][ax][bx][ox];
-                    g[0] += ga * dBx * sAy * sAz - gb * dAx * sBy * sBz;
-                    g[1] += ga * sAx * dBy * sAz - gb * sBx * dAy * sBz;
-                    g[2] += ga * sAx * sAy * dBz - gb * sBx * sBy * dAz;
-                }
-            }
-            if (mode & MOM_FOCK) {
-                const double f = seg_reduce(-0.5 * coef * (fA + fB), take);
-                if (head && pl.active) {
-                    atomicAdd(F + r * bd.nao + c, f);
-                    if (mirror) atomicAdd(F + c * bd.nao + r, f);
-                }
-            }
-        }
-    }
-    if (mode & MOM_MULT) {
-#pragma unroll
-        for (int k = 0; k < 10; ++k) {
-            const double va = seg_reduce(coef * mA[k], take);
-            const double vb = seg_reduce(mirror ? coef * mB[k] : 0.0, take);
-            if (head && pl.active) {
-                atomicAdd(mult + 10 * pl.atomA + k, va);
-                if (mirror) atomicAdd(mult + 10 * pl.atomB + k, vb);
-            }
-        }
-    }
-    if (mode & MOM_PULAY) {
-#pragma unroll
-        for (int x = 0; x < 3; ++x) {
-            const double v = seg_reduce(pulay ? coef * g[x] : 0.0, take);
-            if (head && pl.active && pl.atomA != pl.atomB) {
-                atomicAdd(gqm + 3 * pl.atomA + x, v);
-                atomicAdd(gqm + 3 * pl.atomB + x, -v);
-            }
-        }
-    }
-}
-
-// Operator O_c = (x-K)^ox (y-K)^oy (z-K)^oz of the ten multipole components c (charge, dipole,
-// quadrupole in the order 1, x, y, z, xx, xy, xz, yy, yz, zz); weight 2 for the off-diagonal
-// quadrupole components.  constexpr, so that unrolled loops index the moment tables statically.
 __host__ __device__ constexpr int op_x(int c) { return c == 1 ? 1 : c == 4 ? 2 : (c == 5 || c == 6) ? 1 : 0; }
 __host__ __device__ constexpr int op_y(int c) { return c == 2 ? 1 : c == 7 ? 2 : (c == 5 || c == 8) ? 1 : 0; }
 __host__ __device__ constexpr int op_z(int c) { return c == 3 ? 1 : c == 9 ? 2 : (c == 6 || c == 8) ? 1 : 0; }
-__host__ __device__ constexpr double op_w(int c) { return (c == 5 || c == 6 || c == 8) ? 2.0 : 1.0; }
+// Exponents of the octupole components xxx, xxy, xxz, xyy, xyz, xzz, yyy, yyz, yzz, zzz
+__host__ __device__ constexpr int o3_x(int c) { return c == 0 ? 3 : c <= 2 ? 2 : c <= 5 ? 1 : 0; }
+__host__ __device__ constexpr int o3_z(int c) { return c == 9 ? 3 : (c == 5 || c == 8) ? 2 : (c == 2 || c == 4 || c == 7) ? 1 : 0; }
+__host__ __device__ constexpr int o3_y(int c) { return 3 - o3_x(c) - o3_z(c); }
 
-// The 1-D moments of orders 0..2 about centre K from one Hermite row: (e0, X e0 + e1,
-// (X^2 + h) e0 + 2 X e1 + 2 e2), X = P - K, h = 1/(2p).
-__device__ __forceinline__ void moments3(double e0, double e1, double e2, double X, double h, double (&m)[3])
-{
-    m[0] = e0;
-    m[1] = X * e0 + e1;
-    m[2] = (X * X + h) * e0 + 2.0 * X * e1 + 2.0 * e2;
-}
-
-// E^{r,k}_t, t = 0..2, for one fixed index r of the first kind (runtime, 0..NR) and every k = 0..NK
-// of the second: the recursion runs first in the fixed direction up to r (a short vector, the
-// entry r selected by predicate, so all indexing stays static), then along k.  X1, X2: the
-// displacements P - (centre of the first / second kind); h = 1/(2p).
-template <int NR, int NK>
-__device__ __forceinline__ void hermite_line(double X1, double X2, double h, int r, double (&out)[NK + 1][3])
-{
-    constexpr int T = NR + NK + 1;  // largest t reached
-    double v[T + 1], sel[T + 1];
-#pragma unroll
-    for (int t = 0; t <= T; ++t) v[t] = sel[t] = 0.0;
-    v[0] = 1.0;
-#pragma unroll
-    for (int a = 0; a <= NR; ++a) {
-        if (a == r)
-#pragma unroll
-            for (int t = 0; t <= T; ++t) sel[t] = v[t];
-        if (a < NR) {
-            double w[T + 1];
-#pragma unroll
-            for (int t = 0; t <= T; ++t)
-                w[t] = (t > 0 ? h * v[t - 1] : 0.0) + X1 * v[t] + (t < T ? (t + 1) * v[t + 1] : 0.0);
-#pragma unroll
-            for (int t = 0; t <= T; ++t) v[t] = w[t];
-        }
-    }
-#pragma unroll
-    for (int k = 0; k <= NK; ++k) {
-        out[k][0] = sel[0];
-        out[k][1] = sel[1];
-        out[k][2] = T >= 2 ? sel[T >= 2 ? 2 : 0] : 0.0;
-        if (k < NK) {
-            double w[T + 1];
-#pragma unroll
-            for (int t = 0; t <= T; ++t)
-                w[t] = (t > 0 ? h * sel[t - 1] : 0.0) + X2 * sel[t] + (t < T ? (t + 1) * sel[t + 1] : 0.0);
-#pragma unroll
-            for (int t = 0; t <= T; ++t) sel[t] = w[t];
-        }
-    }
-}
-
-// A side: one thread per (primitive pair, Cartesian component ia of shell A): the moments about
-// A (multipoles of atom A, the Fock term with W_A, and the Pulay term d/dB <a|W_A|b>).  grid
-// (ceil(n/128), NA); the lanes of a warp share ia, so primitive pairs of one shell pair are
-// contiguous lanes and reduce before their atomics.
-template <int LA, int LB>
-__global__ void __launch_bounds__(128) k_mom_a(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm,
-                                               const double *__restrict__ phi, double *__restrict__ mult,
-                                               double *__restrict__ F, double *__restrict__ gqm, int mode)
-{
-    constexpr int NB = ncart(LB);
-    const int lane = threadIdx.x & 31, ia = blockIdx.y;
-    const int i = pp_begin + (blockIdx.x * blockDim.x + threadIdx.x);
-    if (pp_begin + (int)((blockIdx.x * blockDim.x + (threadIdx.x & ~31))) >= pp_end) return;  // whole warp out
-    const PPLane pl = load_pp(bd, i, pp_end);
-    const bool mirror = pl.sp.shA != pl.sp.shB;
-    const bool pulay = (mode & MOM_PULAY) && pl.atomA != pl.atomB;
-    int a3[3];
+// 1-D moments M^e_t about a centre at distance X from P
+template <int ORD>
+struct Mom1 {
+    double m[ORD + 1][ORD + 1];
+    __device__ __forceinline__ Mom1(double X, double h)
     {
-        // the Cartesian exponents of component ia
+        const double X2 = X * X;
+        m[0][0] = 1.0;
+        if constexpr (ORD >= 1) {
+            m[1][0] = X;
+            m[1][1] = 1.0;
+        }
+        if constexpr (ORD >= 2) {
+            m[2][0] = X2 + h;
+            m[2][1] = 2.0 * X;
+            m[2][2] = 2.0;
+        }
+        if constexpr (ORD >= 3) {
+            m[3][0] = X * (X2 + 3.0 * h);
+            m[3][1] = 3.0 * (X2 + h);
+            m[3][2] = 6.0 * X;
+            m[3][3] = 6.0;
+        }
+    }
+};
+
+// H^k_tuv, t + u + v <= 2, of the potential polynomial of atom k (phi: its 20 Taylor components) at
+// displacement X = P - R_k
+__device__ __forceinline__ void potential_hermite(const double *__restrict__ phi, const double (&X)[3], double h,
+                                                  double (&H)[10])
+{
+    const double xx = phi[4], xy = phi[5], xz = phi[6], yy = phi[7], yz = phi[8], zz = phi[9];
+    const double lx = xx * X[0] + xy * X[1] + xz * X[2], ly = xy * X[0] + yy * X[1] + yz * X[2],
+                 lz = xz * X[0] + yz * X[1] + zz * X[2];
+    H[0] = phi[0] + X[0] * (phi[1] + lx) + X[1] * (phi[2] + ly) + X[2] * (phi[3] + lz) + h * (xx + yy + zz);
+    H[hidx(1, 0, 0)] = phi[1] + 2.0 * lx;
+    H[hidx(0, 1, 0)] = phi[2] + 2.0 * ly;
+    H[hidx(0, 0, 1)] = phi[3] + 2.0 * lz;
+    H[hidx(2, 0, 0)] = 2.0 * xx;
+    H[hidx(0, 2, 0)] = 2.0 * yy;
+    H[hidx(0, 0, 2)] = 2.0 * zz;
+    H[hidx(1, 1, 0)] = 2.0 * xy;
+    H[hidx(1, 0, 1)] = 2.0 * xz;
+    H[hidx(0, 1, 1)] = 2.0 * yz;
+}
+
+// Block (32, NA): lane = primitive pair, warp = Cartesian component of shell A.  The warps first
+// share the pair's setup (1-D Hermite tables per direction, prefactor, potentials) through shared
+// memory, then each sweeps the components of shell B, and the sums over the components of A meet
+// in shared memory again: one setup and one set of atomics per pair whatever its component count,
+// and short chains for a pair of high angular momentum.
+// ORD: 2 multipoles to the quadrupole (out: mult), 3 octupoles (out: oct).
+template <int LA, int LB, int ORD, bool FOCK, bool PULAY>
+struct MomShape {
+    static constexpr int NA = ncart(LA), NB = ncart(LB), LBP = PULAY ? LB + 1 : LB;
+    static constexpr int TM = LA + LB < ORD ? LA + LB : ORD;  // highest Hermite order that occurs
+    static constexpr int ND = nherm(TM);
+    static constexpr int NT = 3 * (LA + 1) * (LBP + 1) * (TM + 1);  // table doubles per lane
+    static constexpr int NR = ND + (PULAY ? 3 : 0);                 // sums per lane and warp
+    static constexpr int NP = (FOCK || PULAY) ? 21 : 1;  // coefficient, H^A + H^B, H^B
+    static constexpr int NS = (NT > NA * NR ? NT : NA * NR) + NP;
+};
+
+template <int LA, int LB, int ORD, bool MULT, bool FOCK, bool PULAY>
+__global__ void __launch_bounds__(32 * ncart(LA))
+k_moments(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm, const double *__restrict__ phi,
+          double *__restrict__ mult, double *__restrict__ F, double *__restrict__ gqm)
+{
+    using Sh = MomShape<LA, LB, ORD, FOCK, PULAY>;
+    constexpr int NA = Sh::NA, NB = Sh::NB, LBP = Sh::LBP, TM = Sh::TM, ND = Sh::ND, NR = Sh::NR;
+    extern __shared__ double sm[][32];
+    double(*pairc)[32] = sm + (Sh::NS - Sh::NP);
+    auto tab = [](int d, int a, int b, int t) { return ((d * (LA + 1) + a) * (LBP + 1) + b) * (TM + 1) + t; };
+    const int lane = threadIdx.x, ia = threadIdx.y;
+    const int i = pp_begin + blockIdx.x * 32 + lane;
+    const bool active = i < pp_end;
+    const uint32_t code = __ldg(bd.pp + (active ? i : pp_end - 1));
+    const int s = (int)(code >> 8), ka = (code >> 4) & 15, kb = code & 15;
+    const SPair sp = bd.sp[s];
+    const int pa = __ldg(bd.shell_off + sp.shA) + ka, pb = __ldg(bd.shell_off + sp.shB) + kb;
+    const int atomA = __ldg(bd.shell_atom + sp.shA), atomB = __ldg(bd.shell_atom + sp.shB);
+    const double a = __ldg(bd.exps + pa), b = __ldg(bd.exps + pb), ip = 1.0 / (a + b), h = 0.5 * ip;
+    double XA[3], XB[3];  // P - A, P - B
+    double ab2 = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const double A = bd.qm_xyz[3 * atomA + d], B = bd.qm_xyz[3 * atomB + d];
+        const double P = (a * A + b * B) * ip;
+        XA[d] = P - A;
+        XB[d] = P - B;
+        ab2 += (A - B) * (A - B);
+    }
+    const bool mirror = sp.shA != sp.shB, two = atomA != atomB;
+
+    // setup: tasks 0..2 the tables of one direction, 3 the prefactor, 4 the potentials
+    for (int task = ia; task < 5; task += NA) {
+        if (task < 3) {
+            const double xa = task == 0 ? XA[0] : task == 1 ? XA[1] : XA[2];
+            const double xb = task == 0 ? XB[0] : task == 1 ? XB[1] : XB[2];
+            // E_0 by its two-term recursion, E_t = h/t (i E^{i-1,j}_{t-1} + j E^{i,j-1}_{t-1})
+            double E[LA + 1][LBP + 1][TM + 1];
+            E[0][0][0] = 1.0;
+#pragma unroll
+            for (int k = 0; k <= LA; ++k)
+#pragma unroll
+                for (int j = 0; j <= LBP; ++j) {
+#pragma unroll
+                    for (int t = 1; t <= TM; ++t) {
+                        double e = 0.0;
+                        if (k > 0) e += (double)k * E[k > 0 ? k - 1 : 0][j][t - 1];
+                        if (j > 0) e += (double)j * E[k][j > 0 ? j - 1 : 0][t - 1];
+                        E[k][j][t] = (k + j > 0) ? (h * (1.0 / t)) * e : 0.0;
+                    }
+                    double e1 = 0.0;  // E_1 of (k, j), whatever TM
+                    if constexpr (TM >= 1) e1 = E[k][j][TM >= 1 ? 1 : 0];
+                    else if (j > 0) e1 = h * j * E[k][j > 0 ? j - 1 : 0][0];
+                    if (k == 0 && j < LBP) E[0][j < LBP ? j + 1 : 0][0] = xb * E[0][j][0] + e1;
+                    if (k < LA) E[k < LA ? k + 1 : 0][j][0] = xa * E[k][j][0] + e1;
+                }
+#pragma unroll
+            for (int k = 0; k <= LA; ++k)
+#pragma unroll
+                for (int j = 0; j <= LBP; ++j)
+#pragma unroll
+                    for (int t = 0; t <= TM; ++t) sm[tab(task, k, j, t)][lane] = E[k][j][t];
+        } else if (task == 3) {
+            const double spp = PI * ip;
+            pairc[0][lane] = active ? __ldg(bd.ncoef + pa) * __ldg(bd.ncoef + pb) * exp(-a * b * ip * ab2) * spp * sqrt(spp)
+                                    : 0.0;
+        } else if constexpr (FOCK || PULAY) {
+            double HA[10], HB[10];
+            potential_hermite(phi + 20 * (size_t)atomA, XA, h, HA);
+            potential_hermite(phi + 20 * (size_t)atomB, XB, h, HB);
+#pragma unroll
+            for (int k = 0; k < 10; ++k) {
+                pairc[1 + k][lane] = HA[k] + HB[k];
+                pairc[11 + k][lane] = HB[k];
+            }
+        }
+    }
+    __syncthreads();
+
+    const double coef = pairc[0][lane];
+    bool take[5], head;
+    seg_setup(active ? s : -1 - lane, lane, take, head);
+    int a3[3] = {0, 0, 0};
+    {
         int k = 0;
-        a3[0] = a3[1] = a3[2] = 0;
 #pragma unroll
         for (int x = LA; x >= 0; --x)
 #pragma unroll
-            for (int y = LA - x; y >= 0; --y) {
+            for (int y = LA - x; y >= 0; --y, ++k)
                 if (k == ia) {
                     a3[0] = x;
                     a3[1] = y;
                     a3[2] = LA - x - y;
                 }
-                ++k;
-            }
     }
-    // SA[d][b][o]: moments about A of order o for the row a = a3[d], b <= LB + 1
-    double SA[3][LB + 2][3];
-    const double h = 0.5 * pl.ip;
+    constexpr int NH2 = nherm(TM < 2 ? TM : 2);
+    double Hs[10], Hb[10];
+    if constexpr (FOCK || PULAY) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        double e[LB + 2][3];
-        hermite_line<LA, LB + 1>(pl.P[d] - pl.A[d], pl.P[d] - pl.B[d], h, a3[d], e);
-#pragma unroll
-        for (int b = 0; b <= LB + 1; ++b) moments3(e[b][0], e[b][1], e[b][2], pl.P[d] - pl.A[d], h, SA[d][b]);
+        for (int k = 0; k < NH2; ++k) {
+            Hs[k] = pairc[1 + k][lane];
+            Hb[k] = pairc[11 + k][lane];
+        }
     }
-    const double spp = PI * pl.ip;
-    const double coef = pl.active ? pl.cab * spp * sqrt(spp) : 0.0;
-    double wA[10];
+    double D[ND], Dd[ND], g[3] = {0.0, 0.0, 0.0}, gd[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-    for (int c = 0; c < 10; ++c) wA[c] = op_w(c) * phi[20 * pl.atomA + c];
-    bool take[5], head;
-    seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-    double mA[10], g[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int c = 0; c < 10; ++c) mA[c] = 0.0;
-    const size_t r = pl.sp.aoA + ia;
-#pragma unroll
+    for (int k = 0; k < ND; ++k) D[k] = Dd[k] = 0.0;
+    bool skew = false;  // a density element differs from its transpose
+    const size_t r = sp.aoA + ia;
+#pragma unroll 1
     for (int ib = 0; ib < NB; ++ib) {
-        const int bx = cart_lx(LB, ib), by = cart_ly(LB, ib), bz = cart_lz(LB, ib);
-        const size_t c = pl.sp.aoB + ib;
-        const double g_ba = (pl.active && (mode & (MOM_MULT | MOM_PULAY))) ? dm[c * bd.nao + r] : 0.0;
-        double fA = 0.0;
+        int b3[3] = {0, 0, 0};
+        {
+            int k = 0;
 #pragma unroll
-        for (int op = 0; op < 10; ++op) {
-            const int ox = op_x(op), oy = op_y(op), oz = op_z(op);
-            const double sx = SA[0][bx][ox], sy = SA[1][by][oy], sz = SA[2][bz][oz];
-            const double sa = sx * sy * sz;
-            mA[op] -= g_ba * sa;
-            fA += wA[op] * sa;
-            if (pulay) {
-                // d/dB of <a|W_A|b>: d g_b/dB_x = 2b g_{b+1x} - b_x g_{b-1x}
-                const double dBx = 2.0 * pl.b * SA[0][bx + 1][ox] - (bx > 0 ? bx * SA[0][bx > 0 ? bx - 1 : 0][ox] : 0.0);
-                const double dBy = 2.0 * pl.b * SA[1][by + 1][oy] - (by > 0 ? by * SA[1][by > 0 ? by - 1 : 0][oy] : 0.0);
-                const double dBz = 2.0 * pl.b * SA[2][bz + 1][oz] - (bz > 0 ? bz * SA[2][bz > 0 ? bz - 1 : 0][oz] : 0.0);
-                const double ga = g_ba * wA[op];
-                g[0] += ga * dBx * sy * sz;
-                g[1] += ga * sx * dBy * sz;
-                g[2] += ga * sx * sy * dBz;
+            for (int x = LB; x >= 0; --x)
+#pragma unroll
+                for (int y = LB - x; y >= 0; --y, ++k)
+                    if (k == ib) {
+                        b3[0] = x;
+                        b3[1] = y;
+                        b3[2] = LB - x - y;
+                    }
+        }
+        const size_t c = sp.aoB + ib;
+        double E[3][TM + 1], gm = 0.0, delta = 0.0;
+        if (MULT || PULAY) {
+            if (active) {
+                gm = dm[c * bd.nao + r];
+                delta = dm[r * bd.nao + c] - gm;
             }
         }
-        if (mode & MOM_FOCK) {
-            const double f = seg_reduce(-0.5 * coef * fA, take);
-            if (head && pl.active) {
-                atomicAdd(F + r * bd.nao + c, f);
-                if (mirror) atomicAdd(F + c * bd.nao + r, f);
-            }
-        }
-    }
-    if (mode & MOM_MULT) {
 #pragma unroll
-        for (int k = 0; k < 10; ++k) {
-            const double va = seg_reduce(coef * mA[k], take);
-            if (head && pl.active) atomicAdd(mult + 10 * pl.atomA + k, va);
-        }
-    }
-    if (mode & MOM_PULAY) {
+        for (int d = 0; d < 3; ++d)
 #pragma unroll
-        for (int x = 0; x < 3; ++x) {
-            const double v = seg_reduce(pulay ? coef * g[x] : 0.0, take);
-            if (head && pl.active && pl.atomA != pl.atomB) {
-                atomicAdd(gqm + 3 * pl.atomA + x, v);
-                atomicAdd(gqm + 3 * pl.atomB + x, -v);
-            }
-        }
-    }
-}
-
-// B side: one thread per (primitive pair, Cartesian component ib of shell B): the moments about
-// B (multipoles of atom B for off-diagonal shell pairs, the Fock term with W_B, and the Pulay
-// term d/dA <a|W_B|b>).  grid (ceil(n/128), NB).
-template <int LA, int LB>
-__global__ void __launch_bounds__(128) k_mom_b(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm,
-                                               const double *__restrict__ phi, double *__restrict__ mult,
-                                               double *__restrict__ F, double *__restrict__ gqm, int mode)
-{
-    constexpr int NA = ncart(LA);
-    const int lane = threadIdx.x & 31, ib = blockIdx.y;
-    const int i = pp_begin + (blockIdx.x * blockDim.x + threadIdx.x);
-    if (pp_begin + (int)((blockIdx.x * blockDim.x + (threadIdx.x & ~31))) >= pp_end) return;  // whole warp out
-    const PPLane pl = load_pp(bd, i, pp_end);
-    const bool mirror = pl.sp.shA != pl.sp.shB;
-    const bool pulay = (mode & MOM_PULAY) && pl.atomA != pl.atomB;
-    int b3[3];
-    {
-        int k = 0;
-        b3[0] = b3[1] = b3[2] = 0;
+            for (int t = 0; t <= TM; ++t) E[d][t] = sm[tab(d, a3[d], b3[d], t)][lane];
+        const bool odd = (MULT || PULAY) && __any_sync(FULL, delta != 0.0);
+        skew |= odd;
+        if (MULT || PULAY) {
 #pragma unroll
-        for (int x = LB; x >= 0; --x)
+            for (int t = 0; t <= TM; ++t) {
+                const double gx = gm * E[0][t];
 #pragma unroll
-            for (int y = LB - x; y >= 0; --y) {
-                if (k == ib) {
-                    b3[0] = x;
-                    b3[1] = y;
-                    b3[2] = LB - x - y;
+                for (int u = 0; u <= TM - t; ++u) {
+                    const double gxy = gx * E[1][u];
+#pragma unroll
+                    for (int v = 0; v <= TM - t - u; ++v) D[hidx(t, u, v)] += gxy * E[2][v];
                 }
-                ++k;
             }
-    }
-    // SB[d][a][o]: moments about B of order o for the column b = b3[d], a <= LA + 1
-    double SB[3][LA + 2][3];
-    const double h = 0.5 * pl.ip;
+            if (odd) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        double e[LA + 2][3];
-        hermite_line<LB, LA + 1>(pl.P[d] - pl.B[d], pl.P[d] - pl.A[d], h, b3[d], e);
+                for (int t = 0; t <= TM; ++t)
 #pragma unroll
-        for (int a = 0; a <= LA + 1; ++a) moments3(e[a][0], e[a][1], e[a][2], pl.P[d] - pl.B[d], h, SB[d][a]);
-    }
-    const double spp = PI * pl.ip;
-    const double coef = pl.active ? pl.cab * spp * sqrt(spp) : 0.0;
-    double wB[10];
+                    for (int u = 0; u <= TM - t; ++u)
 #pragma unroll
-    for (int c = 0; c < 10; ++c) wB[c] = op_w(c) * phi[20 * pl.atomB + c];
-    bool take[5], head;
-    seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-    double mB[10], g[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int c = 0; c < 10; ++c) mB[c] = 0.0;
-    const size_t c = pl.sp.aoB + ib;
-#pragma unroll
-    for (int ia = 0; ia < NA; ++ia) {
-        const int ax = cart_lx(LA, ia), ay = cart_ly(LA, ia), az = cart_lz(LA, ia);
-        const size_t r = pl.sp.aoA + ia;
-        const double g_ab = (pl.active && (mode & (MOM_MULT | MOM_PULAY))) ? dm[r * bd.nao + c] : 0.0;
-        double fB = 0.0;
-#pragma unroll
-        for (int op = 0; op < 10; ++op) {
-            const int ox = op_x(op), oy = op_y(op), oz = op_z(op);
-            const double sx = SB[0][ax][ox], sy = SB[1][ay][oy], sz = SB[2][az][oz];
-            const double sb = sx * sy * sz;
-            mB[op] -= g_ab * sb;
-            fB += wB[op] * sb;
-            if (pulay) {
-                // d/dA of <a|W_B|b>
-                const double dAx = 2.0 * pl.a * SB[0][ax + 1][ox] - (ax > 0 ? ax * SB[0][ax > 0 ? ax - 1 : 0][ox] : 0.0);
-                const double dAy = 2.0 * pl.a * SB[1][ay + 1][oy] - (ay > 0 ? ay * SB[1][ay > 0 ? ay - 1 : 0][oy] : 0.0);
-                const double dAz = 2.0 * pl.a * SB[2][az + 1][oz] - (az > 0 ? az * SB[2][az > 0 ? az - 1 : 0][oz] : 0.0);
-                const double gb = g_ab * wB[op];
-                g[0] -= gb * dAx * sy * sz;
-                g[1] -= gb * sx * dAy * sz;
-                g[2] -= gb * sx * sy * dAz;
+                        for (int v = 0; v <= TM - t - u; ++v) Dd[hidx(t, u, v)] += delta * E[0][t] * E[1][u] * E[2][v];
             }
         }
-        if (mode & MOM_FOCK) {
-            const double f = seg_reduce(-0.5 * coef * fB, take);
-            if (head && pl.active) {
-                atomicAdd(F + r * bd.nao + c, f);
-                if (mirror) atomicAdd(F + c * bd.nao + r, f);
+        if constexpr (FOCK || PULAY) {
+            // sum_tuv E^x_t E^y_u E^z_v H_tuv, innermost direction first
+            double hxy[TM + 1][TM + 1], hx[TM + 1], f = 0.0;
+#pragma unroll
+            for (int t = 0; t <= TM; ++t) {
+                hx[t] = 0.0;
+#pragma unroll
+                for (int u = 0; u <= TM - t; ++u) {
+                    hxy[t][u] = 0.0;
+#pragma unroll
+                    for (int v = 0; v <= TM - t - u; ++v) hxy[t][u] += E[2][v] * Hs[hidx(t, u, v)];
+                    hx[t] += E[1][u] * hxy[t][u];
+                }
+                f += E[0][t] * hx[t];
+            }
+            if constexpr (FOCK) {
+                const double v = seg_reduce(-0.5 * coef * f, take);
+                if (head && active) {
+                    atomicAdd(F + r * bd.nao + c, v);
+                    if (mirror) atomicAdd(F + c * bd.nao + r, v);
+                }
+            }
+            if constexpr (PULAY) {
+                // dE^{ij}_t / dX_AB in each direction
+                double dE[3][TM + 1];
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+#pragma unroll
+                    for (int t = 0; t <= TM; ++t) {
+                        double e = -2.0 * b * sm[tab(d, a3[d], b3[d] + 1, t)][lane];
+                        if (b3[d] > 0) e += (double)b3[d] * sm[tab(d, a3[d], b3[d] - 1, t)][lane];
+                        if (t > 0) e += b * ip * E[d][t > 0 ? t - 1 : 0];
+                        dE[d][t] = e;
+                    }
+                double dx = 0.0, dy = 0.0, dz = 0.0;
+#pragma unroll
+                for (int t = 0; t <= TM; ++t) {
+                    double sy = 0.0, sz = 0.0;
+#pragma unroll
+                    for (int u = 0; u <= TM - t; ++u) {
+                        double hz = 0.0;
+#pragma unroll
+                        for (int v = 0; v <= TM - t - u; ++v) hz += dE[2][v] * Hs[hidx(t, u, v)];
+                        sy += dE[1][u] * hxy[t][u];
+                        sz += E[1][u] * hz;
+                    }
+                    dx += dE[0][t] * hx[t];
+                    dy += E[0][t] * sy;
+                    dz += E[0][t] * sz;
+                }
+                g[0] += gm * dx;
+                g[1] += gm * dy;
+                g[2] += gm * dz;
+                if (odd) {
+#pragma unroll
+                    for (int t = 0; t <= TM; ++t)
+#pragma unroll
+                        for (int u = 0; u <= TM - t; ++u)
+#pragma unroll
+                            for (int v = 0; v <= TM - t - u; ++v) {
+                                const double H = delta * Hb[hidx(t, u, v)];
+                                gd[0] += H * dE[0][t] * E[1][u] * E[2][v];
+                                gd[1] += H * E[0][t] * dE[1][u] * E[2][v];
+                                gd[2] += H * E[0][t] * E[1][u] * dE[2][v];
+                            }
+                }
             }
         }
     }
-    if (mode & MOM_MULT) {
+    // sums over the components of A (warps 0, 1, 2, as far as there are, need the totals): the
+    // density's part, then the antisymmetric rest if there is one
+    auto total = [&](double (&d)[ND], double (&v)[3]) {
+        if constexpr (NA > 1) {
+            __syncthreads();
 #pragma unroll
-        for (int k = 0; k < 10; ++k) {
-            const double vb = seg_reduce(mirror ? coef * mB[k] : 0.0, take);
-            if (head && pl.active && mirror) atomicAdd(mult + 10 * pl.atomB + k, vb);
-        }
-    }
-    if (mode & MOM_PULAY) {
+            for (int k = 0; k < ND; ++k) sm[ia * NR + k][lane] = d[k];
+            if constexpr (PULAY) {
 #pragma unroll
-        for (int x = 0; x < 3; ++x) {
-            const double v = seg_reduce(pulay ? coef * g[x] : 0.0, take);
-            if (head && pl.active && pl.atomA != pl.atomB) {
-                atomicAdd(gqm + 3 * pl.atomA + x, v);
-                atomicAdd(gqm + 3 * pl.atomB + x, -v);
+                for (int k = 0; k < 3; ++k) sm[ia * NR + ND + k][lane] = v[k];
+            }
+            __syncthreads();
+            if (ia >= 3) return;
+#pragma unroll
+            for (int k = 0; k < NR; ++k) {
+                double x = 0.0;
+                for (int w = 0; w < NA; ++w) x += sm[w * NR + k][lane];
+                if (k < ND) d[k < ND ? k : 0] = x;
+                else v[k < ND ? 0 : k - ND] = x;
             }
         }
-    }
-}
+    };
+    const bool rest = __syncthreads_or(skew);
+    total(D, g);
+    if (rest) total(Dd, gd);
+    if (ia >= 3) return;
 
-// Mulliken octupoles (SI, fourth multipole definition):
-//   Omega_k,abc = - sum_{mu in k, nu} gamma_{nu mu} <mu|(r-R_k)_a (r-R_k)_b (r-R_k)_c|nu>.
-// Third 1-D moment about K from the Hermite expansion:
-//   M^3 = (X^3 + 3hX, 3X^2 + 3h, 6X, 6), h = 1/(2p), X = P - K.
-__constant__ int c_o3x[10] = {3, 2, 2, 1, 1, 1, 0, 0, 0, 0};
-__constant__ int c_o3y[10] = {0, 1, 0, 2, 1, 0, 3, 2, 1, 0};
-__constant__ int c_o3z[10] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3};
-
-template <int LA, int LB>
-__global__ void __launch_bounds__(128)
-k_octupoles(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm, double *__restrict__ oct)
-{
-    constexpr int NA = ncart(LA), NB = ncart(LB);
-    const int lane = threadIdx.x & 31;
-    const int i = pp_begin + (blockIdx.x * blockDim.x + threadIdx.x);
-    if (pp_begin + (int)((blockIdx.x * blockDim.x + (threadIdx.x & ~31))) >= pp_end) return;  // whole warp out
-    const PPLane pl = load_pp(bd, i, pp_end);
-    const bool mirror = pl.sp.shA != pl.sp.shB;
-    // 1-D moments of order 0 and 3 about A and B, per direction (orders 1, 2 are not needed)
-    double SA[3][LA + 1][LB + 1][4], SB[3][LA + 1][LB + 1][4];
-    {
-        double E[LA + 1][LB + 1][LA + LB + 1];
-        const double h = 0.5 * pl.ip;
+    if constexpr (MULT) {
+        // about A from D (warp 0), about B from D plus the antisymmetric rest (warp 1, or 0 again)
 #pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            if (ia != (NA > 1 ? side : 0)) continue;
+            if (side && rest) {
+#pragma unroll
+                for (int k = 0; k < ND; ++k) D[k] += Dd[k];
+            }
+            const Mom1<ORD> mx(side ? XB[0] : XA[0], h), my(side ? XB[1] : XA[1], h), mz(side ? XB[2] : XA[2], h);
+            const int at = side ? atomB : atomA;
+#pragma unroll
+            for (int k = 0; k < 10; ++k) {
+                const int ox = ORD == 2 ? op_x(k) : o3_x(k), oy = ORD == 2 ? op_y(k) : o3_y(k),
+                          oz = ORD == 2 ? op_z(k) : o3_z(k);
+                double m = 0.0;
+#pragma unroll
+                for (int t = 0; t <= ox; ++t)
+#pragma unroll
+                    for (int u = 0; u <= oy; ++u)
+#pragma unroll
+                        for (int v = 0; v <= oz; ++v)
+                            if (t + u + v <= TM)
+                                m += mx.m[ox][t] * my.m[oy][u] * mz.m[oz][v] * D[t + u + v <= TM ? hidx(t, u, v) : 0];
+                const double v = seg_reduce(side && !mirror ? 0.0 : -coef * m, take);
+                if (head && active && (!side || mirror)) atomicAdd(mult + 10 * at + k, v);
+            }
+        }
+    }
+    if constexpr (PULAY) {
+        if (ia != (NA > 1 ? 2 : 0)) return;
+        double HA[10], HB[10], K[10];
+        potential_hermite(phi + 20 * (size_t)atomA, XA, h, HA);
+        potential_hermite(phi + 20 * (size_t)atomB, XB, h, HB);
+        if (MULT && NA == 1 && rest) {  // this warp's D was B's
+#pragma unroll
+            for (int k = 0; k < ND; ++k) D[k] -= Dd[k];
+        }
+        // D (b/p H^A - a/p H^B) raised once per direction; the antisymmetric rest only meets H^B
+#pragma unroll
+        for (int k = 0; k < 10; ++k) K[k] = b * ip * HA[k] - a * ip * HB[k];
+#pragma unroll
         for (int d = 0; d < 3; ++d) {
-            hermite_E<LA, LB, double>(E, pl.P[d] - pl.A[d], pl.P[d] - pl.B[d], h);
-            const double XA = pl.P[d] - pl.A[d], XB = pl.P[d] - pl.B[d];
+            double v = -g[d], w = -gd[d];
 #pragma unroll
-            for (int a = 0; a <= LA; ++a)
-#pragma unroll
-                for (int b = 0; b <= LB; ++b) {
-                    // E^{ab}_t vanishes for t > a + b; the array holds t <= LA + LB only
-                    const double e0 = E[a][b][0];
-                    double e1 = 0.0, e2 = 0.0, e3 = 0.0;
-                    if constexpr (LA + LB >= 1) e1 = (a + b >= 1) ? E[a][b][1] : 0.0;
-                    if constexpr (LA + LB >= 2) e2 = (a + b >= 2) ? E[a][b][2] : 0.0;
-                    if constexpr (LA + LB >= 3) e3 = (a + b >= 3) ? E[a][b][3] : 0.0;
-                    SA[d][a][b][0] = e0;
-                    SA[d][a][b][1] = XA * e0 + e1;
-                    SA[d][a][b][2] = (XA * XA + h) * e0 + 2.0 * XA * e1 + 2.0 * e2;
-                    SA[d][a][b][3] = (XA * XA + 3.0 * h) * XA * e0 + 3.0 * (XA * XA + h) * e1 + 6.0 * XA * e2 + 6.0 * e3;
-                    SB[d][a][b][0] = e0;
-                    SB[d][a][b][1] = XB * e0 + e1;
-                    SB[d][a][b][2] = (XB * XB + h) * e0 + 2.0 * XB * e1 + 2.0 * e2;
-                    SB[d][a][b][3] = (XB * XB + 3.0 * h) * XB * e0 + 3.0 * (XB * XB + h) * e1 + 6.0 * XB * e2 + 6.0 * e3;
-                }
-        }
-    }
-    const double spp = PI * pl.ip;
-    const double coef = pl.active ? pl.cab * spp * sqrt(spp) : 0.0;
-    bool take[5], head;
-    seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-    double mA[10], mB[10];
-#pragma unroll
-    for (int k = 0; k < 10; ++k) mA[k] = mB[k] = 0.0;
-#pragma unroll 1
-    for (int ia = 0; ia < NA; ++ia) {
-#pragma unroll 1
-        for (int ib = 0; ib < NB; ++ib) {
-            const int ax = cart_lx(LA, ia), ay = cart_ly(LA, ia), az = cart_lz(LA, ia);
-            const int bx = cart_lx(LB, ib), by = cart_ly(LB, ib), bz = cart_lz(LB, ib);
-            const size_t r = pl.sp.aoA + ia, c = pl.sp.aoB + ib;
-            const double g_ba = pl.active ? dm[c * bd.nao + r] : 0.0;
-            const double g_ab = pl.active ? dm[r * bd.nao + c] : 0.0;
-#pragma unroll
-            for (int op = 0; op < 10; ++op) {
-                const int ox = c_o3x[op], oy = c_o3y[op], oz = c_o3z[op];
-                mA[op] -= g_ba * SA[0][ax][bx][ox] * SA[1][ay][by][oy] * SA[2][az][bz][oz];
-                mB[op] -= g_ab * SB[0][ax][bx][ox] * SB[1][ay][by][oy] * SB[2][az][bz][oz];
+            for (int k = 0; k < (TM >= 1 ? 4 : 1); ++k) {
+                const int t = k == 1, u = k == 2, z = k == 3;
+                const int up = hidx(t + (d == 0), u + (d == 1), z + (d == 2));
+                v += D[hidx(t, u, z)] * K[up];
+                if (rest) w -= Dd[hidx(t, u, z)] * (a * ip * HB[up]);
+            }
+            v = seg_reduce(two ? coef * (v + w) : 0.0, take);
+            if (head && active && two) {
+                atomicAdd(gqm + 3 * atomA + d, v);
+                atomicAdd(gqm + 3 * atomB + d, -v);
             }
         }
     }
-#pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        const double va = seg_reduce(coef * mA[k], take);
-        const double vb = seg_reduce(mirror ? coef * mB[k] : 0.0, take);
-        if (head && pl.active) {
-            atomicAdd(oct + 10 * pl.atomA + k, va);
-            if (mirror) atomicAdd(oct + 10 * pl.atomB + k, vb);
-        }
+}
+
+template <int LA, int LB, int ORD, bool MULT, bool FOCK, bool PULAY>
+static cudaError_t launch_mom(const BasisDev &bd, int pp_begin, int pp_end, const double *dm, const double *phi,
+                              double *mult, double *F, double *gqm, cudaStream_t st)
+{
+    const size_t smem = (size_t)MomShape<LA, LB, ORD, FOCK, PULAY>::NS * 32 * sizeof(double);
+    auto kern = k_moments<LA, LB, ORD, MULT, FOCK, PULAY>;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
     }
+    kern<<<(pp_end - pp_begin + 31) / 32, dim3(32, ncart(LA)), smem, st>>>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm);
+    return cudaGetLastError();
 }
 
 template <int LA, int LB>
@@ -505,9 +432,7 @@ struct Octupoles {
     static cudaError_t run(const BasisDev &bd, int pp_begin, int pp_end, const double *dm, double *oct,
                            cudaStream_t st)
     {
-        const int grid = (pp_end - pp_begin + 127) / 128;
-        k_octupoles<LA, LB><<<grid, 128, 0, st>>>(bd, pp_begin, pp_end, dm, oct);
-        return cudaGetLastError();
+        return launch_mom<LA, LB, 3, true, false, false>(bd, pp_begin, pp_end, dm, nullptr, oct, nullptr, nullptr, st);
     }
 };
 
@@ -523,17 +448,17 @@ struct Moments {
     static cudaError_t run(const BasisDev &bd, int pp_begin, int pp_end, const double *dm, const double *phi,
                            double *mult, double *F, double *gqm, int mode, cudaStream_t st)
     {
-        const int n = pp_end - pp_begin;
-        const int gx = (n + 127) / 128;
-        if (!(mode & MOM_PULAY)) {
-            k_moments<LA, LB><<<gx, 128, 0, st>>>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, mode);
-            return cudaGetLastError();
+        switch (mode) {
+        case MOM_MULT: return launch_mom<LA, LB, 2, true, false, false>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, st);
+        case MOM_MULT | MOM_FOCK:
+            return launch_mom<LA, LB, 2, true, true, false>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, st);
+        case MOM_MULT | MOM_PULAY:
+            return launch_mom<LA, LB, 2, true, false, true>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, st);
+        case MOM_PULAY: return launch_mom<LA, LB, 2, false, false, true>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, st);
+        case MOM_PULAY | MOM_FOCK:
+            return launch_mom<LA, LB, 2, false, true, true>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, st);
+        default: return cudaErrorInvalidValue;
         }
-        k_mom_a<LA, LB><<<dim3(gx, ncart(LA)), 128, 0, st>>>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, mode);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_mom_b<LA, LB><<<dim3(gx, ncart(LB)), 128, 0, st>>>(bd, pp_begin, pp_end, dm, phi, mult, F, gqm, mode);
-        return cudaGetLastError();
     }
 };
 
