@@ -145,7 +145,7 @@ int qmmm_set_precision(qmmm_handle *h, int precision);
  *   QMMM_RECIP_AUTO [default]: QMMM_RECIP_TENSOR when (kx + 1)(2 ky + 1)(2 kz + 1) N_MM >= 4e7,
  *     else QMMM_RECIP_CUDA_CORES (small systems, where the extra launches outweigh the work).
  * The tensor-core scratch is allocated the first time the method is in effect: fixed-point
- * phase rows (16 (kx + 4 ky + 4 kz + 5) bytes per charge), the B-operand digit planes and the
+ * phase rows (about 20 (kx + 2 ky + 2 kz) bytes per charge), the B-operand digit planes and the
  * structure factor's partial sums (about 3 KB per charge at kmax 16 in all).
  * Recomputes the region-II potential at the current geometry if the method in effect changes.
  * QMMM_ERR_ARG for another value. */

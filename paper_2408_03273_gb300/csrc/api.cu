@@ -204,11 +204,12 @@ struct qmmm_handle {
     DBuf<double2> S, Spart, A, Az, atom_ph;
     DBuf<float4> Adf, Azdf, gSdf, atom_phdf, mm_filt, qm_filt;
     DBuf<int> err;
-    DBuf<int4> tc_phase;  // tensor-core structure factor scratch (allocated on first use)
+    DBuf<unsigned char> tc_phase;  // tensor-core structure factor scratch (allocated on first use)
+    DBuf<double> tc_real;
     DBuf<uint32_t> tc_bpl;
     DBuf<int> tc_part;
     DBuf<double> tc_bmax;
-    DBuf<int4> mmr_phase;  // tensor-core MM-side reciprocal sum scratch
+    DBuf<unsigned char> mmr_phase;  // tensor-core MM-side reciprocal sum scratch
     DBuf<uint32_t> mmr_bpl;
     DBuf<double> mmr_cscale;
     // charge-lane adjoint sweep (mixed path): pair records and per-pair charge sums, one region
@@ -297,7 +298,7 @@ struct qmmm_handle {
         mult_init.release(); gqm.release(); gchg.release(); dq_int.release(); dR_int.release();
         dq_out.release(); dR_out.release(); Epart.release(); partials.release(); out4.release();
         boys32.release(); S.release(); Spart.release(); A.release(); Az.release(); atom_ph.release(); err.release();
-        tc_phase.release(); tc_bpl.release(); tc_part.release(); tc_bmax.release();
+        tc_phase.release(); tc_real.release(); tc_bpl.release(); tc_part.release(); tc_bmax.release();
         mmr_phase.release(); mmr_bpl.release(); mmr_cscale.release();
         Adf.release(); Azdf.release(); gSdf.release(); atom_phdf.release(); mm_filt.release(); qm_filt.release();
         tune_V.release(); tune_dm.release(); tune_gqm.release(); tune_gchg.release();
@@ -390,23 +391,24 @@ int select_recip(qmmm_handle *h)
     if (m == QMMM_RECIP_TENSOR && !h->tc_part.p) {
         const TcShape &sh = h->ew.tcs;
         int rc;
-        if ((rc = h->tc_phase.ensure(sh.phase_rows)) || (rc = h->tc_bpl.ensure(sh.bplane_words)) ||
-            (rc = h->tc_part.ensure(sh.part_ints)) || (rc = h->tc_bmax.ensure(sh.nbmax)))
+        if ((rc = h->tc_phase.ensure(sh.phase_bytes)) || (rc = h->tc_bpl.ensure(sh.bplane_words)) ||
+            (rc = h->tc_real.ensure(sh.real_sums)) || (rc = h->tc_bmax.ensure(sh.nbmax)) || (rc = h->tc_part.ensure(sh.part_ints)))
             return rc;
         // the padding beyond the last charge is copied but never used; keep it defined
-        CUDA_TRY(cudaMemset(h->tc_phase.p, 0, sh.phase_rows * sizeof(int4)));
+        CUDA_TRY(cudaMemset(h->tc_phase.p, 0, sh.phase_bytes));
         h->ew.tcb.phase = h->tc_phase.p;
         h->ew.tcb.bpl = h->tc_bpl.p;
         h->ew.tcb.part = h->tc_part.p;
+        h->ew.tcb.R = h->tc_real.p;
         h->ew.tcb.bmax = h->tc_bmax.p;
         const MmrShape &m0 = h->ew.mms[0], &m1 = h->ew.mms[1];
         if (m0.supported || m1.supported) {
-            if ((rc = h->mmr_phase.ensure(m0.phase_rows)) ||
+            if ((rc = h->mmr_phase.ensure(m0.phase_bytes)) ||
                 (rc = h->mmr_bpl.ensure(std::max(m0.bplane_words, m1.bplane_words))) ||
                 (rc = h->mmr_cscale.ensure(3 * (h->kmax[0] + 1))))
                 return rc;
             // the rows of padding charges are copied but never used; keep them defined
-            CUDA_TRY(cudaMemset(h->mmr_phase.p, 0, m0.phase_rows * sizeof(int4)));
+            CUDA_TRY(cudaMemset(h->mmr_phase.p, 0, m0.phase_bytes));
             h->ew.mmb.phase = h->mmr_phase.p;
             h->ew.mmb.bpl = h->mmr_bpl.p;
             h->ew.mmb.cscale = h->mmr_cscale.p;

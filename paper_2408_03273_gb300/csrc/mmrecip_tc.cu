@@ -5,14 +5,22 @@
 //
 // over the half space of the kmax cube, with A(G) = 2 g(G) sum_j e^{iG.R_j} (Q_j + i G.mu_j
 // - 1/2 G.theta_j.G) from the QM multipoles and the separable phase e^{-iG.R} = X(n_x) Y(n_y) Z(n_z).
-// Over K = (n_y, n_z) the sum is a product of two matrices followed by a short contraction:
+// Over (n_y, n_z) the sum is a product of two matrices followed by a short contraction:
 //
 //   T_k[i, n_x] = sum_{n_y, n_z} C_k[n_x, n_y, n_z] Y_i(n_y) Z_i(n_z),   C_0 = A, C_1 = G_y A, C_2 = G_z A,
 //   dE/dq_i = Re sum X_i T_0,  f_x = sum G_x Im(X_i T_0),  f_y = sum Im(X_i T_1),  f_z = sum Im(X_i T_2).
 //
-// A operand (M = 128 charges x K): the outer products Y_i(n_y) Z_i(n_z), digitised on chip from
-// fixed-point phase rows staged by TMA; B operand (N = 112 rows (k, n_x, re/im) x K): C_k divided
-// by a power of two per (k, n_x) so that |C| <= 1, digitised once per call into the shared-memory
+// The phases of +n and -n are conjugate, so the product is taken over real functions: per axis
+// cos(2 pi n u), n = 0..k, and sin(2 pi n u), n = 1..k, and K = (2 ky + 1)(2 kz + 1) products of one of
+// each, their complex coefficients B_k the sums of the four C_k(+-n_y, +-n_z) with factors 1, -i, i.
+// Over complex phases K was twice as long and an entry cost two multiplications.  Sum of a 150-atom
+// site (kmax 24, 200 001 charges), mixed path: 4.36 -> 2.64 ms with the real functions, -> 2.02 ms with the
+// z rows resident in shared memory and the y rows of a chunk in one copy; FP64 path 14.9 -> 8.0 ms.
+// Bound: the producers' integer work and barrier round trips per chunk (tensor pipe a third busy).
+//
+// A operand (M = 128 charges x K): the products of the charges' real phases, digitised on chip from
+// fixed-point phase rows staged by TMA; B operand (N = 112 rows (k, n_x, re/im) x K): B_k divided
+// by a power of two per (k, n_x) so that |B| <= 1, digitised once per call into the shared-memory
 // layout.  Digits as for the structure factor (tc_digits.cuh).  FP64 path: seven planes per operand
 // (48-bit fixed point), 28 plane pairs per K-step into FP32 accumulators in tensor memory, five
 // accumulators (levels 0..3 kept apart, 4..6 merged), so at most 96 N rows per tile.  Mixed path:
@@ -22,7 +30,7 @@
 // N row beyond the 6 (kx + 1) in use is computed.  Against the double-float CUDA-core kernel the
 // mixed path's sum differs by 3e-9 (active site, kmax 16) and 1.3e-8 (large site, kmax 24) of the
 // largest MM gradient component, a tenth or less of the mixed path's error against FP64.  Level 0
-// is exact for any input while 4096 x 2 N_y N_z < 2^24 (kmax <= 20) and beyond that unless the
+// is exact for any input while 4096 N_y N_z < 2^24 (kmax <= 31) and beyond that unless the
 // row-normalised coefficients, which decay as exp(-G^2/4 alpha^2), sum to more than 2^11 in
 // magnitude; levels 1 to 3 are sums of random-sign digit products, typically 2^17 or less.  The epilogue
 // (one thread per charge) combines the levels exactly in 64-bit integers, applies the row scales
@@ -40,21 +48,28 @@ namespace {
 using namespace tcd;
 constexpr int MM = 128;                 // charges per tile (MMA M)
 constexpr int NRMAX = 256;              // N rows (channel k, n_x, re/im) of one tile, a multiple of 16
-constexpr int KC = 16;                  // K entries per chunk: 8 (n_y, n_z) pairs x re/im
-constexpr int PCH = KC / 2;             // pairs per chunk
+constexpr int KC = 16;                  // K entries per chunk
+constexpr int YR = 3;                   // y rows that a chunk of 16 entries can touch (N_z >= 8)
 constexpr int NSTGMAX = 3;              // pipeline depth (2 when three stages do not fit)
 constexpr int NACCMAX = 5;              // accumulators: levels 0 .. nacc-2 exact, the rest merged
 constexpr int NPROD = 16;               // producer warps
-constexpr int NTHR = (NPROD + 2) * 32;  // + MMA warp + loader warp
+constexpr int NGRP = 2;                 // groups of producer warps, taking the chunks in turn
+constexpr int NTHR = (NPROD + 3) * 32;  // + MMA warp + phase loader + B plane loader
+constexpr int NYB = 4;                  // buffers of y rows, one chunk's each
 constexpr uint32_t CMK = 128;                    // byte step between core matrices along K
 constexpr uint32_t CMN = (KC / 8) * 128;         // byte step between 8-row groups
 constexpr uint32_t APL = MM * KC * 2;            // A plane bytes per chunk
-constexpr uint32_t ROWB = MM * 16;               // one staged phase row (128 charges, int4)
-constexpr uint32_t PBUF = (2 + PCH) * ROWB;      // Y rows n_y0, n_y0 + 1 and one Z row per pair
+constexpr uint32_t RSTR = MM * 8 + 16;           // bytes of one phase row (128 charges, int2) with its padding:
+                                                 // 16 lanes that read four charges of four rows meet 32
+                                                 // distinct banks; global memory holds the rows the same way
+constexpr uint32_t YBUF = YR * RSTR;             // a chunk's y rows
 constexpr size_t SMEM_MAX = 232448;
 __host__ __device__ inline uint32_t mmr_bpl(int nr) { return (uint32_t)nr * KC * 2; }  // B plane bytes
 __host__ __device__ inline uint32_t mmr_stage(int nr, int np) { return np * (APL + mmr_bpl(nr)); }
-__host__ inline size_t mmr_smem(int nr, int nstg, int np) { return nstg * (size_t)(mmr_stage(nr, np) + PBUF) + 256; }
+__host__ inline size_t mmr_smem(int nr, int nstg, int NZ, int np)
+{
+    return nstg * (size_t)mmr_stage(nr, np) + (size_t)NZ * RSTR + NYB * YBUF + 256;
+}
 // fixed-point width of an operand with NP planes, and the balanced input w of a value at 2^(bits + shift)
 __host__ __device__ constexpr int mmr_bits(int np) { return 6 + 7 * (np - 1); }
 template <int NP>
@@ -64,13 +79,14 @@ __device__ __forceinline__ long long fixw_n(long long v, int shift)
 }
 
 struct MmrArgs {
-    const int4 *Yt, *Zt;   // [NY][npad], [NZ][npad] split 2^61 fixed point, e^{-2 pi i n u}
+    const unsigned char *Yt, *Zt;  // per charge tile NY + 2 and NZ rows of RSTR bytes: split 2^61 fixed
+                                   // point, cos rows, then sin rows
     const uint32_t *bpl;   // B planes per chunk (NP * BPL bytes)
     const double *cscale;  // [3][NX] power-of-two row scales
     const double *mm_xyz, *mm_q;
     double *dq, *dR;
     int *err;
-    int nmm, npad, NX, NY, NZ, npair, nchunk;
+    int nmm, NX, NY, NZ, nent, nchunk;
     int nr, nr_last, cpt, nstg;  // N rows of a tile and of the last tile, channels per tile, stages
     int nacc;                  // accumulators (3 or 5)
     double box0;
@@ -152,10 +168,12 @@ __global__ void __launch_bounds__(NTHR, 1) k_mm_recip_tc(MmrArgs a)
     // the last N tile may hold fewer channels and rows; the smem layout follows its own NR
     const int NSTG = a.nstg, NR = (int)blockIdx.y + 1 == (int)gridDim.y ? a.nr_last : a.nr;
     const uint32_t BPL = mmr_bpl(NR), STG = mmr_stage(NR, NP);
-    unsigned char *pbuf0 = sm + NSTG * STG;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(pbuf0 + NSTG * PBUF);
-    uint64_t *full = bars, *bfull = bars + NSTGMAX, *pfull = bars + 2 * NSTGMAX, *empty = bars + 3 * NSTGMAX;
-    uint64_t *done = bars + 4 * NSTGMAX;
+    unsigned char *zrows = sm + NSTG * STG, *ybuf = zrows + a.NZ * RSTR;
+    // per stage: full (producers), bfull (B copy), empty (MMA done); per y buffer: yfull (copy), yempty
+    // (producers have read it); zfull; done
+    uint64_t *bars = reinterpret_cast<uint64_t *>(ybuf + NYB * YBUF);
+    uint64_t *full = bars, *bfull = bars + NSTGMAX, *empty = bars + 2 * NSTGMAX;
+    uint64_t *yfull = bars + 3 * NSTGMAX, *yempty = yfull + NYB, *zfull = yempty + NYB, *done = zfull + 1;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1);
     volatile int *abort = reinterpret_cast<volatile int *>(tslot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -166,11 +184,15 @@ __global__ void __launch_bounds__(NTHR, 1) k_mm_recip_tc(MmrArgs a)
 
     if (threadIdx.x == 0) {
         for (int k = 0; k < NSTGMAX; ++k) {
-            mbar_init(&full[k], NPROD);
+            mbar_init(&full[k], NPROD / NGRP);
             mbar_init(&bfull[k], 1);
-            mbar_init(&pfull[k], 1);
             mbar_init(&empty[k], 1);
         }
+        for (int k = 0; k < NYB; ++k) {
+            mbar_init(&yfull[k], 1);
+            mbar_init(&yempty[k], NPROD / NGRP);
+        }
+        mbar_init(zfull, 1);
         mbar_init(done, 1);
         *abort = 0;
         fence_mbar_init();
@@ -189,51 +211,56 @@ __global__ void __launch_bounds__(NTHR, 1) k_mm_recip_tc(MmrArgs a)
     };
 
     if (warp < NPROD) {
-        // ---------------- producers: A planes, 128 charges x 8 pairs per chunk ----------------
-        // groups of 8 charges x 4 pairs (32 distinct banks), two per warp
-        constexpr int AJ = 2;
-        int e_m[AJ], e_j[AJ];
+        // ---------------- producers: A planes, 128 charges x 16 entries per chunk ----------------
+        // groups of 8 charges x 4 pairs of entries (32 distinct banks)
+        constexpr int AJ = 32 * NGRP / NPROD;
+        const int grp = warp / (NPROD / NGRP), gw = warp % (NPROD / NGRP);
+        int e_m[AJ], e_k[AJ];
         uint32_t e_off[AJ];
 #pragma unroll
         for (int j = 0; j < AJ; ++j) {
-            const int combo = warp * AJ + j, rg = combo >> 1, cg = combo & 1;
+            const int combo = gw * AJ + j, rg = combo >> 1, cg = combo & 1;
             e_m[j] = rg * 8 + (lane >> 2);
-            e_j[j] = cg * 4 + (lane & 3);
+            e_k[j] = 2 * (cg * 4 + (lane & 3));
             e_off[j] = rg * CMN + cg * CMK + (lane >> 2) * 16 + (lane & 3) * 4;
         }
-        int z0 = 0;  // p0 mod NZ, p0 = ch * PCH (the chunk's first pair)
-        for (int ch = 0; ch < a.nchunk; ++ch, z0 = z0 + PCH >= a.NZ ? z0 + PCH - a.NZ : z0 + PCH) {
-            const int st = ch % NSTG, u = ch / NSTG;
-            if (ch >= NSTG && !tc::mbar_wait_thread(&empty[st], (u - 1) & 1, abort)) {
-                give_up();
-                break;
-            }
-            if (!tc::mbar_wait_thread(&pfull[st], u & 1, abort)) {
+        int z0 = grp * KC % a.NZ;  // z index of the chunk's first entry
+        for (int ch = grp; ch < a.nchunk; ch += NGRP, z0 = (z0 + NGRP * KC) % a.NZ) {
+            const int st = ch % NSTG, u = ch / NSTG, yb = ch % NYB;
+            if ((ch >= NSTG && !tc::mbar_wait_thread(&empty[st], (u - 1) & 1, abort)) ||
+                (ch == grp && !tc::mbar_wait_thread(zfull, 0, abort)) ||
+                !tc::mbar_wait_thread(&yfull[yb], (ch / NYB) & 1, abort)) {
                 give_up();
                 break;
             }
             unsigned char *sA = sm + st * STG;
-            const int4 *Ys = reinterpret_cast<const int4 *>(pbuf0 + st * PBUF), *Zs = Ys + 2 * MM;
-            const int p0 = ch * PCH;
+            const unsigned char *yrows = ybuf + yb * YBUF;
+            const int p0 = ch * KC;
 #pragma unroll
             for (int j = 0; j < AJ; ++j) {
-                const int m = e_m[j], jp = e_j[j], p = p0 + jp;
-                if (m0 + m < a.nmm && p < a.npair) {
-                    long long re, im;  // 2^60 scale; the pair lies in row n_y0 + (z0 + jp >= NZ)
-                    cmul61(Ys[(z0 + jp >= a.NZ ? MM : 0) + m], Zs[jp * MM + m], re, im);
+                const int m = e_m[j];
+                PlanesN<NP> pl[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = e_k[j] + h, z = z0 + k;
+                    const int y = (z >= a.NZ) + (z >= 2 * a.NZ);  // y row of the entry, from the chunk's first
+                    const int2 ys = *reinterpret_cast<const int2 *>(yrows + y * RSTR + m * 8);
+                    const int2 zs = *reinterpret_cast<const int2 *>(zrows + (z - y * a.NZ) * RSTR + m * 8);
                     constexpr int SH = 60 - mmr_bits(NP);
-                    const PlanesN<NP> pr = planes_n<NP>(fixw_n<NP>(re, SH)), pi = planes_n<NP>(fixw_n<NP>(im, SH));
-#pragma unroll
-                    for (int s = 0; s < NP; ++s)
-                        *reinterpret_cast<uint32_t *>(sA + s * APL + e_off[j]) = pack_bf16(pr.p[s], pi.p[s]);
-                } else {
-#pragma unroll
-                    for (int s = 0; s < NP; ++s) *reinterpret_cast<uint32_t *>(sA + s * APL + e_off[j]) = 0u;
+                    long long w = bal<NP>();  // the digits of 0
+                    if (m0 + m < a.nmm && p0 + k < a.nent) w = fixw_n<NP>(rmul61(ys, zs), SH);
+                    pl[h] = planes_n<NP>(w);
                 }
+#pragma unroll
+                for (int s = 0; s < NP; ++s)
+                    *reinterpret_cast<uint32_t *>(sA + s * APL + e_off[j]) = pack_bf16(pl[0].p[s], pl[1].p[s]);
             }
             tc::fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&full[st]);
+            if (lane == 0) {
+                tc::mbar_arrive(&yempty[yb]);
+                tc::mbar_arrive(&full[st]);
+            }
         }
     } else if (warp == NPROD) {
         if (lane == 0) {
@@ -261,50 +288,47 @@ __global__ void __launch_bounds__(NTHR, 1) k_mm_recip_tc(MmrArgs a)
             }
             tc::commit(done);
         }
-    } else {
-        // ---------------- loader warp: phase rows and B planes of chunk ch ----------------
-        // lane 0 waits and posts the expected bytes; the copies of a chunk (two Y rows, one Z row
-        // per pair, the B planes) go out from separate lanes at once
-        int issued = 0, pissued = 0;
+    } else if (warp == NPROD + 1) {
+        if (lane == 0) {
+            // ---------------- phase loader: every z row once, then the y rows of each chunk ----------------
+            // few large copies: with one copy per row of a chunk (19 of 1 KB) their issue set the time of
+            // a chunk (mixed sum of a 150-atom site 2.44 ms, with these copies 2.02)
+            int issued = 0;
+            mbar_arrive_expect_tx(zfull, a.NZ * RSTR);
+            for (uint32_t o = 0; o < a.NZ * RSTR; o += 65536)
+                bulk_g2s(zrows + o, a.Zt + (size_t)blockIdx.x * a.NZ * RSTR + o, min(65536u, a.NZ * RSTR - o), zfull);
+            for (int ch = 0; ch < a.nchunk; ++ch) {
+                const int yb = ch % NYB, u = ch / NYB;
+                if (ch >= NYB && !tc::mbar_wait_thread(&yempty[yb], (u - 1) & 1, abort)) {
+                    give_up();
+                    break;
+                }
+                mbar_arrive_expect_tx(&yfull[yb], YBUF);
+                bulk_g2s(ybuf + yb * YBUF, a.Yt + ((size_t)blockIdx.x * (a.NY + YR - 1) + ch * KC / a.NZ) * RSTR, YBUF,
+                         &yfull[yb]);
+                issued = ch + 1;
+            }
+            // copies possibly still in flight (after a give-up): wait for them to land, bounded in time
+            // only (not cut short by the abort flag), before the block may leave
+            tc::mbar_drain(zfull, 0);
+            for (int ch = issued > NYB ? issued - NYB : 0; ch < issued; ++ch)
+                tc::mbar_drain(&yfull[ch % NYB], (ch / NYB) & 1);
+        }
+    } else if (lane == 0) {
+        // ---------------- B plane loader ----------------
+        int issued = 0;
         for (int ch = 0; ch < a.nchunk; ++ch) {
             const int st = ch % NSTG, u = ch / NSTG;
-            int ok = 1;
-            if (lane == 0 && ch >= NSTG) ok = tc::mbar_wait_thread(&full[st], (u - 1) & 1, abort);
-            if (!__shfl_sync(0xffffffffu, ok, 0)) {
-                if (lane == 0) give_up();
+            if (ch >= NSTG && !tc::mbar_wait_thread(&empty[st], (u - 1) & 1, abort)) {
+                give_up();
                 break;
             }
-            const int p0 = ch * PCH, iy0 = p0 / a.NZ, iy1 = min(iy0 + 1, a.NY - 1);
-            const int nvalid = min(PCH, a.npair - p0);
-            unsigned char *dst = pbuf0 + st * PBUF;
-            if (lane == 0) mbar_arrive_expect_tx(&pfull[st], (2 + nvalid) * ROWB);
-            __syncwarp();
-            if (lane < 2) {
-                bulk_g2s(dst + lane * ROWB, a.Yt + (size_t)(lane ? iy1 : iy0) * a.npad + m0, ROWB, &pfull[st]);
-            } else if (lane < 2 + nvalid) {
-                const int iz = (p0 + lane - 2) % a.NZ;
-                bulk_g2s(dst + lane * ROWB, a.Zt + (size_t)iz * a.npad + m0, ROWB, &pfull[st]);
-            }
-            pissued = ch + 1;
-            if (lane == 0 && ch >= NSTG) ok = tc::mbar_wait_thread(&empty[st], (u - 1) & 1, abort);
-            if (!__shfl_sync(0xffffffffu, ok, 0)) {
-                if (lane == 0) give_up();
-                break;
-            }
-            if (lane == 0) {
-                mbar_arrive_expect_tx(&bfull[st], NP * BPL);
-                bulk_g2s(sm + st * STG + NP * APL, bpl + (size_t)ch * (NP * BPL / 4), NP * BPL, &bfull[st]);
-            }
+            mbar_arrive_expect_tx(&bfull[st], NP * BPL);
+            bulk_g2s(sm + st * STG + NP * APL, bpl + (size_t)ch * (NP * BPL / 4), NP * BPL, &bfull[st]);
             issued = ch + 1;
         }
-        if (lane == 0) {
-            // copies possibly still in flight (after a give-up): wait for them to land, bounded in
-            // time only (not cut short by the abort flag), before the block may leave
-            for (int ch = issued > NSTG ? issued - NSTG : 0; ch < issued; ++ch)
-                tc::mbar_drain(&bfull[ch % NSTG], (ch / NSTG) & 1);
-            for (int ch = pissued > NSTG ? pissued - NSTG : 0; ch < pissued; ++ch)
-                tc::mbar_drain(&pfull[ch % NSTG], (ch / NSTG) & 1);
-        }
+        for (int ch = issued > NSTG ? issued - NSTG : 0; ch < issued; ++ch)
+            tc::mbar_drain(&bfull[ch % NSTG], (ch / NSTG) & 1);
     }
 
     // ---------------- epilogue: one thread per charge (warps 0..3) ----------------
@@ -379,24 +403,25 @@ __global__ void __launch_bounds__(NTHR, 1) k_mm_recip_tc(MmrArgs a)
     }
 }
 
-// Y_i(n_y) = e^{-2 pi i n_y u_y}, Z_i(n_z) = e^{-2 pi i n_z u_z} in rows over the charges:
-// Yt[iy][i], Zt[iz][i] (index iy = n_y + ky), split 2^61 fixed point.  One thread per (axis,
-// charge): the start and the step from FP64 sincospi, the recurrence in fixed point.
-__global__ void k_mmr_phases(EwaldDev e, int npad, int4 *Yt, int4 *Zt)
+// The charges' real phases along y and z, per tile of 128 charges: row r = 0..k holds cos(2 pi r u), row
+// k + n sin(2 pi n u), split 2^61 fixed point, RSTR bytes apart; the y rows of a tile are followed by
+// YR - 1 that only pad the last chunks' copies.  One thread per (axis, charge): the step from FP64
+// sincospi, the recurrence in fixed point.
+__global__ void k_mmr_phases(EwaldDev e, unsigned char *Yt, unsigned char *Zt)
 {
     const long long item = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= 2ll * e.nmm) return;
     const int d = 1 + (int)(item / e.nmm), i = (int)(item - (long long)(d - 1) * e.nmm);
-    const int k = e.kmax[d], len = 2 * k + 1;
-    int4 *col = (d == 1 ? Yt : Zt) + i;
+    const int k = e.kmax[d], rows = 2 * k + (d == 1 ? YR : 1);
+    unsigned char *col = (d == 1 ? Yt : Zt) + (size_t)(i / MM) * rows * RSTR + (i % MM) * 8;
     const double u = e.mm_xyz[3 * i + d] / e.box[d];
     double sn, cs;
-    sincospi(-2.0 * u, &sn, &cs);
+    sincospi(2.0 * u, &sn, &cs);
     const long long sr = fix61(cs), si = fix61(sn);
-    sincospi(2.0 * (double)k * u, &sn, &cs);  // index 0 is n = -k
-    long long pr = fix61(cs), pi = fix61(sn);
-    for (int n = 0; n < len; ++n) {
-        col[(size_t)n * npad] = split61(pr, pi);
+    long long pr = fix61(1.0), pi = 0;
+    for (int n = 0; n <= k; ++n) {
+        *reinterpret_cast<int2 *>(col + (size_t)n * RSTR) = split61r(pr);
+        if (n > 0) *reinterpret_cast<int2 *>(col + (size_t)(k + n) * RSTR) = split61r(pi);
         const long long nr = (mul61(pr, sr) - mul61(pi, si)) * 2;
         const long long ni = (mul61(pr, si) + mul61(pi, sr)) * 2;
         pr = nr;
@@ -412,7 +437,28 @@ __device__ __forceinline__ double2 mmr_channel(const double2 *A, const double2 *
     return k == 1 ? make_double2(gy * c.x, gy * c.y) : c;
 }
 
-// cscale[k NX + n_x] = 2^e >= max over (n_y, n_z) of |Re C_k|, |Im C_k| (1 where C_k vanishes);
+// Coefficient B_k of the product of real phase functions p = (ry, rz) at n_x: the sum over the signs of
+// (n_y, n_z) of C_k times 1 for a cosine, -i (n > 0) or i (n < 0) for a sine
+__device__ __forceinline__ double2 mmr_coef(const EwaldDev &e, const double2 *A, const double2 *Az, int k, int nx, int p)
+{
+    const int ky = e.kmax[1], kz = e.kmax[2], NY = 2 * ky + 1, NZ = 2 * kz + 1;
+    const int ry = p / NZ, rz = p - ry * NZ;
+    const bool siny = ry > ky, sinz = rz > kz;
+    const int ny = siny ? ry - ky : ry, nz = sinz ? rz - kz : rz;
+    double2 s = make_double2(0.0, 0.0);
+    for (int sy = ny ? -1 : 1; sy <= 1; sy += 2)
+        for (int sz = nz ? -1 : 1; sz <= 1; sz += 2) {
+            const double gy = 6.283185307179586476925 * (sy * ny) / e.box[1];
+            double2 c = mmr_channel(A, Az, k, ((size_t)nx * NY + sy * ny + ky) * NZ + sz * nz + kz, gy);
+            if (siny) c = sy > 0 ? make_double2(c.y, -c.x) : make_double2(-c.y, c.x);
+            if (sinz) c = sz > 0 ? make_double2(c.y, -c.x) : make_double2(-c.y, c.x);
+            s.x += c.x;
+            s.y += c.y;
+        }
+    return s;
+}
+
+// cscale[k NX + n_x] = 2^e >= max over the entries of |Re B_k|, |Im B_k| (1 where B_k vanishes);
 // one block per (k, n_x)
 __global__ void __launch_bounds__(256) k_mmr_scale(EwaldDev e, const double2 *A, const double2 *Az, double *cscale)
 {
@@ -421,9 +467,7 @@ __global__ void __launch_bounds__(256) k_mmr_scale(EwaldDev e, const double2 *A,
     const int k = blockIdx.x / NX, nx = blockIdx.x % NX;
     double m = 0.0;
     for (int t = threadIdx.x; t < NY * NZ; t += 256) {
-        const int iy = t / NZ;
-        const double gy = 6.283185307179586476925 * (iy - e.kmax[1]) / e.box[1];
-        const double2 c = mmr_channel(A, Az, k, (size_t)nx * NY * NZ + t, gy);
+        const double2 c = mmr_coef(e, A, Az, k, nx, t);
         m = fmax(m, fmax(fabs(c.x), fabs(c.y)));
     }
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -438,32 +482,34 @@ __global__ void __launch_bounds__(256) k_mmr_scale(EwaldDev e, const double2 *A,
     }
 }
 
-// B planes of one N tile (channels [kfirst, kfirst + nk)), per chunk of 8 (n_y, n_z) pairs, in the
-// shared-memory layout: row (k, n_x, 0) holds (Re C, -Im C), row (k, n_x, 1) holds (Im C, Re C)
-// of C_k / cscale.  A warp writes 8 rows x 4 pairs: 128 contiguous bytes of each plane.
+// B planes of one N tile (channels [kfirst, kfirst + nk)), per chunk of 16 entries, in the
+// shared-memory layout: row (k, n_x, 0) holds Re B_k / cscale, row (k, n_x, 1) Im B_k / cscale.  A warp
+// writes 8 rows x 4 pairs of entries: 128 contiguous bytes of each plane.
 template <int NP>
 __global__ void k_mmr_bplanes(EwaldDev e, const double2 *A, const double2 *Az, const double *cscale, int kfirst,
                               int nk, int nr, int nchunk, uint32_t *bpl)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long per = (long long)nr * PCH;  // (row, pair) items of one chunk
+    const long long per = (long long)nr * (KC / 2);  // (row, pair of entries) items of one chunk
     if (t >= per * nchunk) return;
     const int ch = (int)(t / per), it = (int)(t - (long long)ch * per);
-    const int NX = e.kmax[0] + 1, NY = 2 * e.kmax[1] + 1, NZ = 2 * e.kmax[2] + 1;
+    const int NX = e.kmax[0] + 1, nent = (2 * e.kmax[1] + 1) * (2 * e.kmax[2] + 1);
     const int lane = it & 31, grp = it >> 5;
     const int j = (grp & 1) * 4 + (lane & 3), n = (grp >> 1) * 8 + (lane >> 2);
-    const int p = ch * PCH + j;
     long long w0 = bal<NP>(), w1 = bal<NP>();
-    if (n < 2 * nk * NX && p < NY * NZ) {
+    if (n < 2 * nk * NX) {
         const int kl = n / (2 * NX), nx = (n % (2 * NX)) >> 1, r = n & 1, k = kfirst + kl;
-        const int iy = p / NZ, iz = p - iy * NZ;
-        const double gy = 6.283185307179586476925 * (iy - e.kmax[1]) / e.box[1];
-        const double2 c = mmr_channel(A, Az, k, ((size_t)nx * NY + iy) * NZ + iz, gy);
-        const double sc = 1.0 / cscale[k * NX + nx];  // a power of two: exact
-        const double re = c.x * sc, im = c.y * sc;
-        constexpr double SC = (double)(1ll << mmr_bits(NP));
-        w0 += __double2ll_rn((r ? im : re) * SC);
-        w1 += __double2ll_rn((r ? re : -im) * SC);
+        // over the power-of-two scale (exact), to fixed point
+        const double sc = (double)(1ll << mmr_bits(NP)) / cscale[k * NX + nx];
+        const int p = ch * KC + 2 * j;
+        if (p < nent) {
+            const double2 c = mmr_coef(e, A, Az, k, nx, p);
+            w0 += __double2ll_rn((r ? c.y : c.x) * sc);
+        }
+        if (p + 1 < nent) {
+            const double2 c = mmr_coef(e, A, Az, k, nx, p + 1);
+            w1 += __double2ll_rn((r ? c.y : c.x) * sc);
+        }
     }
     const PlanesN<NP> p0 = planes_n<NP>(w0), p1 = planes_n<NP>(w1);
     const uint32_t words = mmr_bpl(nr) / 4;
@@ -483,9 +529,8 @@ void tc_mmr_shape(const EwaldDev &e, int nacc, int np, MmrShape &sh)
     const int NX = e.kmax[0] + 1, NY = 2 * e.kmax[1] + 1, NZ = 2 * e.kmax[2] + 1;
     sh.nacc = nacc;
     sh.mtiles = (e.nmm + MM - 1) / MM;
-    sh.npad = sh.mtiles * MM;
-    sh.npair = NY * NZ;
-    sh.nchunk = (sh.npair + PCH - 1) / PCH;
+    sh.nent = NY * NZ;
+    sh.nchunk = (sh.nent + KC - 1) / KC;
     const int maxr = std::min(NRMAX, 512 / nacc / 16 * 16);  // N rows that fit nacc accumulators
     int cpt = 3;  // channels per N tile: 2 cpt NX rows
     while (cpt > 1 && 2 * cpt * NX > maxr) --cpt;
@@ -493,15 +538,16 @@ void tc_mmr_shape(const EwaldDev &e, int nacc, int np, MmrShape &sh)
     sh.ntiles = (3 + cpt - 1) / cpt;
     sh.nr = (2 * cpt * NX + 15) / 16 * 16;
     sh.nr_last = (2 * (3 - (sh.ntiles - 1) * cpt) * NX + 15) / 16 * 16;
-    sh.supported = sh.nr <= maxr && NZ >= PCH;  // a chunk of 8 pairs spans at most two n_y rows
-    sh.nstg = mmr_smem(sh.nr, 3, np) <= SMEM_MAX ? 3 : 2;
-    sh.phase_rows = (size_t)(NY + NZ) * sh.npad;
+    // a chunk of 16 entries touches at most YR y rows from N_z = 8
+    sh.supported = sh.nr <= maxr && NZ >= 8 && mmr_smem(sh.nr, 2, NZ, np) <= SMEM_MAX;
+    sh.nstg = mmr_smem(sh.nr, 3, NZ, np) <= SMEM_MAX ? 3 : 2;
+    sh.phase_bytes = (size_t)sh.mtiles * (NY + YR - 1 + NZ) * RSTR;
     sh.bplane_words = ((size_t)(sh.ntiles - 1) * mmr_bpl(sh.nr) + mmr_bpl(sh.nr_last)) * sh.nchunk * np / 4;
 }
 
 template <int NP>
 static cudaError_t mm_recip_np(const EwaldDev &e, const MmrShape &sh, const MmrBuf &b, const double2 *A,
-                               const double2 *Az, const int4 *Yt, const int4 *Zt, double *dq, double *dR, int *err,
+                               const double2 *Az, const unsigned char *Yt, const unsigned char *Zt, double *dq, double *dR, int *err,
                                cudaStream_t st);
 
 cudaError_t launch_mm_recip_tc(const EwaldDev &e, const MmrShape &sh, const MmrBuf &b, const double2 *A,
@@ -510,8 +556,8 @@ cudaError_t launch_mm_recip_tc(const EwaldDev &e, const MmrShape &sh, const MmrB
     if (e.nmm == 0) return cudaSuccess;
     cudaError_t rc;
     const int NX = e.kmax[0] + 1, NY = 2 * e.kmax[1] + 1;
-    int4 *Yt = b.phase, *Zt = Yt + (size_t)NY * sh.npad;
-    k_mmr_phases<<<(unsigned)((2ll * e.nmm + 255) / 256), 256, 0, st>>>(e, sh.npad, Yt, Zt);
+    unsigned char *Yt = b.phase, *Zt = Yt + (size_t)sh.mtiles * (NY + YR - 1) * RSTR;
+    k_mmr_phases<<<(unsigned)((2ll * e.nmm + 255) / 256), 256, 0, st>>>(e, Yt, Zt);
     if ((rc = cudaGetLastError()) != cudaSuccess) return rc;
     k_mmr_scale<<<3 * NX, 256, 0, st>>>(e, A, Az, b.cscale);
     if ((rc = cudaGetLastError()) != cudaSuccess) return rc;
@@ -523,12 +569,12 @@ cudaError_t launch_mm_recip_tc(const EwaldDev &e, const MmrShape &sh, const MmrB
 // B planes and the MMA kernel with NP planes per operand
 template <int NP>
 static cudaError_t mm_recip_np(const EwaldDev &e, const MmrShape &sh, const MmrBuf &b, const double2 *A,
-                               const double2 *Az, const int4 *Yt, const int4 *Zt, double *dq, double *dR, int *err,
+                               const double2 *Az, const unsigned char *Yt, const unsigned char *Zt, double *dq, double *dR, int *err,
                                cudaStream_t st)
 {
     cudaError_t rc;
     const int NX = e.kmax[0] + 1, NY = 2 * e.kmax[1] + 1, NZ = 2 * e.kmax[2] + 1;
-    const size_t smem = mmr_smem(sh.nr, sh.nstg, NP);
+    const size_t smem = mmr_smem(sh.nr, sh.nstg, NZ, NP);
     static size_t at = 0;
     if (smem > at) {
         if ((rc = cudaFuncSetAttribute((const void *)k_mm_recip_tc<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -540,7 +586,7 @@ static cudaError_t mm_recip_np(const EwaldDev &e, const MmrShape &sh, const MmrB
     for (int tl = 0; tl < sh.ntiles; ++tl) {
         const int kfirst = tl * sh.cpt, nk = std::min(sh.cpt, 3 - kfirst);
         const int nr = tl + 1 == sh.ntiles ? sh.nr_last : sh.nr;
-        const long long n = (long long)nr * PCH * sh.nchunk;
+        const long long n = (long long)nr * (KC / 2) * sh.nchunk;
         k_mmr_bplanes<NP><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(e, A, Az, b.cscale, kfirst, nk, nr,
                                                                         sh.nchunk, b.bpl + tl * tile_words);
         if ((rc = cudaGetLastError()) != cudaSuccess) return rc;
@@ -556,11 +602,10 @@ static cudaError_t mm_recip_np(const EwaldDev &e, const MmrShape &sh, const MmrB
     a.dR = dR;
     a.err = err;
     a.nmm = e.nmm;
-    a.npad = sh.npad;
     a.NX = NX;
     a.NY = NY;
     a.NZ = NZ;
-    a.npair = sh.npair;
+    a.nent = sh.nent;
     a.nchunk = sh.nchunk;
     a.nr = sh.nr;
     a.nr_last = sh.nr_last;

@@ -156,12 +156,14 @@ struct TcShape {
     int NL = 0, mtiles = 0, ntiles = 0, ntr = 0, nkb = 0;  // lines, line tiles, N tiles (rows each), charge blocks
     int nbmax = 0;           // blocks of the max|q| reduction
     size_t part_ints = 0;    // per-CTA accumulator partials, int32 words
-    size_t phase_rows = 0;   // fixed-point phase entries (int4: re hi/lo, im hi/lo), whole charge blocks
+    size_t phase_bytes = 0;  // fixed-point real phase rows, whole charge blocks
     size_t bplane_words = 0; // digit planes of the B operand (32-bit words), in shared-memory layout
+    size_t real_sums = 0;    // sums over real phase functions (doubles)
     bool staged = false;     // phase rows of each chunk staged in shared memory by TMA bulk copies
 };
 struct TcBuf {
-    int4 *phase = nullptr;      // qX [npad][NX], Y [npad][NY], Z [npad][NZ] (2^61 fixed point, split)
+    unsigned char *phase = nullptr;  // qX, Y, Z rows of every chunk (k_tc_phases)
+    double *R = nullptr;        // sums over real phase functions [NZ][NL]
     uint32_t *bpl = nullptr;    // B digit planes per (charge block, chunk, N tile)
     int *part = nullptr;
     double *bmax = nullptr;     // per-block max |q|
@@ -177,17 +179,17 @@ cudaError_t launch_structure_factor_tc(const EwaldDev &e, const TcShape &sh, con
 // region-I sweeps (about 1e-7 of the largest gradient; the 5-plane sum adds about 1e-8 at most)
 constexpr int MMR_NP_FP64 = 7, MMR_NP_MIXED = 5;
 struct MmrShape {
-    int mtiles = 0, npad = 0, npair = 0, nchunk = 0;  // charge tiles (128), padded charges, (n_y, n_z) pairs, chunks of 8
+    int mtiles = 0, nent = 0, nchunk = 0;             // charge tiles (128), K entries, chunks of 16
     int cpt = 3, ntiles = 1, nr = 0, nstg = 3;        // channels per N tile, N tiles, N rows, stages
     int nr_last = 0;                                  // N rows of the last N tile (fewer channels)
     int nacc = 4;                                     // accumulators (exact levels + 1)
     int np = 7;                                       // digit planes per operand (5 or 7)
     bool supported = false;                           // kx small enough for one channel per tile
-    size_t phase_rows = 0;                            // Y and Z phase rows (int4)
+    size_t phase_bytes = 0;                           // real y and z phase rows
     size_t bplane_words = 0;                          // B digit planes of all N tiles (32-bit words)
 };
 struct MmrBuf {
-    int4 *phase = nullptr;     // Yt [NY][npad], Zt [NZ][npad]
+    unsigned char *phase = nullptr;  // y rows of every charge tile, then z rows (k_mmr_phases)
     uint32_t *bpl = nullptr;   // B planes per N tile and chunk
     double *cscale = nullptr;  // [3][NX] power-of-two row scales
 };

@@ -66,6 +66,12 @@ __device__ __forceinline__ void cmul61(const int4 x, const int4 y, long long &re
     re = (long long)x.x * y.x - (long long)x.z * y.z + (mr >> 31);
     im = (long long)x.x * y.z + (long long)x.z * y.x + (mi >> 31);
 }
+// a real split value, and the product of two at 2^60 scale, within 1 unit
+__device__ __forceinline__ int2 split61r(long long x) { return make_int2((int)(x >> 31), (int)(x & 0x7fffffff)); }
+__device__ __forceinline__ long long rmul61(int2 x, int2 y)
+{
+    return (long long)x.x * y.x + (((long long)x.x * y.y + (long long)x.y * y.x) >> 31);
+}
 // balanced-digit input w of a value v at 2^(48 + shift) scale: rounded to 2^-48, offset by BAL
 __device__ __forceinline__ long long fixw(long long v, int shift)
 {
