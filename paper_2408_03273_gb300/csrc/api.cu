@@ -217,6 +217,8 @@ struct qmmm_handle {
     DBuf<float4> cl_rec;
     DBuf<double> cl_psum;
     size_t cl_rec_off[NCLASS] = {}, cl_psum_off[NCLASS] = {};
+    DBuf<double> pair_ws;  // FP64 adjoint: per-pair density coefficients and charge sums, per class
+    size_t pair_off[NCLASS] = {};
 
     BasisDev basis() const
     {
@@ -304,7 +306,7 @@ struct qmmm_handle {
         tune_V.release(); tune_dm.release(); tune_gqm.release(); tune_gchg.release();
         oct.release(); oct_bins.release(); oct_err.release();
         qmq_ws.release(); qmq_u.release(); qmq_g.release(); qmq_E.release(); qmq_F.release();
-        Vslices.release(); centre_d.release(); cl_rec.release(); cl_psum.release();
+        Vslices.release(); centre_d.release(); cl_rec.release(); cl_psum.release(); pair_ws.release();
     }
 };
 
@@ -680,7 +682,7 @@ constexpr int MAX_SLICES = 16;
 double setup_charges(int L, int kind)
 {
     if (kind_is_mixed(kind)) return 64.0;
-    return kind_is_grad(kind) ? 3.0 + 1.5 * L * L : 3.0 + 0.6 * L * L;
+    return kind_is_grad(kind) ? 3.0 : 3.0 + 0.6 * L * L;  // (the adjoint's pair algebra has kernels of its own)
 }
 
 // How the classes of a sweep over nch charges are cut into blocks: charge slices per class, launch
@@ -794,6 +796,17 @@ int ensure_cl(qmmm_handle *h)
     return QMMM_OK;
 }
 
+// Per-pair scratch of the FP64 adjoint, one region per class.
+int ensure_pairs(qmmm_handle *h)
+{
+    size_t n = 0;
+    for (int c = 0; c < NCLASS; ++c) {
+        h->pair_off[c] = n;
+        n += (size_t)(h->class_off[c + 1] - h->class_off[c]) * vgrad_pair_doubles(la_of_class(c) + lb_of_class(c));
+    }
+    return h->pair_ws.ensure(std::max<size_t>(n, 1));
+}
+
 // One class sweep of the given kind over region-I charges [c0, c1): nblk blocks of `threads` threads
 // in each of nslice block rows (the mixed adjoint: its variant in place of `threads`); V kernels
 // write slice s into V + s * vstride.
@@ -812,7 +825,7 @@ cudaError_t launch_sweep(const qmmm_handle *h, int kind, int cls, int p0, int p1
                                cs);
     case SW_VGRAD_F64:
         return launch_vgrad_f64(b, r, cls, p0, p1, c0, c1, h->boys64.p, ddm, gqm, gchg, h->err.p, nblk, threads,
-                                nslice, cs);
+                                nslice, h->pair_ws.p + h->pair_off[cls], cs);
     case SW_VGRAD_F32: {
         ClScratch cl;
         if (h->cl_rec.p && h->cl_psum.p) {
@@ -1304,6 +1317,15 @@ int qmmm_set_positions(qmmm_handle *h, const double *qm_xyz, const double *mm_xy
     return run_positions(h, qm_xyz, mm_xyz, mm_q);
 }
 
+// The partial V matrices that the V sweep's charge slices write (1: none, straight into V).
+static int ensure_vslices(qmmm_handle *h, int *nbuf)
+{
+    const int kind = sweep_kind(h, false), ch = chunk_for_kind(kind);
+    *nbuf = 1;
+    for (int c0 = 0; c0 < h->nI; c0 += ch) *nbuf = std::max(*nbuf, cut_classes(h, kind, std::min(ch, h->nI - c0)).most);
+    return *nbuf > 1 ? h->Vslices.ensure((size_t)*nbuf * h->nao * h->nao) : QMMM_OK;
+}
+
 // qmmm_vpot in parts (a batch runs the mixed V sweeps of all its frames together):
 // vpot_prep clears V, or the per-slice partial matrices when slices is set (then *Vdst points at
 // them and *nbuf is their count); vpot_sweep runs the class sweeps; vpot_end sums the slices, adds
@@ -1318,10 +1340,8 @@ static int vpot_prep(qmmm_handle *h, bool slices, double **Vdst, int *nbuf)
     *Vdst = h->V.p;
     *nbuf = 1;
     if (!slices) return QMMM_OK;
-    const int kind = sweep_kind(h, false), ch = chunk_for_kind(kind);
-    for (int c0 = 0; c0 < h->nI; c0 += ch) *nbuf = std::max(*nbuf, cut_classes(h, kind, std::min(ch, h->nI - c0)).most);
+    if ((rc = ensure_vslices(h, nbuf))) return rc;
     if (*nbuf > 1) {  // per-slice partial V, summed in a fixed order afterwards
-        if ((rc = h->Vslices.ensure((size_t)*nbuf * n2))) return rc;
         CUDA_TRY(cudaMemsetAsync(h->Vslices.p, 0, (size_t)*nbuf * n2 * sizeof(double), st));
         *Vdst = h->Vslices.p;
     }
@@ -1483,7 +1503,7 @@ static int forces_sweep(qmmm_handle *h, const double *ddm)
 {
     int rc;
     const int kind = sweep_kind(h, true), ch = chunk_for_kind(kind);
-    if (kind == SW_VGRAD_F32 && (rc = ensure_cl(h))) return rc;
+    if ((rc = kind == SW_VGRAD_F32 ? ensure_cl(h) : ensure_pairs(h))) return rc;
     for (int c0 = 0; c0 < h->nI; c0 += ch) {
         const int c1 = std::min(h->nI, c0 + ch);
         rc = run_classes(
@@ -1677,7 +1697,7 @@ int qmmm_autotune(qmmm_handle *h, int flags)
     const int nch = std::min(h->nI, TUNE_CHARGES);
     int rc;
     if ((rc = h->tune_V.ensure(n2)) || (rc = h->tune_dm.ensure(n2)) || (rc = h->tune_gqm.ensure(3 * (size_t)h->natm)) ||
-        (rc = h->tune_gchg.ensure(4 * (size_t)nch)) || (rc = ensure_cl(h)))
+        (rc = h->tune_gchg.ensure(4 * (size_t)nch)) || (rc = ensure_cl(h)) || (rc = ensure_pairs(h)))
         return rc;
     // a zero density: the sweeps' work does not depend on its values
     CUDA_TRY(cudaMemsetAsync(h->tune_dm.p, 0, n2 * sizeof(double), h->stream));
@@ -2075,6 +2095,12 @@ int qmmm_batch_run(qmmm_batch *b, const double *const *dm, double *const *V, dou
             if (batch_defers(b->f[i])) deferred.push_back(i);
         for (int i : deferred)
             if ((rc = ensure_cl(b->f[i]))) break;
+        // the others' sweep scratch, which follows the pair list, likewise
+        for (int i = 0; i < n && !rc; ++i)
+            if (!batch_defers(b->f[i])) {
+                int nbuf;
+                if ((rc = ensure_pairs(b->f[i])) || (rc = ensure_vslices(b->f[i], &nbuf))) break;
+            }
         if (!rc && !deferred.empty()) rc = batch_build_jobs(b, dm);
         if (rc) {
             restore();

@@ -62,40 +62,11 @@ __device__ __forceinline__ double pair_density(const PPLane &pl, const BasisDev 
     return g * (TWO_PI * pl.ip * pl.cab);
 }
 
-// D0_tuv = sum_ab g_ab E^x_t E^y_u E^z_v: the density folded into the Hermite coefficients of the
-// pair (Eq. 9 contracted with the density matrix), once per primitive pair.
-template <int LA, int LB>
-__device__ __forceinline__ void fold_density(const PPLane &pl, const BasisDev &bd, const double *__restrict__ dm,
-                                             double (&D0)[nherm(LA + LB)])
-{
-    constexpr int L = LA + LB, NA = ncart(LA), NB = ncart(LB);
-#pragma unroll
-    for (int k = 0; k < nherm(L); ++k) D0[k] = 0.0;
-    double Ex[LA + 1][LB + 1][L + 1], Ey[LA + 1][LB + 1][L + 1], Ez[LA + 1][LB + 1][L + 1];
-    hermite_E<LA, LB, double>(Ex, pl.P[0] - pl.A[0], pl.P[0] - pl.B[0], 0.5 * pl.ip);
-    hermite_E<LA, LB, double>(Ey, pl.P[1] - pl.A[1], pl.P[1] - pl.B[1], 0.5 * pl.ip);
-    hermite_E<LA, LB, double>(Ez, pl.P[2] - pl.A[2], pl.P[2] - pl.B[2], 0.5 * pl.ip);
-#pragma unroll
-    for (int ia = 0; ia < NA; ++ia)
-#pragma unroll
-        for (int ib = 0; ib < NB; ++ib) {
-            const int ax = cart_lx(LA, ia), ay = cart_ly(LA, ia), az = cart_lz(LA, ia);
-            const int bx = cart_lx(LB, ib), by = cart_ly(LB, ib), bz = cart_lz(LB, ib);
-            const double g = pair_density(pl, bd, dm, ia, ib);
-#pragma unroll
-            for (int t = 0; t <= ax + bx; ++t)
-#pragma unroll
-                for (int u = 0; u <= ay + by; ++u) {
-                    const double gxy = g * Ex[ax][bx][t] * Ey[ay][by][u];
-#pragma unroll
-                    for (int w = 0; w <= az + bz; ++w) D0[hidx(t, u, w)] += gxy * Ez[az][bz][w];
-                }
-        }
-}
-
-// The centre-A derivative coefficients themselves, Da_tuv = sum_ab g_ab E'^a_{tuv} (E'^a as in
-// contract_dA below), for a sweep that contracts them with partial charge sums.
-// With WITH_D0, D0 (as in fold_density) is formed in the same pass.
+// The centre-A derivative coefficients Da_tuv = sum_ab g_ab E'^a_{tuv}, E'^a the product of Hermite
+// coefficients with the factor of direction a replaced by
+//   E'^{ij}_t = dE^{ij}_t / dX_AB = 2a E^{i+1,j}_t - i E^{i-1,j}_t - (a/p) E^{ij}_{t-1}
+// (t <= i + j; E'_{i+j+1} vanishes), for the mixed sweep, which contracts them per charge.
+// With WITH_D0, D0_tuv = sum_ab g_ab E^x_t E^y_u E^z_v is formed in the same pass.
 template <int LA, int LB, bool WITH_D0 = false>
 __device__ __forceinline__ void fold_density_dA(const PPLane &pl, const BasisDev &bd, const double *__restrict__ dm,
                                                 double (&Dx)[nherm(LA + LB)], double (&Dy)[nherm(LA + LB)],
@@ -154,73 +125,6 @@ __device__ __forceinline__ void fold_density_dA(const PPLane &pl, const BasisDev
                         Dz[k] += gx * ey * dEz[w];
                         if constexpr (WITH_D0) D0[k] += gx * ey * ez;
                     }
-        }
-}
-
-// The centre-A derivative part of the adjoint for one primitive pair, contracted with the
-// charge sums S_tuv = sum_C q_C R_tuv(P - C):
-//   d_a = sum_ab g_ab sum_tuv E'^a_{tuv} S_tuv,   a = x, y, z,
-// where E'^a is the product of Hermite coefficients with the a-factor replaced by
-//   E'^{ij}_t = dE^{ij}_t / dX_AB = 2a E^{i+1,j}_t - i E^{i-1,j}_t - (a/p) E^{ij}_{t-1}
-// (t <= i + j; E'_{i+j+1} vanishes).  Per-charge terms d_a(C) = sum E' R(C) enter the pair
-// gradient only through their q-weighted sum, so summing R over the charges first and
-// contracting once per pair gives the same sum.
-template <int LA, int LB>
-__device__ __forceinline__ void contract_dA(const PPLane &pl, const BasisDev &bd, const double *__restrict__ dm,
-                                            const double (&S)[nherm(LA + LB)], double (&d)[3])
-{
-    constexpr int L = LA + LB, NA = ncart(LA), NB = ncart(LB);
-    const double aop = pl.a * pl.ip;
-    d[0] = d[1] = d[2] = 0.0;
-    double Ex[LA + 2][LB + 1][L + 2], Ey[LA + 2][LB + 1][L + 2], Ez[LA + 2][LB + 1][L + 2];
-    hermite_E<LA + 1, LB, double>(Ex, pl.P[0] - pl.A[0], pl.P[0] - pl.B[0], 0.5 * pl.ip);
-    hermite_E<LA + 1, LB, double>(Ey, pl.P[1] - pl.A[1], pl.P[1] - pl.B[1], 0.5 * pl.ip);
-    hermite_E<LA + 1, LB, double>(Ez, pl.P[2] - pl.A[2], pl.P[2] - pl.B[2], 0.5 * pl.ip);
-#pragma unroll
-    for (int ia = 0; ia < NA; ++ia)
-#pragma unroll
-        for (int ib = 0; ib < NB; ++ib) {
-            const int ax = cart_lx(LA, ia), ay = cart_ly(LA, ia), az = cart_lz(LA, ia);
-            const int bx = cart_lx(LB, ib), by = cart_ly(LB, ib), bz = cart_lz(LB, ib);
-            const double g = pair_density(pl, bd, dm, ia, ib);
-            double dEx[L + 1], dEy[L + 1], dEz[L + 1];
-#pragma unroll
-            for (int t = 0; t <= ax + bx; ++t) {
-                double e = 2.0 * pl.a * Ex[ax + 1][bx][t];
-                if (ax > 0) e -= ax * Ex[ax - 1][bx][t];
-                if (t > 0) e -= aop * Ex[ax][bx][t - 1];
-                dEx[t] = e;
-            }
-#pragma unroll
-            for (int u = 0; u <= ay + by; ++u) {
-                double e = 2.0 * pl.a * Ey[ay + 1][by][u];
-                if (ay > 0) e -= ay * Ey[ay - 1][by][u];
-                if (u > 0) e -= aop * Ey[ay][by][u - 1];
-                dEy[u] = e;
-            }
-#pragma unroll
-            for (int w = 0; w <= az + bz; ++w) {
-                double e = 2.0 * pl.a * Ez[az + 1][bz][w];
-                if (az > 0) e -= az * Ez[az - 1][bz][w];
-                if (w > 0) e -= aop * Ez[az][bz][w - 1];
-                dEz[w] = e;
-            }
-            double sx = 0.0, sy = 0.0, sz = 0.0;
-#pragma unroll
-            for (int t = 0; t <= ax + bx; ++t)
-#pragma unroll
-                for (int u = 0; u <= ay + by; ++u)
-#pragma unroll
-                    for (int w = 0; w <= az + bz; ++w) {
-                        const double s = S[hidx(t, u, w)];
-                        const double ex = Ex[ax][bx][t], ey = Ey[ay][by][u], ez = Ez[az][bz][w];
-                        sx += dEx[t] * ey * ez * s;
-                        sy += ex * dEy[u] * ez * s;
-                        sz += ex * ey * dEz[w] * s;
-                    }
-            d[0] += g * sx;
-            d[1] += g * sy;
-            d[2] += g * sz;
         }
 }
 

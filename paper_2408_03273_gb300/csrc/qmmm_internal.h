@@ -72,10 +72,13 @@ struct VJob {
 // into its frame's V; maxch: the most charges of one slice (<= CHUNK_F32).
 cudaError_t launch_vpot_f32_jobs(int cls, const VJob *jobs, int njob, int nblk, int maxch, const float *boys,
                                  int *err, int variant, cudaStream_t st);
+// pairs: scratch of the class, vgrad_pair_doubles(L) per primitive pair (harmonic density
+// coefficients, charge sums)
+__host__ __device__ constexpr int vgrad_pair_doubles(int L) { return (L + 1) * (L + 2) * (L + 3) / 3 + 3; }
 cudaError_t launch_vgrad_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                              int ch_begin, int ch_end, const double *boys, const double *dm, double *gqm,
                              double *gchg /* n*4: dC xyz, dq */, int *err, int nblk, int threads, int nslice,
-                             cudaStream_t st);
+                             double *pairs, cudaStream_t st);
 // Scratch of one class's charge-lane adjoint sweep (mixed path): pair
 // records (cl_rec_floats(L) floats per primitive pair) and per-pair charge sums (6 doubles).
 struct ClScratch {

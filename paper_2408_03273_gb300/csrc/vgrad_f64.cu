@@ -9,16 +9,24 @@
 // (recomputed for every charge, never stored):
 //   dI/dA_a = d_a + (a/p) e_a,   dI/dB_a = -d_a + (b/p) e_a,   dI/dC_a = -e_a,
 // and E contains -q_C I.  The d_a enter only through sum_C q_C d_a(C) = sum Da_tuv W_tuv with
-// W_tuv = sum_C q_C R_tuv, so the sweep accumulates the charge sums and Da is formed and contracted
-// once per pair after it (contract_dA).
+// W_tuv = sum_C q_C R_tuv, so the sweep accumulates the charge sums and Da is contracted with them once
+// per pair after it.  Three kernels per class:
+//   k_pair_fold      D0 of every primitive pair, as solid-harmonic coefficients M (block: 32 pairs x the
+//                    Cartesian components of shell A);
+//   k_vgrad_f64      the sweep: M in, charge gradients and the pairs' charge sums out;
+//   k_pair_contract  Da . W and the pair gradients onto the atoms (blocks as k_pair_fold).
+// With the fold and the contraction in the sweep, one lane did them all for its pair, once per charge
+// slice: some 7 000 FP64 instructions for a (d,d) pair and 30 000 for (f,f), a chain that set the time
+// of small systems.  Sweep of a QM water 0.53 -> 0.34 ms, of 17 atoms with f shells 4.31 -> 2.05 ms; of the
+// 60- and the 150-atom site, which hide the chain, unchanged (45 and 194 ms).
 //
 // Bound: the FP64 pipe, 2 lanes per clock and SM, 85-91% busy, with 7-8% of the issue slots used: the
 // kernel's time is its count of FP64 instructions.  So the tensors R are never formed: D0 and W are
 // kept as solid-harmonic components (harm.cuh), per charge one recursion of (L+1)^2 harmonics, one
 // multiply-add per harmonic for the value, the charge sum and each gradient component (these with
 // the coefficients N of the differentiated harmonics, one order lower).  FP64 instructions per
-// (warp, charge) on a 60-atom active site, setup included: (s,s) 30, (p,p) 77, (d,s) 87, (d,p) 141,
-// (d,d) 262.  Coefficients and sums of the high classes spill to local memory ((f,f): 4.7 KB
+// (warp, charge) on a 60-atom active site, setup included: (s,s) 30, (p,p) 77, (d,s) 87, (d,p) 140,
+// (d,d) 241.  Coefficients and sums of the high classes spill to local memory ((f,f): 2.9 KB
 // stores), which the idle load pipe carries.  Adjoint sweep against the Hermite recursion with its
 // contractions: active site 78.3 -> 60.9 ms, a 150-atom site with f shells 412 -> 242 ms, a QM
 // water 1.35 -> 0.82 ms (untuned handles).
@@ -37,17 +45,251 @@ template <int LA, int LB>
 struct VgradF64 {
     static cudaError_t run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
                            int ch_end, const double *boys, const double *dm, double *gqm, double *gchg, int *err,
-                           int nblk, int threads, int nslice,
-                           cudaStream_t st);
+                           int nblk, int threads, int nslice, double *pairs, cudaStream_t st);
 };
 
 #ifdef QMMM_SPLIT_CLASS  // one angular class per compilation
 
+// ---------------------------------------------------------------------------------------------
+// Per-pair algebra: block (32, NA), lane = primitive pair, warp = component of shell A.  The warps
+// share the pair's 1-D Hermite tables through shared memory.
+// ---------------------------------------------------------------------------------------------
+// E^{ij}_t of one direction for i <= LA, j <= JB, t <= T into tab[((i (JB + 1) + j) (T + 1) + t)][lane]:
+// E_0 by its two-term recursion, E_t = h/t (i E^{i-1,j}_{t-1} + j E^{i,j-1}_{t-1}), h = 1/(2p)
+template <int LA, int JB, int T>
+__device__ __forceinline__ void hermite_table(double (*tab)[32], int lane, double xa, double xb, double h)
+{
+    auto at = [](int i, int j, int t) { return (i * (JB + 1) + j) * (T + 1) + t; };
+    for (int i = 0; i <= LA; ++i)
+        for (int j = 0; j <= JB; ++j) {
+            double e = 1.0;
+            if (j > 0) e = xb * tab[at(i, j - 1, 0)][lane] + (T > 0 ? tab[at(i, j - 1, T > 0 ? 1 : 0)][lane] : 0.0);
+            else if (i > 0) e = xa * tab[at(i - 1, 0, 0)][lane] + (T > 0 ? tab[at(i - 1, 0, T > 0 ? 1 : 0)][lane] : 0.0);
+            tab[at(i, j, 0)][lane] = e;
+            for (int t = 1; t <= T; ++t) {
+                double s = 0.0;
+                if (i > 0) s += i * tab[at(i - 1, j, t - 1)][lane];
+                if (j > 0) s += j * tab[at(i, j - 1, t - 1)][lane];
+                tab[at(i, j, t)][lane] = h / t * s;
+            }
+        }
+}
+
+template <int LA, int LB>
+struct PairShape {
+    static constexpr int L = LA + LB, NH = nherm(L), NA = ncart(LA), NB = ncart(LB);
+    // Hermite order needed: E_1 also where L = 0 (the derivative of (s, s))
+    static constexpr int T = L > 0 ? L : 1;
+    static constexpr int NF = 3 * (LA + 1) * (LB + 1) * (T + 1);  // table doubles per lane: fold
+    static constexpr int NC = 3 * (LA + 1) * (LB + 2) * (T + 1);  // contraction (shell B up to LB + 1)
+    static constexpr int KR = NH < 28 ? NH : 28;                  // components summed over warps at a time
+    static constexpr int FS = (NF > NA * KR ? NF : NA * KR) + NH, CS = NC + NH + 3 * NA;
+};
+__device__ __forceinline__ void cart_of(int l, int k, int (&c)[3])
+{
+    int i = 0;
+    for (int x = l; x >= 0; --x)
+        for (int y = l - x; y >= 0; --y, ++i)
+            if (i == k) {
+                c[0] = x;
+                c[1] = y;
+                c[2] = l - x - y;
+            }
+}
+
+// M[k npair + i]: harmonic coefficients of pair i, in the sweep's units; the charge sums are cleared
+template <int LA, int LB>
+__global__ void __launch_bounds__(32 * ncart(LA))
+k_pair_fold(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm, double *__restrict__ pairs)
+{
+    using Sh = PairShape<LA, LB>;
+    constexpr int L = Sh::L, NH = Sh::NH, NA = Sh::NA, NB = Sh::NB, T = Sh::T, KR = Sh::KR;
+    extern __shared__ double sm[][32];
+    double(*dsum)[32] = sm + (Sh::FS - NH);
+    const int lane = threadIdx.x, ia = threadIdx.y, i = pp_begin + blockIdx.x * 32 + lane;
+    const size_t np = pp_end - pp_begin, ip = blockIdx.x * 32 + lane;
+    const PPLane pl = load_pp(bd, i, pp_end);
+    constexpr int TD = (LA + 1) * (LB + 1) * (T + 1);
+    for (int d = ia; d < 3; d += NA) {
+        const double xa = d == 0 ? pl.P[0] - pl.A[0] : d == 1 ? pl.P[1] - pl.A[1] : pl.P[2] - pl.A[2];
+        const double xb = d == 0 ? pl.P[0] - pl.B[0] : d == 1 ? pl.P[1] - pl.B[1] : pl.P[2] - pl.B[2];
+        hermite_table<LA, LB, T>(sm + d * TD, lane, xa, xb, 0.5 * pl.ip);
+    }
+    __syncthreads();
+    int a3[3] = {0, 0, 0};
+    cart_of(LA, ia, a3);
+    double D[NH];
+#pragma unroll
+    for (int k = 0; k < NH; ++k) D[k] = 0.0;
+    const double unit = HALF_SQRT_PI * sqrt(pl.ip);
+#pragma unroll 1
+    for (int ib = 0; ib < NB; ++ib) {
+        int b3[3] = {0, 0, 0};
+        cart_of(LB, ib, b3);
+        const double g = unit * pair_density(pl, bd, dm, ia, ib);
+        // E_t vanishes beyond t = i + j: bounds uniform over the warp
+        const int lx = a3[0] + b3[0], ly = a3[1] + b3[1], lz = a3[2] + b3[2];
+        double E[3][L + 1];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int t = 0; t <= L; ++t) E[d][t] = sm[d * TD + (a3[d] * (LB + 1) + b3[d]) * (T + 1) + t][lane];
+#pragma unroll
+        for (int t = 0; t <= L; ++t) {
+            if (t > lx) continue;
+            const double gx = g * E[0][t];
+#pragma unroll
+            for (int u = 0; u <= L - t; ++u) {
+                if (u > ly) continue;
+                const double gxy = gx * E[1][u];
+#pragma unroll
+                for (int v = 0; v <= L - t - u; ++v)
+                    if (v <= lz) D[hidx(t, u, v)] = fma(gxy, E[2][v], D[hidx(t, u, v)]);
+            }
+        }
+    }
+    // sum over the components of A, KR Hermite indices at a time
+#pragma unroll
+    for (int k0 = 0; k0 < NH; k0 += KR) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < KR; ++k)
+            if (k0 + k < NH) sm[ia * KR + k][lane] = D[k0 + k < NH ? k0 + k : 0];
+        __syncthreads();
+        for (int k = ia; k < KR && k0 + k < NH; k += NA) {
+            double s = 0.0;
+            for (int w = 0; w < NA; ++w) s += sm[w * KR + k][lane];
+            dsum[k0 + k][lane] = s;
+        }
+    }
+    __syncthreads();
+    if (i >= pp_end) return;
+    // change of basis: a harmonic component's entries are consecutive in the table
+    double m = 0.0;
+    for (int e = 0; e < HT.tend[L]; ++e) {
+        const HarmEntry &t = HT.t[e];
+        const int j = harm_off(L, t.k) + t.lm;
+        if (j % NA != ia) continue;
+        m += t.c * dsum[t.herm][lane];
+        if (e + 1 == HT.tend[L] || HT.t[e + 1].k != t.k || HT.t[e + 1].lm != t.lm) {
+            pairs[j * np + ip] = m;
+            m = 0.0;
+        }
+    }
+    for (int k = ia; k < NH + 3; k += NA) pairs[(NH + k) * np + ip] = 0.0;
+}
+
+// The pairs' gradients from the charge sums: d_a = sum_ab g_ab sum_tuv E'^a_tuv W_tuv with
+// E'_t = dE^{ij}_t / dX_AB = (b/p) E^{ij}_{t-1} - 2b E^{i,j+1}_t + j E^{i,j-1}_t in direction a, then
+// dE/dA = -(d + a/p se), dE/dB = d - b/p se, se = sum_C q_C e(C)
+template <int LA, int LB>
+__global__ void __launch_bounds__(32 * ncart(LA))
+k_pair_contract(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm, const double *__restrict__ pairs,
+                double *__restrict__ gqm)
+{
+    using Sh = PairShape<LA, LB>;
+    constexpr int L = Sh::L, NH = Sh::NH, NA = Sh::NA, NB = Sh::NB, T = Sh::T;
+    extern __shared__ double sm[][32];
+    double(*W)[32] = sm + Sh::NC, (*dsum)[32] = W + NH;
+    const int lane = threadIdx.x, ia = threadIdx.y, i = pp_begin + blockIdx.x * 32 + lane;
+    const size_t np = pp_end - pp_begin, ip = min(blockIdx.x * 32 + lane, (int)np - 1);
+    const PPLane pl = load_pp(bd, i, pp_end);
+    constexpr int TD = (LA + 1) * (LB + 2) * (T + 1);
+    for (int d = ia; d < 3; d += NA) {
+        const double xa = d == 0 ? pl.P[0] - pl.A[0] : d == 1 ? pl.P[1] - pl.A[1] : pl.P[2] - pl.A[2];
+        const double xb = d == 0 ? pl.P[0] - pl.B[0] : d == 1 ? pl.P[1] - pl.B[1] : pl.P[2] - pl.B[2];
+        hermite_table<LA, LB + 1, T>(sm + d * TD, lane, xa, xb, 0.5 * pl.ip);
+    }
+    // harmonic sums -> W (a warp per Hermite index at a time)
+    for (int k = ia; k < NH; k += NA) W[k][lane] = 0.0;
+    for (int e = 0; e < HT.tend[L]; ++e) {
+        const HarmEntry &t = HT.t[e];
+        if (t.herm % NA == ia) W[t.herm][lane] += t.c * __ldg(pairs + (NH + harm_off(L, t.k) + t.lm) * np + ip);
+    }
+    __syncthreads();
+    int a3[3] = {0, 0, 0};
+    cart_of(LA, ia, a3);
+    double dx = 0.0, dy = 0.0, dz = 0.0;
+#pragma unroll 1
+    for (int ib = 0; ib < NB; ++ib) {
+        int b3[3] = {0, 0, 0};
+        cart_of(LB, ib, b3);
+        const double g = pair_density(pl, bd, dm, ia, ib);
+        // E_t and E'_t vanish beyond t = i + j: bounds uniform over the warp, tables read as they are
+        const int lx = a3[0] + b3[0], ly = a3[1] + b3[1], lz = a3[2] + b3[2];
+        const double(*row[3])[32];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) row[d] = sm + d * TD + (a3[d] * (LB + 2) + b3[d]) * (T + 1);
+        auto deriv = [&](int d, int t) {
+            double e = -2.0 * pl.b * row[d][T + 1 + t][lane];
+            if (b3[d] > 0) e += (double)b3[d] * row[d][t - (T + 1)][lane];
+            if (t > 0) e += pl.b * pl.ip * row[d][t - 1][lane];
+            return e;
+        };
+        double Ez[L + 1], dEz[L + 1], dEy[L + 1];
+#pragma unroll
+        for (int t = 0; t <= L; ++t) {
+            if (t <= lz) {
+                Ez[t] = row[2][t][lane];
+                dEz[t] = deriv(2, t);
+            }
+            if (t <= ly) dEy[t] = deriv(1, t);
+        }
+        double sx = 0.0, sy = 0.0, sz = 0.0;
+#pragma unroll 1
+        for (int t = 0; t <= lx; ++t) {
+            double h = 0.0, hy = 0.0, hz = 0.0;
+#pragma unroll
+            for (int u = 0; u <= L; ++u) {
+                if (u > ly) continue;
+                double w = 0.0, wz = 0.0;
+#pragma unroll
+                for (int v = 0; v <= L - u; ++v)
+                    if (v <= lz) {
+                        const double x = W[hidx(t, u, v)][lane];
+                        w = fma(Ez[v], x, w);
+                        wz = fma(dEz[v], x, wz);
+                    }
+                const double Ey = row[1][u][lane];
+                h = fma(Ey, w, h);
+                hy = fma(dEy[u], w, hy);
+                hz = fma(Ey, wz, hz);
+            }
+            const double Ex = row[0][t][lane];
+            sx = fma(deriv(0, t), h, sx);
+            sy = fma(Ex, hy, sy);
+            sz = fma(Ex, hz, sz);
+        }
+        dx = fma(g, sx, dx);
+        dy = fma(g, sy, dy);
+        dz = fma(g, sz, dz);
+    }
+    dsum[3 * ia][lane] = dx;
+    dsum[3 * ia + 1][lane] = dy;
+    dsum[3 * ia + 2][lane] = dz;
+    __syncthreads();
+    if (ia > 0) return;
+    const double unit = HALF_SQRT_PI * sqrt(pl.ip), aop = pl.a * pl.ip, bop = pl.b * pl.ip;
+    bool take[5], head;
+    seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        double d = 0.0;
+        for (int w = 0; w < NA; ++w) d += dsum[3 * w + x][lane];
+        d *= unit;
+        const double se = pl.active ? pairs[(2 * NH + x) * np + ip] : 0.0;
+        const double gA = seg_reduce(-(d + aop * se), take), gB = seg_reduce(d - bop * se, take);
+        if (head && pl.active) {
+            atomicAdd(gqm + 3 * pl.atomA + x, gA);
+            atomicAdd(gqm + 3 * pl.atomB + x, gB);
+        }
+    }
+}
+
 template <int LA, int LB, int NT>
 __global__ void __launch_bounds__(NT, 1)
 k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, int ch_end,
-            const double *__restrict__ boys, const double *__restrict__ dm, double *__restrict__ gqm,
-            double *__restrict__ gchg, int *err)
+            const double *__restrict__ boys, double *__restrict__ pairs, double *__restrict__ gchg, int *err)
 {
     constexpr int L = LA + LB, NH = nherm(L), NG = nhgrad(L) + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -69,19 +311,12 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
     const int ntile = (pp_end - pp_begin + 31) >> 5;
     for (int tile = blockIdx.x * nwarp + warp; tile < ntile; tile += gridDim.x * nwarp) {
         const PPLane pl = load_pp(bd, pp_begin + tile * 32 + lane, pp_end);
-        const double aop = pl.a * pl.ip, bop = pl.b * pl.ip;
-        // the density-folded Hermite coefficients as harmonic ones, their gradients, and the charge
-        // sums S (harm.cuh); unit: the unit of the harmonic factors
-        const double unit = HALF_SQRT_PI * sqrt(pl.ip);
+        // the density-folded coefficients (k_pair_fold), their gradients, and the charge sums S
+        const size_t np = pp_end - pp_begin, ip = min(tile * 32 + lane, (int)np - 1);
         double M[NH], Nx[NG], Ny[NG], Nz[NG], S[NH];
-        {
-            double D0[NH];
-            fold_density<LA, LB>(pl, bd, dm, D0);
 #pragma unroll
-            for (int k = 0; k < NH; ++k) D0[k] *= unit;
-            harm_fold<L>(D0, M);
-            harm_grad<L>(M, Nx, Ny, Nz);
-        }
+        for (int k = 0; k < NH; ++k) M[k] = pl.active ? pairs[k * np + ip] : 0.0;
+        harm_grad<L>(M, Nx, Ny, Nz);
 #pragma unroll
         for (int k = 0; k < NH; ++k) S[k] = 0.0;
 
@@ -135,27 +370,12 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
                 }
             }
         }
-        double sd[3];
-        {
-            double W[NH];
-            harm_unfold<L>(S, W);
+        if (pl.active) {
 #pragma unroll
-            for (int k = 0; k < NH; ++k) W[k] *= unit;
-            contract_dA<LA, LB>(pl, bd, dm, W, sd);
-        }
-        // dE/dA = -(sd + a/p se), dE/dB = sd - b/p se
-        double g[6] = {-(sd[0] + aop * sex), -(sd[1] + aop * sey), -(sd[2] + aop * sez),
-                       sd[0] - bop * sex, sd[1] - bop * sey, sd[2] - bop * sez};
-        bool take[5], head;
-        seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) g[k] = seg_reduce(g[k], take);
-        if (head && pl.active) {
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                atomicAdd(gqm + 3 * pl.atomA + x, g[x]);
-                atomicAdd(gqm + 3 * pl.atomB + x, g[3 + x]);
-            }
+            for (int k = 0; k < NH; ++k) atomicAdd(pairs + (NH + k) * np + ip, S[k]);
+            atomicAdd(pairs + 2 * NH * np + ip, sex);
+            atomicAdd(pairs + (2 * NH + 1) * np + ip, sey);
+            atomicAdd(pairs + (2 * NH + 2) * np + ip, sez);
         }
     }
     __syncthreads();
@@ -167,8 +387,8 @@ k_vgrad_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, i
 
 template <int LA, int LB, int NT>
 static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                             int ch_end, const double *boys, const double *dm, double *gqm, double *gchg, int *err,
-                             int nblk, int threads, int nslice, cudaStream_t st)
+                             int ch_end, const double *boys, double *pairs, double *gchg, int *err, int nblk,
+                             int threads, int nslice, cudaStream_t st)
 {
     const int nper = (ch_end - ch_begin + nslice - 1) / nslice;  // charges per slice
     const size_t smem = std::max((size_t)nper * (sizeof(double4_32a) + 4 * sizeof(double)), SWEEP_SMEM_MIN);
@@ -179,25 +399,45 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
         if (e != cudaSuccess) return e;
         attr = true;
     }
-        k_vgrad_f64<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
-                                                                  dm, gqm, gchg, err);
+    k_vgrad_f64<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
+                                                                       pairs, gchg, err);
     return cudaGetLastError();
 }
 
 template <int LA, int LB>
 cudaError_t VgradF64<LA, LB>::run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
                                   int ch_end, const double *boys, const double *dm, double *gqm, double *gchg,
-                                  int *err,
-                                  int nblk, int threads, int nslice,
-                                  cudaStream_t st)
+                                  int *err, int nblk, int threads, int nslice, double *pairs, cudaStream_t st)
 {
+    using Sh = PairShape<LA, LB>;
+    constexpr size_t row = 32 * sizeof(double);
+    static bool attr = false;
+    cudaError_t e;
+    if (!attr) {
+        if ((e = cudaFuncSetAttribute(k_pair_fold<LA, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(Sh::FS * row))) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(k_pair_contract<LA, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(Sh::CS * row))) != cudaSuccess)
+            return e;
+        attr = true;
+    }
+    const int tiles = (pp_end - pp_begin + 31) / 32;
+    k_pair_fold<LA, LB><<<tiles, dim3(32, Sh::NA), Sh::FS * row, st>>>(bd, pp_begin, pp_end, dm, pairs);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     constexpr int W = sweep_wide_threads(SW_VGRAD_F64, class_of(LA, LB));
+    bool wide = false;
     if constexpr (W > 0)
-        if (threads == W)
-            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nblk, threads,
-                                        nslice, st);
-    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nblk, threads,
-                                  nslice, st);
+        if (threads == W) {
+            wide = true;
+            e = launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, pairs, gchg, err, nblk, threads,
+                                     nslice, st);
+        }
+    if (!wide)
+        e = launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, pairs, gchg, err, nblk, threads,
+                                   nslice, st);
+    if (e != cudaSuccess) return e;
+    k_pair_contract<LA, LB><<<tiles, dim3(32, Sh::NA), Sh::CS * row, st>>>(bd, pp_begin, pp_end, dm, pairs, gqm);
+    return cudaGetLastError();
 }
 
 template struct VgradF64<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_CLASS)>;
@@ -206,10 +446,11 @@ template struct VgradF64<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_C
 
 cudaError_t launch_vgrad_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                              int ch_begin, int ch_end, const double *boys, const double *dm, double *gqm,
-                             double *gchg, int *err, int nblk, int threads, int nslice, cudaStream_t st)
+                             double *gchg, int *err, int nblk, int threads, int nslice, double *pairs, cudaStream_t st)
 {
     if (pp_end <= pp_begin || ch_end <= ch_begin) return cudaSuccess;
-    return dispatch_class<VgradF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nblk, threads, nslice, st);
+    return dispatch_class<VgradF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, dm, gqm, gchg, err, nblk,
+                                    threads, nslice, pairs, st);
 }
 
 #endif
