@@ -274,9 +274,10 @@ k_moments(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm, 
             }
             if constexpr (FOCK) {
                 const double v = seg_reduce(-0.5 * coef * f, take);
-                if (head && active) {
+                // a shell with itself: one triangle and its mirror, so that F is symmetric bit for bit
+                if (head && active && (mirror || ia <= ib)) {
                     atomicAdd(F + r * bd.nao + c, v);
-                    if (mirror) atomicAdd(F + c * bd.nao + r, v);
+                    if (mirror || ia < ib) atomicAdd(F + c * bd.nao + r, v);
                 }
             }
             if constexpr (PULAY) {
