@@ -39,17 +39,24 @@ __device__ __forceinline__ int region1_images(const EwaldDev &e, int i, Fn f)
     const double n0z = -rint((z - e.centre[2]) / e.box[2]);
     const int mx = (int)ceil(e.rcut / e.box[0]), my = (int)ceil(e.rcut / e.box[1]), mz = (int)ceil(e.rcut / e.box[2]);
     int cnt = 0;
-    for (int a = -mx; a <= mx; ++a)
-        for (int b = -my; b <= my; ++b)
+    // a component beyond the radius by itself rules an image out (the full test's sum is no smaller):
+    // of the 27 images the distance is formed for one or two
+    const double rc2 = e.rcut * e.rcut;
+    for (int a = -mx; a <= mx; ++a) {
+        const double px = x + (n0x + a) * e.box[0], dx = px - e.centre[0];
+        if (dx * dx >= rc2) continue;
+        for (int b = -my; b <= my; ++b) {
+            const double py = y + (n0y + b) * e.box[1], dy = py - e.centre[1];
+            if (dy * dy >= rc2) continue;
             for (int c = -mz; c <= mz; ++c) {
-                const double px = x + (n0x + a) * e.box[0];
-                const double py = y + (n0y + b) * e.box[1];
                 const double pz = z + (n0z + c) * e.box[2];
                 if (in_region1(e, px, py, pz)) {
                     f(px, py, pz, cnt);
                     ++cnt;
                 }
             }
+        }
+    }
     return cnt;
 }
 
@@ -241,18 +248,47 @@ __global__ void k_filter_prep(EwaldDev e, float4 *mmf, float4 *qmf)
 // QM-site potential: real space (psi_SR and the T-hat correction of Eq. 10)
 // grid (nslice, natm); partial[(j*nslice + slice)*20 + c]
 // ---------------------------------------------------------------------------------------------
-// The charges of a slice are scanned 256 at a time with the FP32 filter; the survivors are
-// compacted into a shared queue in charge order (warp ballots and a block scan, so the order and
-// hence the sums are the same on every run) and evaluated in FP64 by all threads once 256 have
-// gathered, so the FP64 pipe runs full warps instead of one or two lanes of each.
-constexpr int PR_Q = 512;
+// The charges of a slice are scanned 1024 at a time (four per thread) with the FP32 filter; the
+// survivors are compacted into a shared queue in charge order (warp ballots and a block scan, so the
+// order and hence the sums are the same on every run) and evaluated in FP64 by all threads once 256
+// have gathered, so the FP64 pipe runs full warps instead of one or two lanes of each.
+constexpr int PR_S = 4, PR_Q = 256 + PR_S * 256;
+
+// Compact the candidates cand[s] (item base + s 256 + thread) behind the `count` entries of the
+// queue, in item order; every thread of the block of 256 calls it; returns the new count.  wcnt:
+// shared scratch.  The caller synchronises before the queue is read.
+template <int S>
+__device__ __forceinline__ int queue_candidates(const bool (&cand)[S], int base, int count, int *queue, int (*wcnt)[8])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned bal[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        bal[s] = __ballot_sync(FULL, cand[s]);
+        if (lane == 0) wcnt[s][warp] = __popc(bal[s]);
+    }
+    __syncthreads();
+    // lane l of every warp holds the count of group l (in item order) and scans it
+    const int mine = lane < 8 * S ? wcnt[lane >> 3][lane & 7] : 0;
+    int sum = mine;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        const int o = __shfl_up_sync(FULL, sum, k);
+        if (lane >= k) sum += o;
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        const int off = count + __shfl_sync(FULL, sum - mine, 8 * s + warp) + __popc(bal[s] & ((1u << lane) - 1u));
+        if (cand[s]) queue[off] = base + s * 256 + threadIdx.x;
+    }
+    return count + __shfl_sync(FULL, sum, 31);
+}
 __global__ void __launch_bounds__(256) k_phi_real(EwaldDev e, double *partial)
 {
     __shared__ double scratch[8 * 20];
     __shared__ int queue[PR_Q];
-    __shared__ int wcnt[8];
+    __shared__ int wcnt[PR_S][8];
     const int j = blockIdx.y, nslice = gridDim.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double Rx = e.qm_xyz[3 * j], Ry = e.qm_xyz[3 * j + 1], Rz = e.qm_xyz[3 * j + 2];
     const float4 aj = e.qm_filt[j];
     const double rc2 = e.ewald_rc * e.ewald_rc;
@@ -262,22 +298,16 @@ __global__ void __launch_bounds__(256) k_phi_real(EwaldDev e, double *partial)
     for (int k = 0; k < 20; ++k) acc[k] = 0.0;
     double T[20];
     int count = 0;  // block-uniform
-    for (int base = i0; base < i1; base += 256) {
-        const int i = base + threadIdx.x;
-        bool cand = false;
-        if (i < i1) cand = !far_min_image_f(e, aj, __ldg(e.mm_filt + i));
-        const unsigned bal = __ballot_sync(0xffffffffu, cand);
-        if (lane == 0) wcnt[warp] = __popc(bal);
-        __syncthreads();
-        int off = count, tot = 0;
-        for (int w = 0; w < 8; ++w) {
-            if (w < warp) off += wcnt[w];
-            tot += wcnt[w];
+    for (int base = i0; base < i1; base += PR_S * 256) {
+        bool cand[PR_S];
+#pragma unroll
+        for (int s = 0; s < PR_S; ++s) {
+            const int i = base + s * 256 + threadIdx.x;
+            cand[s] = i < i1 && !far_min_image_f(e, aj, __ldg(e.mm_filt + i));
         }
-        if (cand) queue[off + __popc(bal & ((1u << lane) - 1u))] = i;
-        count += tot;
+        count = queue_candidates<PR_S>(cand, base, count, queue, wcnt);
         __syncthreads();
-        if (count < 256 && base + 256 < i1) continue;
+        if (count < 256 && base + PR_S * 256 < i1) continue;
         // FP64 evaluation of the queued charges, entry q by thread q mod 256
         for (int qi = threadIdx.x; qi < count; qi += 256) {
             const int ic = queue[qi];
@@ -884,90 +914,106 @@ __device__ __forceinline__ void mmq_reduce(double (&red)[4][MMQ_WARPS][MMQ_CH], 
             for (int v = 0; v < 4; ++v) out[v] += red[v][w][lane];
 }
 
-// Blocks of 32 MM charges.  The (charge, QM atom) pairs of a block are scanned 256 at a time with
+// Potential of the multipoles M at displacement (x, y, z) under a radial function (f, g1, g2, g3 as
+// radial_tensor) and its gradient, contracted before any tensor is formed:
+//   Q f + (mu.x) g1 + 1/2 (tr theta g1 + x.theta.x g2)
+__device__ __forceinline__ void multipole_field(const double *M, double x, double y, double z, double f, double g1,
+                                                double g2, double g3, double s, double &pot, double (&fld)[3])
+{
+    const double tx = M[4] * x + M[5] * y + M[6] * z, ty = M[5] * x + M[7] * y + M[8] * z,
+                 tz = M[6] * x + M[8] * y + M[9] * z;
+    const double mu = M[1] * x + M[2] * y + M[3] * z, tr = 0.5 * (M[4] + M[7] + M[9]), xx = 0.5 * (tx * x + ty * y + tz * z);
+    pot += s * (M[0] * f + (mu + tr) * g1 + xx * g2);
+    const double w = s * (M[0] * g1 + (mu + tr) * g2 + xx * g3), h1 = s * g1, h2 = s * g2;
+    fld[0] += w * x + h1 * M[1] + h2 * tx;
+    fld[1] += w * y + h1 * M[2] + h2 * ty;
+    fld[2] += w * z + h1 * M[3] + h2 * tz;
+}
+
+// Blocks of 32 MM charges.  The (charge, QM atom) pairs of a block are scanned 1024 at a time with
 // the FP32 filter and the survivors compacted in pair order (charge-major) into a shared queue;
-// all threads then evaluate the queued pairs in FP64, and each charge's owner thread adds its
-// pairs' contributions in queue order (the same order on every run).
-constexpr int MR_Q = 1024;
+// all threads then evaluate the queued pairs in FP64, and a lane per charge adds its pairs'
+// contributions, which are consecutive, in queue order (the same order on every run).  The kernel
+// is bound by latency, a few near pairs per charge: scanning the queue for each charge's entries
+// took most of its time (150-atom site 1.21 -> 0.63 ms, 60 atoms 0.50 -> 0.21 ms).
+constexpr int MR_S = 4, MR_Q = 2048;
 __global__ void __launch_bounds__(256) k_mm_real(EwaldDev e, const double *mult, double *dq, double *dR)
 {
     __shared__ int queue[MR_Q];
-    __shared__ double contrib[MR_Q][4];
-    __shared__ int wcnt[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double contrib[4][MR_Q / 2];
+    __shared__ int wcnt[MR_S][8], nof[MMQ_CH];
     const int c0 = blockIdx.x * MMQ_CH, nch = min(MMQ_CH, e.nmm - c0), natm = e.natm;
     const int npairs = nch * natm;
     const double rc2 = e.ewald_rc * e.ewald_rc;
     double sum[4] = {0.0, 0.0, 0.0, 0.0};  // charge threadIdx.x (< nch)
-    double T[20];
     int count = 0;  // block-uniform
-    for (int base = 0; base < npairs; base += 256) {
-        const int t = base + threadIdx.x;
-        bool cand = false;
-        if (t < npairs) {
-            const int il = t / natm, j = t - il * natm;
-            cand = !far_min_image_f(e, __ldg(e.qm_filt + j), __ldg(e.mm_filt + c0 + il));
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, cand);
-        if (lane == 0) wcnt[warp] = __popc(bal);
-        __syncthreads();
-        int off = count, tot = 0;
-        for (int w = 0; w < 8; ++w) {
-            if (w < warp) off += wcnt[w];
-            tot += wcnt[w];
-        }
-        if (cand) queue[off + __popc(bal & ((1u << lane) - 1u))] = t;
-        count += tot;
-        __syncthreads();
-        if (count <= MR_Q - 256 && base + 256 < npairs) continue;
-        for (int qi = threadIdx.x; qi < count; qi += 256) {
-            const int tq = queue[qi], il = tq / natm, j = tq - il * natm, i = c0 + il;
-            const double beta = e.mm_beta[i];
-            const double xi = e.mm_xyz[3 * i], yi = e.mm_xyz[3 * i + 1], zi = e.mm_xyz[3 * i + 2];
-            const double rhat2 = beta > 0.0 ? (9.0 / beta) * (9.0 / beta) : -1.0;
-            const double dx0 = __ldg(e.qm_xyz + 3 * j) - xi, dy0 = __ldg(e.qm_xyz + 3 * j + 1) - yi,
-                         dz0 = __ldg(e.qm_xyz + 3 * j + 2) - zi;
-            const double nx0 = rint(dx0 / e.box[0]), ny0 = rint(dy0 / e.box[1]), nz0 = rint(dz0 / e.box[2]);
-            double pot = 0.0, fld[3] = {0.0, 0.0, 0.0};
-            for (int a = -e.img[0]; a <= e.img[0]; ++a)
-                for (int b = -e.img[1]; b <= e.img[1]; ++b)
-                    for (int c = -e.img[2]; c <= e.img[2]; ++c) {
-                        const double sx = (nx0 + a) * e.box[0], sy = (ny0 + b) * e.box[1], sz = (nz0 + c) * e.box[2];
-                        const double x = dx0 - sx, y = dy0 - sy, z = dz0 - sz;
-                        const double r2 = x * x + y * y + z * z;
-                        const bool sr = r2 < rc2;
-                        const bool hat = r2 < rhat2 && !in_region1(e, xi + sx, yi + sy, zi + sz);
-                        if (!sr && !hat) continue;
-                        double Mj[10];
+    for (int base = 0; base < npairs; base += MR_S * 256) {
+        bool cand[MR_S];
 #pragma unroll
-                        for (int k = 0; k < 10; ++k) Mj[k] = __ldg(mult + 10 * j + k);
-                        double f, g1, g2, g3, p, fl[3];
-                        if (sr) {
-                            screened_radial(r2, e.alpha, f, g1, g2, g3);
-                            radial_tensor(f, g1, g2, g3, x, y, z, T, 3);
-                            contract_pot_field(Mj, T, p, fl);
-                            pot += p; fld[0] += fl[0]; fld[1] += fl[1]; fld[2] += fl[2];
-                        }
-                        if (hat) {
-                            screened_radial(r2, beta, f, g1, g2, g3);
-                            radial_tensor(f, g1, g2, g3, x, y, z, T, 3);
-                            contract_pot_field(Mj, T, p, fl);
-                            pot -= p; fld[0] -= fl[0]; fld[1] -= fl[1]; fld[2] -= fl[2];
-                        }
-                    }
-            contrib[qi][0] = pot;
-            contrib[qi][1] = fld[0];
-            contrib[qi][2] = fld[1];
-            contrib[qi][3] = fld[2];
+        for (int s = 0; s < MR_S; ++s) {
+            const int t = base + s * 256 + threadIdx.x, il = t / natm;
+            cand[s] = t < npairs && !far_min_image_f(e, __ldg(e.qm_filt + t - il * natm), __ldg(e.mm_filt + c0 + il));
         }
+        count = queue_candidates<MR_S>(cand, base, count, queue, wcnt);
         __syncthreads();
-        if (threadIdx.x < nch)
-            for (int qi = 0; qi < count; ++qi)
-                if (queue[qi] / natm == (int)threadIdx.x)
+        if (count <= MR_Q - MR_S * 256 && base + MR_S * 256 < npairs) continue;
+        for (int q0 = 0; q0 < count; q0 += MR_Q / 2) {  // as many pairs at a time as results fit
+            const int q1 = min(count, q0 + MR_Q / 2);
+            if (threadIdx.x < MMQ_CH) nof[threadIdx.x] = 0;
+            __syncthreads();
+            for (int qi = q0 + threadIdx.x; qi < q1; qi += 256) {
+                const int tq = queue[qi], il = tq / natm, j = tq - il * natm, i = c0 + il;
+                atomicAdd(nof + il, 1);
+                const double beta = e.mm_beta[i];
+                const double xi = e.mm_xyz[3 * i], yi = e.mm_xyz[3 * i + 1], zi = e.mm_xyz[3 * i + 2];
+                const double rhat2 = beta > 0.0 ? (9.0 / beta) * (9.0 / beta) : -1.0;
+                const double dx0 = __ldg(e.qm_xyz + 3 * j) - xi, dy0 = __ldg(e.qm_xyz + 3 * j + 1) - yi,
+                             dz0 = __ldg(e.qm_xyz + 3 * j + 2) - zi;
+                const double nx0 = rint(dx0 / e.box[0]), ny0 = rint(dy0 / e.box[1]), nz0 = rint(dz0 / e.box[2]);
+                double pot = 0.0, fld[3] = {0.0, 0.0, 0.0};
+                for (int a = -e.img[0]; a <= e.img[0]; ++a)
+                    for (int b = -e.img[1]; b <= e.img[1]; ++b)
+                        for (int c = -e.img[2]; c <= e.img[2]; ++c) {
+                            const double sx = (nx0 + a) * e.box[0], sy = (ny0 + b) * e.box[1], sz = (nz0 + c) * e.box[2];
+                            const double x = dx0 - sx, y = dy0 - sy, z = dz0 - sz;
+                            const double r2 = x * x + y * y + z * z;
+                            const bool sr = r2 < rc2;
+                            const bool hat = r2 < rhat2 && !in_region1(e, xi + sx, yi + sy, zi + sz);
+                            if (!sr && !hat) continue;
+                            double Mj[10];
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) sum[v] += contrib[qi][v];
+                            for (int k = 0; k < 10; ++k) Mj[k] = __ldg(mult + 10 * j + k);
+                            double f, g1, g2, g3;
+                            if (sr) {
+                                screened_radial(r2, e.alpha, f, g1, g2, g3);
+                                multipole_field(Mj, x, y, z, f, g1, g2, g3, 1.0, pot, fld);
+                            }
+                            if (hat) {
+                                screened_radial(r2, beta, f, g1, g2, g3);
+                                multipole_field(Mj, x, y, z, f, g1, g2, g3, -1.0, pot, fld);
+                            }
+                        }
+                contrib[0][qi - q0] = pot;
+                contrib[1][qi - q0] = fld[0];
+                contrib[2][qi - q0] = fld[1];
+                contrib[3][qi - q0] = fld[2];
+            }
+            __syncthreads();
+            if (threadIdx.x < MMQ_CH) {
+                const int n = nof[threadIdx.x];
+                int end = n;
+#pragma unroll
+                for (int k = 1; k < 32; k <<= 1) {
+                    const int o = __shfl_up_sync(FULL, end, k);
+                    if ((int)threadIdx.x >= k) end += o;
+                }
+                for (int k = end - n; k < end; ++k)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) sum[v] += contrib[v][k];
+            }
+            __syncthreads();
+        }
         count = 0;
-        __syncthreads();
     }
     if (threadIdx.x < nch) {
         const int i = c0 + threadIdx.x;
@@ -990,17 +1036,15 @@ __global__ void __launch_bounds__(MMQ_CH *MMQ_WARPS) k_mm_region1(EwaldDev e, co
     double4_32a c;
     c.x = c.y = c.z = c.w = 0.0;
     if (act) c = rI[k];
-    double pot = 0.0, fld[3] = {0.0, 0.0, 0.0}, T[20];
+    double pot = 0.0, fld[3] = {0.0, 0.0, 0.0};
     for (int j = warp; act && j < e.natm; j += MMQ_WARPS) {
         const double x = __ldg(e.qm_xyz + 3 * j) - c.x, y = __ldg(e.qm_xyz + 3 * j + 1) - c.y,
                      z = __ldg(e.qm_xyz + 3 * j + 2) - c.z;
-        double f, g1, g2, g3, p, fl[3], Mj[10];
+        double f, g1, g2, g3, Mj[10];
 #pragma unroll
         for (int m = 0; m < 10; ++m) Mj[m] = __ldg(mult + 10 * j + m);
         point_radial(x * x + y * y + z * z, f, g1, g2, g3);
-        radial_tensor(f, g1, g2, g3, x, y, z, T, 3);
-        contract_pot_field(Mj, T, p, fl);
-        pot += p; fld[0] += fl[0]; fld[1] += fl[1]; fld[2] += fl[2];
+        multipole_field(Mj, x, y, z, f, g1, g2, g3, 1.0, pot, fld);
     }
     double t[4];
     mmq_reduce(red, pot, fld, t);
@@ -1559,42 +1603,78 @@ __constant__ double c_mult3[10] = {1, 3, 3, 3, 6, 3, 1, 3, 3, 1};  // multiplici
 
 // bins[k], k < nbin - 1: images with r_lo + k dr <= d < r_lo + (k + 1) dr;  bins[nbin - 1]: images
 // with r_min <= d < r_lo;  bins[nbin]: images with r_min <= d < rc.  e.rcut must be r_max.
-__global__ void __launch_bounds__(256) k_oct_shell(EwaldDev e, const double *oct, double r_min, double r_lo,
-                                                   double dr, int nbin, double rc, double *bins)
+// Block: 32 charges (lanes) x 8 warps, warp w taking the atoms j = w, w + 8, ..; the octupole term of
+// an atom is 1/2 g2 (t.x) + 1/6 g3 Omega(x, x, x) with the trace vector t_a = sum_b Omega_abb, without
+// forming the tensor.  A thread per charge over all atoms was one long chain in mostly idle warps
+// (60 atoms, 60 000 charges: 0.46 -> 0.12 ms).
+constexpr int OS_CH = 32, OS_WARPS = 8;
+__global__ void __launch_bounds__(OS_CH *OS_WARPS) k_oct_shell(EwaldDev e, const double *oct, double r_min, double r_lo,
+                                                              double dr, int nbin, double rc, double *bins)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= e.nmm) return;
-    const double q = e.mm_q[i], beta = e.mm_beta[i];
-    const double rhat2 = beta > 0.0 ? (9.0 / beta) * (9.0 / beta) : -1.0;
-    region1_images(e, i, [&](double px, double py, double pz, int) {
+    __shared__ double part[OS_WARPS][OS_CH], pos[3][OS_CH];
+    __shared__ int images[OS_CH], most;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * OS_CH + lane;
+    const bool act = i < e.nmm;
+    const double beta = act ? e.mm_beta[i] : 0.0, rhat2 = beta > 0.0 ? (9.0 / beta) * (9.0 / beta) : -1.0;
+    if (warp == 0) {
+        const int n = act ? region1_images(e, i, [](double, double, double, int) {}) : 0;
+        images[lane] = n;
+        const int m = __reduce_max_sync(FULL, n);
+        if (lane == 0) most = m;
+    }
+    __syncthreads();
+    const int nimg = images[lane];
+    for (int k = 0; k < most; ++k) {  // the k-th image of every lane
+        if (warp == 0 && k < nimg)
+            region1_images(e, i, [&](double x, double y, double z, int n) {
+                if (n == k) {
+                    pos[0][lane] = x;
+                    pos[1][lane] = y;
+                    pos[2][lane] = z;
+                }
+            });
+        __syncthreads();
+        const double px = pos[0][lane], py = pos[1][lane], pz = pos[2][lane];
         const double cx = px - e.centre[0], cy = py - e.centre[1], cz = pz - e.centre[2];
         const double d = sqrt(cx * cx + cy * cy + cz * cz);
-        if (d < r_min) return;
-        double ei = 0.0, T[20], Th[20];
-        for (int j = 0; j < e.natm; ++j) {
+        const bool use = k < nimg && d >= r_min;
+        double ei = 0.0;
+        for (int j = warp; use && j < e.natm; j += OS_WARPS) {
             const double x = __ldg(e.qm_xyz + 3 * j) - px, y = __ldg(e.qm_xyz + 3 * j + 1) - py,
                          z = __ldg(e.qm_xyz + 3 * j + 2) - pz;
             const double r2 = x * x + y * y + z * z;
             double f, g1, g2, g3;
             point_radial(r2, f, g1, g2, g3);
-            radial_tensor(f, g1, g2, g3, x, y, z, T, 3);
             if (r2 < rhat2) {
-                screened_radial(r2, beta, f, g1, g2, g3);
-                radial_tensor(f, g1, g2, g3, x, y, z, Th, 3);
-#pragma unroll
-                for (int c = 10; c < 20; ++c) T[c] -= Th[c];
+                double h1, h2, h3;
+                screened_radial(r2, beta, f, h1, h2, h3);
+                g2 -= h2;
+                g3 -= h3;
             }
+            double o[10];
 #pragma unroll
-            for (int c = 0; c < 10; ++c) ei += c_mult3[c] * __ldg(oct + 10 * j + c) * T[10 + c];
+            for (int c = 0; c < 10; ++c) o[c] = __ldg(oct + 10 * j + c);
+            const double t = (o[0] + o[3] + o[5]) * x + (o[1] + o[6] + o[8]) * y + (o[2] + o[7] + o[9]) * z;
+            const double cube = x * (x * (o[0] * x + 3.0 * (o[1] * y + o[2] * z)) + 6.0 * o[4] * y * z +
+                                     3.0 * (o[3] * y * y + o[5] * z * z)) +
+                                y * y * (o[6] * y + 3.0 * o[7] * z) + z * z * (3.0 * o[8] * y + o[9] * z);
+            ei += 0.5 * g2 * t + (1.0 / 6.0) * g3 * cube;
         }
-        ei *= q;
-        if (d < r_lo) atomicAdd(bins + nbin - 1, ei);
-        else {
-            const int k = (int)floor((d - r_lo) / dr);
-            if (k < nbin - 1) atomicAdd(bins + k, ei);
+        part[warp][lane] = ei;
+        __syncthreads();
+        if (warp == 0 && use) {
+            double s = 0.0;
+            for (int w = 0; w < OS_WARPS; ++w) s += part[w][lane];
+            s *= e.mm_q[i];
+            if (d < r_lo) atomicAdd(bins + nbin - 1, s);
+            else {
+                const int b = (int)floor((d - r_lo) / dr);
+                if (b < nbin - 1) atomicAdd(bins + b, s);
+            }
+            if (d < rc) atomicAdd(bins + nbin, s);
         }
-        if (d < rc) atomicAdd(bins + nbin, ei);
-    });
+        __syncthreads();
+    }
 }
 
 // E0 = sum_j Omega_j : v_j(rc) and err[k] = E0 + F(rc) - F(R_k); one block
@@ -1628,7 +1708,7 @@ cudaError_t launch_octupole_error(const EwaldDev &e0, const double *oct, const d
     cudaError_t err_ = cudaMemsetAsync(bins, 0, (n + 1) * sizeof(double), st);
     if (err_ != cudaSuccess) return err_;
     if (e.nmm > 0) {
-        k_oct_shell<<<(e.nmm + 255) / 256, 256, 0, st>>>(e, oct, r_min, r_lo, dr, n, rc, bins);
+        k_oct_shell<<<(e.nmm + OS_CH - 1) / OS_CH, OS_CH * OS_WARPS, 0, st>>>(e, oct, r_min, r_lo, dr, n, rc, bins);
         if ((err_ = cudaGetLastError()) != cudaSuccess) return err_;
     }
     k_oct_finish<<<1, 256, 0, st>>>(oct, phi, e.natm, bins, n, err);
