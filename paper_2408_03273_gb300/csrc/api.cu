@@ -218,7 +218,7 @@ struct qmmm_handle {
     DBuf<double> cl_psum;
     size_t cl_rec_off[NCLASS] = {}, cl_psum_off[NCLASS] = {};
     DBuf<double> pair_ws;  // FP64 adjoint: per-pair density coefficients and charge sums, per class
-    size_t pair_off[NCLASS] = {};
+    size_t pair_off[NCLASS] = {}, vpair_off[NCLASS] = {};  // (the FP64 V sweep shares it: sums per slice)
 
     BasisDev basis() const
     {
@@ -679,10 +679,10 @@ constexpr int MAX_SLICES = 16;
 
 // Per-pair work of a sweep outside its charge loop, in charges of loop work: the Hermite and
 // density algebra, FP64 in both precisions (against an FP32 charge loop on the mixed path).
-double setup_charges(int L, int kind)
+double setup_charges(int kind)
 {
     if (kind_is_mixed(kind)) return 64.0;
-    return kind_is_grad(kind) ? 3.0 : 3.0 + 0.6 * L * L;  // (the adjoint's pair algebra has kernels of its own)
+    return 3.0;  // (the FP64 sweeps' pair algebra has kernels of its own)
 }
 
 // How the classes of a sweep over nch charges are cut into blocks: charge slices per class, launch
@@ -699,10 +699,11 @@ Cut cut_classes(const qmmm_handle *h, int kind, int nch)
     for (int c = 0; c < NCLASS; ++c) {
         tiles[c] = (h->class_off[c + 1] - h->class_off[c] + 31) / 32;
         w[c] = std::max(h->cls_cost[kind][c], 1e-30);
-        setup[c] = setup_charges(la_of_class(c) + lb_of_class(c), kind);
+        setup[c] = setup_charges(kind);
     }
     const size_t n2 = (size_t)h->nao * h->nao;
-    fine_slices(NCLASS, tiles, w, setup, nch, h->nsm, kind_is_grad(kind) ? MAX_SLICES : vpot_slice_cap(n2, MAX_SLICES),
+    // the mixed V sweep writes a partial V per slice
+    fine_slices(NCLASS, tiles, w, setup, nch, h->nsm, kind == SW_VPOT_F32 ? vpot_slice_cap(n2, MAX_SLICES) : MAX_SLICES,
                 k.ns);
     slice_order(NCLASS, tiles, w, k.ns, k.order);
     long long warps = 0;
@@ -807,6 +808,18 @@ int ensure_pairs(qmmm_handle *h)
     return h->pair_ws.ensure(std::max<size_t>(n, 1));
 }
 
+// The same buffer for the FP64 V sweep over nch charges: per class and charge slice the pairs' sums.
+int ensure_vpairs(qmmm_handle *h, int nch)
+{
+    const Cut k = cut_classes(h, SW_VPOT_F64, nch);
+    size_t n = 0;
+    for (int c = 0; c < NCLASS; ++c) {
+        h->vpair_off[c] = n;
+        n += (size_t)(h->class_off[c + 1] - h->class_off[c]) * nherm(la_of_class(c) + lb_of_class(c)) * k.ns[c];
+    }
+    return h->pair_ws.ensure(std::max<size_t>(n, 1));
+}
+
 // One class sweep of the given kind over region-I charges [c0, c1): nblk blocks of `threads` threads
 // in each of nslice block rows (the mixed adjoint: its variant in place of `threads`); V kernels
 // write slice s into V + s * vstride.
@@ -818,8 +831,8 @@ cudaError_t launch_sweep(const qmmm_handle *h, int kind, int cls, int p0, int p1
     const RegionDev r = h->region();
     switch (kind) {
     case SW_VPOT_F64:
-        return launch_vpot_f64(b, r, cls, p0, p1, c0, c1, h->boys64.p, V, h->err.p, nblk, threads, nslice, vstride,
-                               cs);
+        return launch_vpot_f64(b, r, cls, p0, p1, c0, c1, h->boys64.p, V, h->err.p, nblk, threads, nslice,
+                               h->pair_ws.p + h->vpair_off[cls], cs);
     case SW_VPOT_F32:
         return launch_vpot_f32(b, r, cls, p0, p1, c0, c1, h->boys32.p, V, h->err.p, nblk, threads, nslice, vstride,
                                cs);
@@ -867,6 +880,10 @@ int time_best(qmmm_handle *h, cudaEvent_t e0, cudaEvent_t e1, F run, float *ms)
 int tune_launch(qmmm_handle *h, int kind, int cls, int share, int variant)
 {
     const int c1 = std::min(h->nI, std::min(chunk_for_kind(kind), TUNE_CHARGES));
+    if (kind == SW_VPOT_F64) {
+        const int rc = ensure_vpairs(h, c1);
+        if (rc) return rc;
+    }
     auto one = [&](int c, int p0, int p1, int nblk, int threads, int ns, cudaStream_t cs) {
         return launch_sweep(h, kind, c, p0, p1, 0, c1, nblk, threads, ns, 0, h->tune_dm.p, h->tune_V.p, h->tune_gqm.p,
                             h->tune_gchg.p, cs);
@@ -1322,6 +1339,7 @@ static int ensure_vslices(qmmm_handle *h, int *nbuf)
 {
     const int kind = sweep_kind(h, false), ch = chunk_for_kind(kind);
     *nbuf = 1;
+    if (kind == SW_VPOT_F64) return QMMM_OK;  // slices of sums instead (ensure_vpairs)
     for (int c0 = 0; c0 < h->nI; c0 += ch) *nbuf = std::max(*nbuf, cut_classes(h, kind, std::min(ch, h->nI - c0)).most);
     return *nbuf > 1 ? h->Vslices.ensure((size_t)*nbuf * h->nao * h->nao) : QMMM_OK;
 }
@@ -1356,6 +1374,7 @@ static int vpot_sweep(qmmm_handle *h, double *Vdst, int nbuf)
     const size_t n2 = (size_t)h->nao * h->nao;
     for (int c0 = 0; c0 < h->nI; c0 += ch) {
         const int c1 = std::min(h->nI, c0 + ch);
+        if (kind == SW_VPOT_F64 && (rc = ensure_vpairs(h, c1 - c0))) return rc;
         rc = run_classes(
             h, kind,
             [&](int cls, int p0, int p1, int nblk, int threads, int nsl, cudaStream_t cs) {
@@ -1844,6 +1863,10 @@ std::vector<long long> batch_key(const qmmm_batch *b, const double *const *dm, d
                 k.push_back(bits);
                 k.push_back(h->cls_variant[kind][c]);
             }
+        // scratch whose size follows the charge slices: a plain call under another sweep configuration
+        // may have moved it
+        k.push_back(ptr(h->pair_ws.p));
+        k.push_back(ptr(h->Vslices.p));
         k.push_back(ptr(dm[i]));
         k.push_back(ptr(V ? V[i] : nullptr));
         k.push_back(ptr(E ? E[i] : nullptr));
@@ -2099,7 +2122,10 @@ int qmmm_batch_run(qmmm_batch *b, const double *const *dm, double *const *V, dou
         for (int i = 0; i < n && !rc; ++i)
             if (!batch_defers(b->f[i])) {
                 int nbuf;
-                if ((rc = ensure_pairs(b->f[i])) || (rc = ensure_vslices(b->f[i], &nbuf))) break;
+                qmmm_handle *h = b->f[i];
+                if ((rc = ensure_pairs(h)) || (rc = ensure_vslices(h, &nbuf)) ||
+                    (rc = ensure_vpairs(h, std::min(h->nI, chunk_for_kind(SW_VPOT_F64)))))
+                    break;
             }
         if (!rc && !deferred.empty()) rc = batch_build_jobs(b, dm);
         if (rc) {
@@ -2191,7 +2217,7 @@ int qmmm_batch_run(qmmm_batch *b, const double *const *dm, double *const *V, dou
             ++b->instantiations;
         }
         cudaGraphDestroy(graph);
-        b->key = key;
+        b->key = batch_key(b, dm, V, E, dE_dRqm, dE_dRmm, dE_dq);  // (the plain pass sized the scratch)
         ++b->captures;
     }
     CUDA_TRY(cudaGraphLaunch(b->exec, b->stream));

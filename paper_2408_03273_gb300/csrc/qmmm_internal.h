@@ -47,14 +47,15 @@ struct qmmm_handle_impl;
 // launchers (defined in the .cu files); all return a cudaError_t of the last launch
 // Region-I sweeps.  A launch has `nblk` blocks of `threads` threads per charge slice (at most 256, or
 // the class's wide block, sweep_wide_threads, where one exists); its warps take the class's tiles in
-// turn.  `nslice` splits the charge chunk over that many block rows, the V kernels then writing
-// slice s into V + s * vstride.  The mixed adjoint (launch_vgrad_f32) sizes its own grid; `variant`
+// turn.  `nslice` splits the charge chunk over that many block rows, the mixed V kernels then writing
+// slice s into V + s * vstride (FP64: slices of the pairs' sums, added before the contraction).  The mixed adjoint (launch_vgrad_f32) sizes its own grid; `variant`
 // picks its charges per lane (cl_variant).
 // dst[k] = sum_s src[s*n + k], s < nslice, in order (the V slices)
 cudaError_t launch_sum_slices_d(const double *src, int nslice, size_t n, double *dst, cudaStream_t st);
+// sums: scratch of the class, nslice x the Hermite sums of every primitive pair
 cudaError_t launch_vpot_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                             int ch_begin, int ch_end, const double *boys, double *V, int *err, int nblk, int threads,
-                            int nslice, size_t vstride, cudaStream_t st);
+                            int nslice, double *sums, cudaStream_t st);
 cudaError_t launch_vpot_f32(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                             int ch_begin, int ch_end, const float *boys, double *V, int *err, int nblk, int threads,
                             int nslice, size_t vstride, cudaStream_t st);

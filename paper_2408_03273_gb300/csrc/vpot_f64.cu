@@ -11,13 +11,20 @@
 // (s,s), 38 (d,s), 106 (d,d) on a 60-atom active site.  V sweep against the Hermite recursion:
 // active site 33.5 -> 24.4 ms, a 150-atom site with f shells 147 -> 104 ms, a QM water 0.43 ->
 // 0.33 ms (untuned handles).  Charges are grouped by Gaussian width so that rho is formed once per
-// (primitive pair, width class).  The E-contraction runs once per primitive pair; primitive pairs
-// of a shell pair are summed by a segmented warp-shuffle reduction and the head lane adds the block
-// into V (and its mirror).  A shell pair spans at most two tiles when it has at most 32 primitive
-// pairs, so at most two additions reach any element: the result does not depend on scheduling.
+// (primitive pair, width class).
+//
+// The sweep leaves the sums of every pair and charge slice; k_pair_V adds the slices in a fixed order
+// and contracts them with E once per primitive pair, in blocks of 32 pairs x the components of shell
+// A (in the sweep this was one lane's chain, some 1 500 FP64 instructions for (d,d) and 6 000 for (f,f),
+// once per slice, into one partial V per slice: sweep of 17 atoms with f shells 1.18 -> 0.70 ms, of a QM
+// water 0.205 -> 0.138 ms, of the 60-atom site 19.8 -> 19.7 ms).  Primitive pairs of a
+// shell pair are summed by a segmented warp-shuffle reduction and the head lane adds the block into
+// V (and its mirror).  A shell pair spans at most two tiles when it has at most 32 primitive pairs,
+// so at most two additions reach any element: the result does not depend on scheduling.
 #include <algorithm>
 
 #include "harm.cuh"
+#include "pair_block.cuh"
 #include "pp_tile.cuh"
 
 namespace qmmm {
@@ -26,8 +33,7 @@ template <int LA, int LB>
 struct VpotF64 {
     static cudaError_t run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
                            int ch_end, const double *boys, double *V, int *err, int nblk, int threads, int nslice,
-                           size_t vstride,
-                           cudaStream_t st);
+                           double *sums, cudaStream_t st);
 };
 
 #ifdef QMMM_SPLIT_CLASS  // one angular class per compilation
@@ -35,10 +41,11 @@ struct VpotF64 {
 template <int LA, int LB, int NT>
 __global__ void __launch_bounds__(NT, 1)
 k_vpot_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, int ch_end,
-           const double *__restrict__ boys, double *__restrict__ V, size_t vstride, int *err)
+           const double *__restrict__ boys, double *__restrict__ sums, int *err)
 {
-    V += (size_t)blockIdx.y * vstride;  // per-slice partial V when the charges are split
-    constexpr int L = LA + LB, NH = nherm(L), NA = ncart(LA), NB = ncart(LB);
+    constexpr int L = LA + LB, NH = nherm(L);
+    const size_t np = pp_end - pp_begin;
+    sums += (size_t)blockIdx.y * NH * np;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t bar;
     double4_32a *chg = reinterpret_cast<double4_32a *>(smem_raw);
@@ -48,9 +55,8 @@ k_vpot_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, in
         ch_begin += (int)blockIdx.y * per;
         ch_end = min(ch_end, ch_begin + per);
     }
-    if (ch_begin >= ch_end) return;
-    const int nch = ch_end - ch_begin;
-    if (!stage_to_smem(chg, rg.chg + ch_begin, (unsigned)(nch * sizeof(double4_32a)), &bar, err)) return;
+    const int nch = max(ch_end - ch_begin, 0);  // (an empty last slice leaves zero sums)
+    if (nch > 0 && !stage_to_smem(chg, rg.chg + ch_begin, (unsigned)(nch * sizeof(double4_32a)), &bar, err)) return;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int ntile = (pp_end - pp_begin + 31) >> 5;
@@ -82,48 +88,87 @@ k_vpot_f64(BasisDev bd, RegionDev rg, int pp_begin, int pp_end, int ch_begin, in
                 }
             }
         }
-        double W[NH];
-        harm_unfold<L>(S, W);
+        if (pl.active)
+#pragma unroll
+            for (int k = 0; k < NH; ++k) sums[k * np + tile * 32 + lane] = S[k];
+    }
+}
 
-        double Ex[LA + 1][LB + 1][L + 1], Ey[LA + 1][LB + 1][L + 1], Ez[LA + 1][LB + 1][L + 1];
-        hermite_E<LA, LB, double>(Ex, pl.P[0] - pl.A[0], pl.P[0] - pl.B[0], 0.5 * pl.ip);
-        hermite_E<LA, LB, double>(Ey, pl.P[1] - pl.A[1], pl.P[1] - pl.B[1], 0.5 * pl.ip);
-        hermite_E<LA, LB, double>(Ez, pl.P[2] - pl.A[2], pl.P[2] - pl.B[2], 0.5 * pl.ip);
-        const double coef = -TWO_PI * pl.ip * pl.cab * HALF_SQRT_PI * sqrt(pl.ip);
-
-        bool take[5], head;
-        seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-        const bool mirror = pl.sp.shA != pl.sp.shB;
+template <int LA, int LB>
+__global__ void __launch_bounds__(32 * ncart(LA))
+k_pair_V(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ sums, int nslice, double *__restrict__ V)
+{
+    using Sh = PairShape<LA, LB>;
+    constexpr int L = Sh::L, NH = Sh::NH, NA = Sh::NA, NB = Sh::NB, T = Sh::T;
+    extern __shared__ double sm[][32];
+    double(*S)[32] = sm + Sh::NF, (*W)[32] = S + NH;
+    const int lane = threadIdx.x, ia = threadIdx.y, i = pp_begin + blockIdx.x * 32 + lane;
+    const size_t np = pp_end - pp_begin, ip = min(blockIdx.x * 32 + lane, (int)np - 1);
+    const PPLane pl = load_pp(bd, i, pp_end);
+    constexpr int TD = (LA + 1) * (LB + 1) * (T + 1);
+    for (int d = ia; d < 3; d += NA) {
+        const double xa = d == 0 ? pl.P[0] - pl.A[0] : d == 1 ? pl.P[1] - pl.A[1] : pl.P[2] - pl.A[2];
+        const double xb = d == 0 ? pl.P[0] - pl.B[0] : d == 1 ? pl.P[1] - pl.B[1] : pl.P[2] - pl.B[2];
+        hermite_table<LA, LB, T>(sm + d * TD, lane, xa, xb, 0.5 * pl.ip);
+    }
+    for (int k = ia; k < NH; k += NA) {
+        double s = 0.0;
+        for (int sl = 0; sl < nslice; ++sl) s += sums[((size_t)sl * NH + k) * np + ip];
+        S[k][lane] = s;
+        W[k][lane] = 0.0;
+    }
+    __syncthreads();
+    // harmonic sums -> Hermite sums, a warp per Hermite index at a time
+    for (int e = 0; e < HT.tend[L]; ++e) {
+        const HarmEntry &t = HT.t[e];
+        if (t.herm % NA == ia) W[t.herm][lane] += t.c * S[harm_off(L, t.k) + t.lm][lane];
+    }
+    __syncthreads();
+    int a3[3] = {0, 0, 0};
+    cart_of(LA, ia, a3);
+    const double coef = -TWO_PI * pl.ip * pl.cab * HALF_SQRT_PI * sqrt(pl.ip);
+    bool take[5], head;
+    seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
+    const bool mirror = pl.sp.shA != pl.sp.shB;
+#pragma unroll 1
+    for (int ib = 0; ib < NB; ++ib) {
+        int b3[3] = {0, 0, 0};
+        cart_of(LB, ib, b3);
+        // E_t vanishes beyond t = i + j: bounds uniform over the warp
+        const int lx = a3[0] + b3[0], ly = a3[1] + b3[1], lz = a3[2] + b3[2];
+        const double(*row[3])[32];
 #pragma unroll
-        for (int ia = 0; ia < NA; ++ia) {
+        for (int d = 0; d < 3; ++d) row[d] = sm + d * TD + (a3[d] * (LB + 1) + b3[d]) * (T + 1);
+        double Ez[L + 1], v = 0.0;
 #pragma unroll
-            for (int ib = 0; ib < NB; ++ib) {
-                const int ax = cart_lx(LA, ia), ay = cart_ly(LA, ia), az = cart_lz(LA, ia);
-                const int bx = cart_lx(LB, ib), by = cart_ly(LB, ib), bz = cart_lz(LB, ib);
-                double v = 0.0;
+        for (int t = 0; t <= L; ++t) Ez[t] = t <= lz ? row[2][t][lane] : 0.0;
+#pragma unroll 1
+        for (int t = 0; t <= lx; ++t) {
+            double h = 0.0;
+#pragma unroll 1
+            for (int u = 0; u <= ly; ++u) {
+                double w = 0.0;
 #pragma unroll
-                for (int t = 0; t <= ax + bx; ++t)
-#pragma unroll
-                    for (int u = 0; u <= ay + by; ++u) {
-                        const double exy = Ex[ax][bx][t] * Ey[ay][by][u];
-#pragma unroll
-                        for (int w = 0; w <= az + bz; ++w) v += exy * Ez[az][bz][w] * W[hidx(t, u, w)];
-                    }
-                v = seg_reduce(coef * v, take);
-                if (head && pl.active) {
-                    const size_t r = pl.sp.aoA + ia, c = pl.sp.aoB + ib;
-                    atomicAdd(V + r * bd.nao + c, v);
-                    if (mirror) atomicAdd(V + c * bd.nao + r, v);
-                }
+                for (int z = 0; z <= L; ++z)
+                    if (z <= lz) w = fma(Ez[z], W[hidx(t, u, z)][lane], w);
+                h = fma(row[1][u][lane], w, h);
             }
+            v = fma(row[0][t][lane], h, v);
+        }
+        v = seg_reduce(coef * v, take);
+        // a shell with itself: one triangle and its mirror, so that V is symmetric bit for bit
+        if (head && pl.active && (mirror || ia <= ib)) {
+            const size_t r = pl.sp.aoA + ia, c = pl.sp.aoB + ib;
+            atomicAdd(V + r * bd.nao + c, v);
+            if (mirror || ia < ib) atomicAdd(V + c * bd.nao + r, v);
         }
     }
 }
 
 template <int LA, int LB, int NT>
 static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
-                             int ch_end, const double *boys, double *V, int *err, int nblk, int threads, int nslice,
-                             size_t vstride, cudaStream_t st)
+                             int ch_end, const double *boys, double *sums, int *err, int nblk, int threads, int nslice,
+                             cudaStream_t st)
 {
     const int per = (ch_end - ch_begin + nslice - 1) / nslice;
     const size_t smem = std::max((size_t)per * sizeof(double4_32a), SWEEP_SMEM_MIN);
@@ -135,22 +180,40 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
         attr = true;
     }
         k_vpot_f64<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
-                                                                 V, vstride, err);
+                                                                      sums, err);
     return cudaGetLastError();
 }
 
 template <int LA, int LB>
 cudaError_t VpotF64<LA, LB>::run(const BasisDev &bd, const RegionDev &rg, int pp_begin, int pp_end, int ch_begin,
                                  int ch_end, const double *boys, double *V, int *err, int nblk, int threads,
-                                 int nslice, size_t vstride,
-                                 cudaStream_t st)
+                                 int nslice, double *sums, cudaStream_t st)
 {
+    using Sh = PairShape<LA, LB>;
+    constexpr size_t smem = Sh::VS * 32 * sizeof(double);
+    static bool attr = false;
+    cudaError_t e;
+    if (!attr) {
+        if ((e = cudaFuncSetAttribute(k_pair_V<LA, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+            cudaSuccess)
+            return e;
+        attr = true;
+    }
     constexpr int W = sweep_wide_threads(SW_VPOT_F64, class_of(LA, LB));
+    bool wide = false;
     if constexpr (W > 0)
-        if (threads == W)
-            return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice,
-                                        vstride, st);
-    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice, vstride, st);
+        if (threads == W) {
+            wide = true;
+            e = launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, sums, err, nblk, threads, nslice,
+                                     st);
+        }
+    if (!wide)
+        e = launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, sums, err, nblk, threads, nslice,
+                                   st);
+    if (e != cudaSuccess) return e;
+    k_pair_V<LA, LB><<<(pp_end - pp_begin + 31) / 32, dim3(32, Sh::NA), smem, st>>>(bd, pp_begin, pp_end, sums, nslice,
+                                                                                    V);
+    return cudaGetLastError();
 }
 
 template struct VpotF64<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_CLASS)>;
@@ -159,12 +222,11 @@ template struct VpotF64<la_of_class(QMMM_SPLIT_CLASS), lb_of_class(QMMM_SPLIT_CL
 
 cudaError_t launch_vpot_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                             int ch_begin, int ch_end, const double *boys, double *V, int *err, int nblk,
-                            int threads, int nslice, size_t vstride,
-                            cudaStream_t st)
+                            int threads, int nslice, double *sums, cudaStream_t st)
 {
     if (pp_end <= pp_begin || ch_end <= ch_begin) return cudaSuccess;
-    return dispatch_class<VpotF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads,
-                                   nslice, vstride, st);
+    return dispatch_class<VpotF64>(cls, b, r, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice,
+                                   sums, st);
 }
 
 #endif
