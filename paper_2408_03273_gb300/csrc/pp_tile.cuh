@@ -140,6 +140,7 @@ __host__ __device__ constexpr int cl_rec_floats(int L) { return 8 + 4 * nherm(L)
 // primitive pairs per staged batch (two batches of records in shared memory: <= 22 KB)
 __host__ __device__ constexpr int cl_batch(int L) { return L <= 4 ? 16 : 8; }
 constexpr int CL_BPB = 8;  // batches per block
+constexpr int CL_MIN_ITEMS = 152;  // items a single small system's class is spread over (VgradF32::run)
 // Charge-lane variants: (charges per lane, blocks per SM) for variant v of class order L; 0 where
 // the class has no such variant.  Charges per lane amortise the per-pair warp reduction and give
 // each lane independent chains; the register budget (65536 / (256 x blocks per SM)) bounds them.
@@ -224,10 +225,9 @@ __host__ __device__ constexpr int sweep_wide_threads(int kind, int cls)
 }
 
 // Dynamic shared memory of every FP64 sweep block is at least this much: more than half of an
-// SM's 228 KB, so no two FP64 sweep blocks share an SM.  The concurrent class sweeps split the
-// SMs in shares, one block per SM; with a region I small enough for two charge chunks to fit in
-// one SM, the block scheduler would otherwise stack blocks of different classes on some SMs
-// (which then share one saturated FP64 pipe) while others stay idle.  The FP32 sweeps are
+// SM's 228 KB, so no two FP64 sweep blocks share an SM: where the blocks are fewer than the SMs can
+// hold, the block scheduler would otherwise stack blocks of different classes on some SMs (which
+// then share one saturated FP64 pipe) while others stay idle.  The FP32 sweeps are
 // latency-bound instead and gain from a second block on an SM, so they are not padded.
 constexpr size_t SWEEP_SMEM_MIN = 116 * 1024;
 
