@@ -48,19 +48,26 @@ def comb(n, k):
 
 
 def flops_forward(L):
-    """Algorithmic FLOPs per (primitive pair, charge) of the V sweep: Boys 25+3L, R recursion
+    """Algorithmic FLOPs per (primitive pair, charge) of the mixed V sweep: Boys 25+3L, R recursion
     2 C(L+4,4), Hermite accumulation 2 C(L+3,3), setup 15."""
     return 25 + 3 * L + 2 * comb(L + 4, 4) + 2 * comb(L + 3, 3) + 15
 
 
 def flops_adjoint(L):
-    """Per (primitive pair, charge) of the adjoint sweep: Boys to L+1 (28+3L), R recursion to L+1
-    2 C(L+5,4), the four density contractions (e_0, e_x, e_y, e_z) and the charge sum
+    """Per (primitive pair, charge) of the mixed adjoint sweep: Boys to L+1 (28+3L), R recursion to
+    L+1 2 C(L+5,4), the four density contractions (e_0, e_x, e_y, e_z) and the charge sum
     S += q R over the C(L+3,3) Hermite terms 10 C(L+3,3), setup/accumulation/reduction 47.  The
     centre-A derivative coefficients meet S once per pair, not per charge, so they are not
-    counted per term (the FP64 kernels of the f-shell classes with L >= 5 contract them per
-    charge instead: 4 C(L+3,3) more than counted here)."""
+    counted per term."""
     return 28 + 3 * L + 2 * comb(L + 5, 4) + 10 * comb(L + 3, 3) + 47
+
+
+def flops_fp64(L, adjoint):
+    """The same for the FP64 sweeps, which work in solid harmonics: (L+1)^2 harmonics with one radial
+    factor per l, and per harmonic a multiply-add for the charge sum (the adjoint: the value, the charge
+    sum and the gradient).  Two FLOPs per executed FP64 instruction, by a fit to their counts:
+    10 + 3.1 (L+1)^2 for V, 23 + 7.1 (L+1)^2 for the adjoint."""
+    return 2 * (23 + 7.1 * (L + 1) ** 2 if adjoint else 10 + 3.1 * (L + 1) ** 2)
 
 
 CLASS_L = [la + lb for la in range(4) for lb in range(la + 1)]  # class index la(la+1)/2 + lb
@@ -69,11 +76,13 @@ CLASS_L = [la + lb for la in range(4) for lb in range(la + 1)]  # class index la
 # path's pair records and pair gradients included), per (workload, precision), from one ncu
 # capture of the current kernels (dram__bytes_read.sum + dram__bytes_write.sum); a workload or
 # precision without a capture of the current kernels reports None.
-SWEEP_TRAFFIC = {("c4", "fp64"): 153_470_720, ("c4", "mixed"): 364_729_600}
+SWEEP_TRAFFIC = {("c4", "mixed"): 364_729_600}
 
 
-def sweep_flops(info, adjoint):
-    f = flops_adjoint if adjoint else flops_forward
+def sweep_flops(info, adjoint, fp64):
+    def f(L):
+        return flops_fp64(L, adjoint) if fp64 else (flops_adjoint if adjoint else flops_forward)(L)
+
     return sum(n * info["n_region1"] * f(CLASS_L[c]) for c, n in enumerate(info["n_prim_pairs_class"]))
 
 
@@ -548,7 +557,7 @@ def main():
     # dominant kernel (region-I sweep) against the plain-ALU roofline
     t_v, t_g = float(np.mean(rec["vpot"])), float(np.mean(rec["grad"]))
     dom_adj = t_g >= t_v
-    fl = sweep_flops(info, dom_adj)
+    fl = sweep_flops(info, dom_adj, prec == q.QMMM_FP64)
     achieved = fl / ((t_g if dom_adj else t_v) * 1e-3) / 1e12
     peak = FP64_PEAK_TFLOPS if prec == q.QMMM_FP64 else FP32_PEAK_TFLOPS
     roof = {"kernel": "vgrad (region-I adjoint sweep)" if dom_adj else "vpot (region-I sweep)",
@@ -565,23 +574,23 @@ def main():
     #   set_positions: gather, region-I count/scan/fill, real-space pre-filter inputs, real-space,
     #     region-I tensors, background sum, QM-site reciprocal, final = 10 (mixed path: + the
     #     double-float g(G) S(G) table),
-    #     plus the structure factor (tensor cores: max|q|, phases, B planes, MMA, reduction = 5;
+    #     plus the structure factor (tensor cores: max|q|, phases, B planes, MMA, reduction, combination = 6;
     #     CUDA cores: kernel + slice sum = 2)
-    #   vpot: one kernel per class and charge chunk + nuclear-MM term and its sum
+    #   vpot: one kernel per class and charge chunk (FP64: and the contraction of its pair sums) +
+    #     nuclear-MM term and its sum
     #   ewald: one moments kernel per class + the energy terms
-    #   forces: two moments kernels per class (Pulay) + the adjoint sweep per class and chunk
-    #     (mixed path: pair records, charge-lane sweep, pair gradients = 3 per class and chunk)
+    #   forces: one moments kernel per class (Pulay) + the adjoint per class and chunk: density fold (mixed
+    #     path: pair records), sweep, pair gradients = 3
     #     + 8 fixed (nuclear-MM, sum, real space, region I, background, tensor
     #     gradient, scatter, unpermute) + the MM-side reciprocal sum (tensor cores: atom phases,
     #     multipole structure factor, phases, scales, B planes per N tile, MMA = 5 + tiles; CUDA
     #     cores: 3)
-    # vpot adds one V slice-sum kernel when its classes split their charges (per-class slices:
-    # 256 or more region-I charges and room for two partial matrices in 512 MB; or small systems
-    # whose classes ask for less than half the SMs, which have fewer charges than that here).
+    # The mixed vpot adds one V slice-sum kernel when its classes split their charges (128 or more
+    # region-I charges and room for two partial matrices in 512 MB).
     def launches_per_step(precision):
         ncls = sum(1 for n in info["n_prim_pairs_class"] if n > 0)
         nI = info["n_region1"]
-        v_maxsl = min(8, min(nI, 4096) // 128, (512 << 20) // max(1, 8 * s.nao * s.nao))
+        v_maxsl = min(min(nI, 4096) // 64, (512 << 20) // max(1, 8 * s.nao * s.nao))
         ch_f = math.ceil(nI / 4096) if nI else 0
         ch_g = math.ceil(nI / 2560) if nI else 0
         tensor = recip_in_effect(precision).startswith("tensor cores")
@@ -592,10 +601,10 @@ def main():
         cpt = next((c for c in (3, 2, 1) if 2 * c * kx <= lim), 1)
         mm_tc = tensor and (2 * cpt * kx + 15) // 16 * 16 <= lim and 2 * s.kmax[2] + 1 >= 8
         mm_tiles = -(-3 // cpt)
-        sweep_g = ncls * ch_g * (3 if precision == q.QMMM_MIXED else 1)
         mixed = precision == q.QMMM_MIXED
-        return (10 + (1 if mixed else 0) + (5 if tensor else 2)) + (ncls * ch_f + 2 + (1 if v_maxsl > 1 else 0)) + (ncls + 1) + \
-            (2 * ncls + sweep_g + 8 + ((5 + mm_tiles) if mm_tc else 3))
+        vpot = ncls * ch_f + (1 if v_maxsl > 1 else 0) if mixed else 2 * ncls * ch_f
+        return (10 + (1 if mixed else 0) + (6 if tensor else 2)) + (vpot + 2) + (ncls + 1) + \
+            (ncls + 3 * ncls * ch_g + 8 + ((5 + mm_tiles) if mm_tc else 3))
 
     per_step = launches_per_step(prec)
     launches = per_step * args.steps
@@ -619,7 +628,7 @@ def main():
         gerr = max(raw.values())
         escale = float(E64[1].abs() + E64[2].abs() + E64[3].abs())
         t_vm, t_gm = float(np.mean(rec_m["vpot"])), float(np.mean(rec_m["grad"]))
-        flm = sweep_flops(info, t_gm >= t_vm)
+        flm = sweep_flops(info, t_gm >= t_vm, False)
         ach_m = flm / (max(t_gm, t_vm) * 1e-3) / 1e12
         ms_m = max_over_ranks(ms_m, dist, dev)
         mixed = {"value": job_rate(world, units_per_step, ms_m), "ms_per_step": ms_m,

@@ -238,13 +238,13 @@ int qmmm_rcut_search(qmmm_handle *h, const double *dm, double r_lo, double dr, i
 
 /* Autotuner (the paper has no counterpart: its integrals come from a library).  The region-I
  * sweeps run one kernel per angular class (l_A, l_B), all classes at once on their own streams,
- * each with a cap on its grid -- its share of the SMs -- and a block shape.  By default the
- * shares follow a flop model of each class's work and every class uses 256-thread blocks.
+ * each cut into blocks (charge slices, launch order) by the classes' costs, with a block shape.  By
+ * default the costs follow a model of each class's work and every class uses 256-thread blocks
+ * (128 on systems too small to fill the SMs).
  * qmmm_autotune times each class kernel alone on this handle's geometry, in each block shape
  * it has (256 threads, or a wider block where registers allow: more pair tiles per CTA on the
- * same staged charges), keeps the faster shape, sets each class's share in proportion to its
- * measured SM-time so that the classes finish together, and keeps the tuned configuration only
- * if the concurrent sweep is faster than the untuned one.
+ * same staged charges), keeps the faster shape, takes its measured SM-time as its cost, and keeps
+ * the tuned configuration only if the concurrent sweep is faster than the untuned one.
  *   flags: QMMM_TUNE_V and/or QMMM_TUNE_FORCES select the V and adjoint sweeps (0 = both);
  *   QMMM_TUNE_BOTH_PRECISIONS tunes the FP64 and the mixed kernels, else the current precision.
  * Needs a geometry (qmmm_create / qmmm_set_positions).  It works in scratch buffers with a zero
@@ -257,10 +257,10 @@ int qmmm_autotune(qmmm_handle *h, int flags);
 
 /* The sweep configuration in use for one kernel kind (0 V FP64, 1 V mixed, 2 adjoint FP64,
  * 3 adjoint mixed), per angular class in the order (0,0) (1,0) (1,1) (2,0) (2,1) (2,2) (3,0)
- * (3,1) (3,2) (3,3): threads[10] per block, share[10] = grid cap (SMs; 0 for an empty class),
+ * (3,1) (3,2) (3,3): threads[10] per block, share[10] = its part of the SMs by cost (0 for an empty class),
  * ms[10] = the class's measured time alone at that share (0 if not measured), wide[10] = the
  * class's wide block size (0: it has only 256-thread blocks), weight[10] = the SM-time per
- * primitive pair that sets the shares (ms x blocks / pairs when tuned, the flop model if not;
+ * primitive pair, its cost (ms x blocks / pairs when tuned, the work model if not;
  * qmmm_set_tuning accepts it back, e.g. to share one frame's tuning with similar frames).  Any
  * array may be NULL.  Returns 1 if the kind was tuned, 0 if it runs the model configuration, <0
  * on error. */
@@ -269,8 +269,8 @@ int qmmm_get_tuning(const qmmm_handle *h, int kind, int *threads, int *share, do
 
 /* Install a sweep configuration (e.g. one saved from qmmm_get_tuning on an earlier run of the
  * same system): threads[10] per class must be 256 or that class's wide block size (the values
- * qmmm_get_tuning can report); weight[10] (NULL = the flop model) is each class's SM-time per
- * primitive pair, in any common unit, from which the SM shares follow.  QMMM_ERR_ARG if a block
+ * qmmm_get_tuning can report); weight[10] (NULL = the work model) is each class's SM-time per
+ * primitive pair, in any common unit, from which the cut into blocks follows.  QMMM_ERR_ARG if a block
  * size is not available for its class or a weight is not positive. */
 int qmmm_set_tuning(qmmm_handle *h, int kind, const int *threads, const double *weight);
 

@@ -646,7 +646,8 @@ int tile_cap(const qmmm_handle *h, int kind, int cls, int variant)
     return std::max(1, ((npp + 31) / 32 + nwarp - 1) / nwarp);
 }
 
-// Grid caps of the concurrent class sweeps: shares of the SMs in proportion to each class's
+// Grid caps of the class kernels that the autotuner times alone, and the shares that qmmm_get_tuning
+// reports: shares of the SMs in proportion to each class's
 // SM-time (primitive pairs x cost), but never more blocks than the class has warps' worth of
 // 32-pair tiles for (times maxsl, when a class may split its charges over maxsl block rows);
 // what a capped class cannot use goes to the others.  Returns false when no class has work.
