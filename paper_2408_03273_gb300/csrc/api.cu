@@ -735,8 +735,6 @@ int run_classes(qmmm_handle *h, int kind, F launch, int nch = 0, bool join = tru
     if (h->n_pp == 0) return QMMM_OK;
     const bool cl = kind == SW_VGRAD_F32;
     const Cut k = cut_classes(h, kind, nch);
-    int share[NCLASS];
-    split_sms(h, kind, h->cls_variant[kind], share);
     CUDA_TRY(cudaEventRecord(h->fork, h->stream));
     for (int i = 0; i < NCLASS; ++i) {
         const int c = cl ? NCLASS - 1 - i : k.order[i];
@@ -744,8 +742,8 @@ int run_classes(qmmm_handle *h, int kind, F launch, int nch = 0, bool join = tru
         if (p1 <= p0) continue;
         CUDA_TRY(cudaStreamWaitEvent(h->side[c], h->fork, 0));
         const int nwarp = k.threads[c] / 32, blocks = ((p1 - p0 + 31) / 32 + nwarp - 1) / nwarp;
-        CUDA_TRY(launch(c, p0, p1, cl ? share[c] : blocks, cl ? h->cls_variant[kind][c] : k.threads[c], cl ? 1 : k.ns[c],
-                        h->side[c]));
+        CUDA_TRY(launch(c, p0, p1, cl ? h->nsm : blocks, cl ? h->cls_variant[kind][c] : k.threads[c],
+                        cl ? 1 : k.ns[c], h->side[c]));
         CUDA_TRY(cudaEventRecord(h->join[c], h->side[c]));
     }
     if (join)
@@ -822,7 +820,8 @@ int ensure_vpairs(qmmm_handle *h, int nch)
 }
 
 // One class sweep of the given kind over region-I charges [c0, c1): nblk blocks of `threads` threads
-// in each of nslice block rows (the mixed adjoint: its variant in place of `threads`); V kernels
+// in each of nslice block rows (the mixed adjoint: the SM count in place of nblk, its variant in place of
+// `threads`); V kernels
 // write slice s into V + s * vstride.
 cudaError_t launch_sweep(const qmmm_handle *h, int kind, int cls, int p0, int p1, int c0, int c1, int nblk,
                          int threads, int nslice, size_t vstride, const double *ddm, double *V, double *gqm,
@@ -893,8 +892,9 @@ int tune_launch(qmmm_handle *h, int kind, int cls, int share, int variant)
         // the slices of the real sweep (V slices all add into the one scratch matrix here)
         return run_classes(h, kind, one, c1);
     }
-    CUDA_TRY(one(cls, h->class_off[cls], h->class_off[cls + 1], share,
-                 kind == SW_VGRAD_F32 ? variant : variant_threads(kind, cls, variant), 1, h->stream));
+    const bool cl = kind == SW_VGRAD_F32;
+    CUDA_TRY(one(cls, h->class_off[cls], h->class_off[cls + 1], cl ? h->nsm : share,
+                 cl ? variant : variant_threads(kind, cls, variant), 1, h->stream));
     return QMMM_OK;
 }
 

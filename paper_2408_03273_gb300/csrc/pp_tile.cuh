@@ -140,7 +140,6 @@ __host__ __device__ constexpr int cl_rec_floats(int L) { return 8 + 4 * nherm(L)
 // primitive pairs per staged batch (two batches of records in shared memory: <= 22 KB)
 __host__ __device__ constexpr int cl_batch(int L) { return L <= 4 ? 16 : 8; }
 constexpr int CL_BPB = 8;  // batches per block
-constexpr int CL_MIN_ITEMS = 152;  // items a single small system's class is spread over (VgradF32::run)
 // Charge-lane variants: (charges per lane, blocks per SM) for variant v of class order L; 0 where
 // the class has no such variant.  Charges per lane amortise the per-pair warp reduction and give
 // each lane independent chains; the register budget (65536 / (256 x blocks per SM)) bounds them.

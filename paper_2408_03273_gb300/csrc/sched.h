@@ -78,6 +78,17 @@ inline void block_threads(int n, const int *tiles, const int *ns, int nsm, const
     for (int c = 0; c < n; ++c) threads[c] = asked[c] > 0 ? asked[c] : warps <= 4LL * nsm ? 128 : 256;
 }
 
+// Ranges of pair batches of one class of the mixed adjoint (charge lanes), whose items are gx ranges times
+// ntile charge tiles.  A small system's class has a few charge tiles, and ranges of several batches
+// would leave it with a handful of blocks, each a long serial chain: its batches are spread over nsm
+// items instead, down to one batch each.  From nsm items on, several batches to a block save more
+// atomics and staging than more blocks gain.
+inline int spread_ranges(int gx, int ntile, int nbatch, int nsm)
+{
+    if (ntile <= 0 || (long long)gx * ntile >= nsm) return gx;
+    return std::max(gx, std::min(nbatch, nsm / ntile));
+}
+
 // Class indices in order of falling block time w / ns (empty classes last).
 inline void slice_order(int n, const int *tiles, const double *w, const int *ns, int *order)
 {

@@ -6,6 +6,7 @@
 // double-float registers, per-pair sums go through a warp reduce-scatter, compensated FP32
 // shared-memory atomics and one FP64 global atomic per block (see the comment above k_vgrad_cl).
 #include "pp_tile.cuh"
+#include "sched.h"
 
 namespace qmmm {
 
@@ -807,16 +808,10 @@ cudaError_t VgradF32<LA, LB>::run(const BasisDev &bd, const RegionDev &rg, int p
     one.ch_end = ch_end;
     constexpr int L = LA + LB;
     cl_decompose(L, variant, pp_end - pp_begin, ch_end - ch_begin, rg.ncls, one.gx, one.ntile);
-    // A small system's class has a few charge tiles and CL_BPB batches to an item would leave it with
-    // a handful of blocks, each a long serial chain: its batches are spread over CL_MIN_ITEMS items
-    // instead, down to one batch each (QM water, 645 charges: the sweep 0.218 -> 0.084 ms).  The line
-    // is the SM count: from there on CL_BPB batches to a block save more atomics and staging than
-    // more blocks gain (60-atom site unchanged).  The batched launches keep cl_decompose's count:
-    // their frames fill the SMs together.
-    if (one.ntile > 0 && one.gx * one.ntile < CL_MIN_ITEMS) {
-        const int nbatch = (pp_end - pp_begin + cl_batch(L) - 1) / cl_batch(L);
-        one.gx = std::max(one.gx, std::min(nbatch, CL_MIN_ITEMS / one.ntile));
-    }
+    // small systems: spread over the SMs (QM water, 645 charges: the sweep 0.218 -> 0.084 ms; the 60-atom
+    // site is unchanged).  The batched launches keep cl_decompose's count: their frames fill the SMs
+    // together.
+    one.gx = spread_ranges(one.gx, one.ntile, (pp_end - pp_begin + cl_batch(L) - 1) / cl_batch(L), nsm);
     const int nthr = (pp_end - pp_begin + 31) / 32 * 32, nitems = one.gx * one.ntile;
     if (variant == 1) {
         if constexpr (cl_variant(L, 1, 0) > 0)
