@@ -451,8 +451,9 @@ void tc_sf_shape(const EwaldDev &e, TcShape &sh)
     const int NX = 2 * e.kmax[0] + 1, NY = 2 * e.kmax[1] + 1, NZ = 2 * e.kmax[2] + 1;
     sh.NL = NX * NY;
     sh.mtiles = (sh.NL + TCM - 1) / TCM;
-    // N tiles of at most 64 rows: two pipeline stages with their phase rows fit in shared memory
-    // up to ky = 47, and seven accumulators (448 columns) in tensor memory
+    // N tiles of at most 64 rows: seven accumulators (448 columns) fit in tensor memory, and two
+    // pipeline stages with their phase rows in shared memory up to ky = 45 (narrower N tiles: for every
+    // ky; 64 rows: kz 24..31 and from 48 on).  Beyond that the producers read the rows from global memory
     sh.ntiles = (NZ + 63) / 64;
     sh.ntr = ((NZ + sh.ntiles - 1) / sh.ntiles + 15) / 16 * 16;
     sh.nkb = (e.nmm + TCCPB - 1) / TCCPB;
