@@ -498,7 +498,7 @@ def main():
         for k in range(4):
             t = hh.tuning(k)
             if t["tuned"]:
-                tuning[q.SWEEP_KINDS[k]] = {"threads": hh.sweep_threads(k), "share": t["share"]}
+                tuning[q.SWEEP_KINDS[k]] = {"threads": t["threads"], "share": t["share"]}
 
     tune(h)
     t = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device=dev)  # noqa: E731
@@ -683,7 +683,7 @@ def main():
                       "units_per_step": units_per_step,
                       "prim_pairs_per_class": dict(zip(["ss", "ps", "pp", "ds", "dp", "dd", "fs", "fp", "fd", "ff"],
                                                        info["n_prim_pairs_class"])),
-                      "sweep_schedule": ({"work model": {q.SWEEP_KINDS[k]: {"threads": h.sweep_threads(k)} for k in range(4)}}
+                      "sweep_schedule": ("work model, 256-thread blocks"
                                          if args.no_autotune else {"autotuned": tuning})},
            "roofline": roof, "gpu_launches": launches, "clocks": clk.summary(),
            "e2e": {"value": job_rate(world, units_per_step, ms_e2e), "unit": UNIT, "ms_per_step": ms_e2e,

@@ -239,8 +239,7 @@ int qmmm_rcut_search(qmmm_handle *h, const double *dm, double r_lo, double dr, i
 /* Autotuner (the paper has no counterpart: its integrals come from a library).  The region-I
  * sweeps run one kernel per angular class (l_A, l_B), all classes at once on their own streams,
  * each cut into blocks (charge slices, launch order) by the classes' costs, with a block shape.  By
- * default the costs follow a model of each class's work and every class uses 256-thread blocks
- * (128 where the whole sweep has at most four warps per SM; qmmm_sweep_threads tells).
+ * default the costs follow a model of each class's work and every class uses 256-thread blocks.
  * qmmm_autotune times each class kernel alone on this handle's geometry, in each block shape
  * it has (256 threads, or a wider block where registers allow: more pair tiles per CTA on the
  * same staged charges), keeps the faster shape, takes its measured SM-time as its cost, and keeps
@@ -257,8 +256,7 @@ int qmmm_autotune(qmmm_handle *h, int flags);
 
 /* The sweep configuration in use for one kernel kind (0 V FP64, 1 V mixed, 2 adjoint FP64,
  * 3 adjoint mixed), per angular class in the order (0,0) (1,0) (1,1) (2,0) (2,1) (2,2) (3,0)
- * (3,1) (3,2) (3,3): threads[10] per block (256: the default shape, or that size where it came from
- * qmmm_set_tuning; qmmm_sweep_threads reports what is launched), share[10] = its part of the SMs by cost (0 for an empty class),
+ * (3,1) (3,2) (3,3): threads[10] per block, share[10] = its part of the SMs by cost (0 for an empty class),
  * ms[10] = the class's measured time alone at that share (0 if not measured), wide[10] = the
  * class's wide block size (0: it has only 256-thread blocks), weight[10] = the SM-time per
  * primitive pair, its cost (ms x blocks / pairs when tuned, the work model if not;
@@ -270,15 +268,10 @@ int qmmm_get_tuning(const qmmm_handle *h, int kind, int *threads, int *share, do
 
 /* Install a sweep configuration (e.g. one saved from qmmm_get_tuning on an earlier run of the
  * same system): threads[10] per class must be 256 or that class's wide block size (the values
- * qmmm_get_tuning can report) and is launched as given; weight[10] (NULL = the work model) is each class's SM-time per
+ * qmmm_get_tuning can report); weight[10] (NULL = the work model) is each class's SM-time per
  * primitive pair, in any common unit, from which the cut into blocks follows.  QMMM_ERR_ARG if a block
  * size is not available for its class or a weight is not positive. */
 int qmmm_set_tuning(qmmm_handle *h, int kind, const int *threads, const double *weight);
-
-/* threads[10]: the block size that the sweep of the kind launches for each class over the current
- * region I (0 for an empty class).  It differs from qmmm_get_tuning's on small systems whose shape
- * is the default one. */
-int qmmm_sweep_threads(const qmmm_handle *h, int kind, int *threads);
 
 /* ---------------------------------------------------------------------------------------------
  * Batches of independent systems (MD frames or sampling replicas of uneven sizes).  The paper

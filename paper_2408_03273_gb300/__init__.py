@@ -32,7 +32,6 @@ from ._lib import (  # noqa: F401
     qmmm_autotune,
     qmmm_get_tuning,
     qmmm_set_tuning,
-    qmmm_sweep_threads,
     library_path,
     qmmm_create,
     qmmm_destroy,

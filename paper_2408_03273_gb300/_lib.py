@@ -59,7 +59,7 @@ _L = None
 
 EXPORTS = ("qmmm_create", "qmmm_set_stream", "qmmm_set_precision", "qmmm_set_recip_method", "qmmm_set_positions", "qmmm_vpot", "qmmm_ewald",
            "qmmm_energy", "qmmm_density_gradient", "qmmm_forces", "qmmm_get_info", "qmmm_nao", "qmmm_get_potential", "qmmm_last_timing",
-           "qmmm_qm_images", "qmmm_aspc_predict", "qmmm_selftest_bounded_wait", "qmmm_octupole_error", "qmmm_rcut_search", "qmmm_autotune", "qmmm_get_tuning", "qmmm_set_tuning", "qmmm_sweep_threads", "qmmm_batch_create", "qmmm_batch_run",
+           "qmmm_qm_images", "qmmm_aspc_predict", "qmmm_selftest_bounded_wait", "qmmm_octupole_error", "qmmm_rcut_search", "qmmm_autotune", "qmmm_get_tuning", "qmmm_set_tuning", "qmmm_batch_create", "qmmm_batch_run",
            "qmmm_batch_timing", "qmmm_batch_captures", "qmmm_batch_counts", "qmmm_batch_destroy", "qmmm_destroy", "qmmm_strerror", "qmmm_last_error", "qmmm_nuclear_mm_energy_static")
 
 
@@ -103,7 +103,6 @@ def load(build_if_needed: bool = True):
         "qmmm_autotune": (c_int, [c_void_p, c_int]),
         "qmmm_get_tuning": (c_int, [c_void_p, c_int, P(c_int), P(c_int), P(c_double), P(c_int), P(c_double)]),
         "qmmm_set_tuning": (c_int, [c_void_p, c_int, P(c_int), P(c_double)]),
-        "qmmm_sweep_threads": (c_int, [c_void_p, c_int, P(c_int)]),
         "qmmm_batch_create": (c_int, [P(c_void_p), c_int, c_void_p, P(c_void_p)]),
         "qmmm_batch_run": (c_int, [c_void_p, P(c_void_p), P(c_void_p), P(c_void_p), P(c_void_p), P(c_void_p),
                                    P(c_void_p)]),
@@ -359,13 +358,6 @@ def qmmm_set_tuning(h, kind, threads, weight=None):
     th = (c_int * 10)(*[int(t) for t in threads])
     w = (c_double * 10)(*[float(x) for x in weight]) if weight is not None else None
     _check(load().qmmm_set_tuning(h, int(kind), th, w), "qmmm_set_tuning")
-
-
-def qmmm_sweep_threads(h, kind):
-    """Threads per block that the sweep of the kind launches, per angular class (0: empty class)."""
-    th = (c_int * 10)()
-    _check(load().qmmm_sweep_threads(h, int(kind), th), "qmmm_sweep_threads")
-    return list(th)
 
 
 def qmmm_batch_create(handles, stream=None):

@@ -183,7 +183,6 @@ struct qmmm_handle {
     int cls_variant[SW_NKIND][NCLASS] = {};
     double cls_ms[SW_NKIND][NCLASS] = {};
     int tuned_mask = 0, tuned_nI = 0;
-    int installed_mask = 0;  // kinds whose block sizes came from qmmm_set_tuning
     DBuf<double> tune_V, tune_dm, tune_gqm, tune_gchg;  // autotuner scratch
     DBuf<double> oct, oct_bins, oct_err;                  // octupole error estimate
     DBuf<double> qmq_ws, qmq_u, qmq_g, qmq_E, qmq_F;       // QM-QM periodic images
@@ -631,7 +630,6 @@ void reset_tuning(qmmm_handle *h, int kind)
         h->cls_ms[kind][c] = 0.0;
     }
     h->tuned_mask &= ~(1 << kind);
-    h->installed_mask &= ~(1 << kind);
 }
 
 int variant_threads(int kind, int cls, int variant)
@@ -709,14 +707,10 @@ Cut cut_classes(const qmmm_handle *h, int kind, int nch)
     fine_slices(NCLASS, tiles, w, setup, nch, h->nsm, kind == SW_VPOT_F32 ? vpot_slice_cap(n2, MAX_SLICES) : MAX_SLICES,
                 k.ns);
     slice_order(NCLASS, tiles, w, k.ns, k.order);
-    int asked[NCLASS];
     for (int c = 0; c < NCLASS; ++c) {
         k.most = std::max(k.most, k.ns[c]);
-        // a shape from qmmm_set_tuning, or a wide one that the autotuner chose, is launched as it is
-        const int v = h->cls_variant[kind][c];
-        asked[c] = v == 1 || ((h->installed_mask >> kind) & 1) ? variant_threads(kind, c, v) : 0;
+        k.threads[c] = variant_threads(kind, c, h->cls_variant[kind][c]);
     }
-    block_threads(NCLASS, tiles, k.ns, h->nsm, asked, k.threads);
     return k;
 }
 
@@ -1769,17 +1763,7 @@ int qmmm_set_tuning(qmmm_handle *h, int kind, const int *threads, const double *
         h->cls_variant[kind][c] = var[c];
         if (weight) h->cls_cost[kind][c] = weight[c];
     }
-    h->installed_mask |= 1 << kind;
     h->tuned_nI = h->nI;
-    return QMMM_OK;
-}
-
-int qmmm_sweep_threads(const qmmm_handle *h, int kind, int *threads)
-{
-    if (!h || kind < 0 || kind >= SW_NKIND || !threads) return fail(QMMM_ERR_ARG, "null argument or unknown kind");
-    const Cut k = cut_classes(h, kind, std::min(h->nI, chunk_for_kind(kind)));
-    for (int c = 0; c < NCLASS; ++c)  // (the charge lanes of the mixed adjoint have one block size)
-        threads[c] = h->class_off[c + 1] == h->class_off[c] ? 0 : kind == SW_VGRAD_F32 ? CL_NT : k.threads[c];
     return QMMM_OK;
 }
 
@@ -1874,7 +1858,6 @@ std::vector<long long> batch_key(const qmmm_batch *b, const double *const *dm, d
                 k.push_back(bits);
                 k.push_back(h->cls_variant[kind][c]);
             }
-        k.push_back(h->installed_mask);
         // scratch whose size follows the charge slices: a plain call under another sweep configuration
         // may have moved it
         k.push_back(ptr(h->pair_ws.p));

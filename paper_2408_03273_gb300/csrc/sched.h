@@ -67,17 +67,6 @@ inline void fine_slices(int n, const int *tiles, const double *w, const double *
     }
 }
 
-// Threads per block of class sweeps cut as above.  asked[c] > 0: the block size that was chosen for the
-// class, launched as it is.  0: the default, 256 threads, or 128 where all classes together have at most
-// four warps per SM: four warps to a block then put one on each SM sub-partition, which has an FP64 pipe
-// of its own.
-inline void block_threads(int n, const int *tiles, const int *ns, int nsm, const int *asked, int *threads)
-{
-    long long warps = 0;
-    for (int c = 0; c < n; ++c) warps += (long long)std::max(tiles[c], 0) * ns[c];
-    for (int c = 0; c < n; ++c) threads[c] = asked[c] > 0 ? asked[c] : warps <= 4LL * nsm ? 128 : 256;
-}
-
 // Ranges of pair batches of one class of the mixed adjoint (charge lanes), whose items are gx ranges times
 // ntile charge tiles.  A small system's class has a few charge tiles, and ranges of several batches
 // would leave it with a handful of blocks, each a long serial chain: its batches are spread over nsm

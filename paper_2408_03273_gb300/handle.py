@@ -79,9 +79,6 @@ class Handle:
     def set_tuning(self, kind: int, threads, weight=None):
         L.qmmm_set_tuning(self.h, kind, threads, weight)
 
-    def sweep_threads(self, kind: int):
-        return L.qmmm_sweep_threads(self.h, kind)
-
     def last_timing(self):
         return L.qmmm_last_timing(self.h)
 

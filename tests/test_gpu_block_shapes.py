@@ -1,17 +1,19 @@
-"""The block sizes that the class sweeps launch (qmmm_sweep_threads): an installed one on a system of
-few warps, the 128-thread default there, and the 256-thread default above four warps per SM; results
-in every shape against the oracle."""
-import numpy as np
+"""The block sizes that the class sweeps really launch, from a trace of the kernels: those that
+qmmm_get_tuning reports, on a system of few warps too, for the default, the 256-thread and the wide
+shapes; results in every shape against the oracle."""
+import json
+import re
+
 import pytest
 
 import oracle
 import workloads
-from _gpuutil import TOL_FP64, TOL_MIXED, check_V, gpu_all, grad_err
+from _gpuutil import TOL_FP64, TOL_MIXED, check_V, grad_err
 
 pytestmark = pytest.mark.gpu
 
-KINDS = {0: (0, 2), 1: (1, 3)}  # precision -> (V sweep kind, adjoint sweep kind)
-CHARGE_LANES = 3                # mixed adjoint: 256-thread blocks in every variant
+KERNELS = {0: "k_vpot_f64", 1: "k_vpot_f32", 2: "k_vgrad_f64"}  # sweep kind -> kernel
+KINDS = {0: (0, 2), 1: (1,)}  # precision -> kinds (the mixed adjoint's charge lanes have one block size)
 
 
 @pytest.fixture(scope="module")
@@ -23,61 +25,46 @@ def small():
     return s, ref
 
 
-def _sizes(h, kind, size):
-    return [size if n else 0 for n in h.info["n_prim_pairs_class"]]
+def _traced(call, path):
+    """The call's result and {(kernel, class): block sizes} of the sweep kernels that it launched."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(2):  # the first trace of a process can be empty: the tracer starts up in it
+        torch.zeros(1, device="cuda")
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            out = call()
+            torch.cuda.synchronize()
+    prof.export_chrome_trace(str(path))
+    sizes = {}
+    for e in json.loads(path.read_text())["traceEvents"]:
+        m = re.search(r"(k_v(?:pot|grad)_f\d\d)<(\d), (\d), \d+>", e.get("name", ""))
+        if m and e.get("cat") == "kernel":
+            la, lb = int(m.group(2)), int(m.group(3))
+            sizes.setdefault((m.group(1), la * (la + 1) // 2 + lb), set()).add(e["args"]["block"][0])
+    return out, sizes
 
 
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("shape", ["default", "256", "wide"])
-def test_launched_block_sizes(small, precision, shape):
+def test_launched_block_sizes(small, precision, shape, tmp_path):
+    pytest.importorskip("torch")
+    import paper_2408_03273_gb300 as q
     s, ref = small
-
-    def setup(h):
+    h = q.Handle(s, precision=precision, screen_tol=0.0)
+    try:
         for k in KINDS[precision]:
             wide = h.tuning(k)["wide"]
-            if shape == "256":
-                h.set_tuning(k, [256] * 10)
-            elif shape == "wide":
-                h.set_tuning(k, [w or 256 for w in wide])
-            if k == CHARGE_LANES or shape == "256":
-                want = _sizes(h, k, 256)
-            elif shape == "default":
-                want = _sizes(h, k, 128)
-            else:
-                want = [(w or 256) if n else 0 for w, n in zip(wide, h.info["n_prim_pairs_class"])]
-            assert h.sweep_threads(k) == want, k
-
-    g = gpu_all(s, precision=precision, screen_tol=0.0, setup=setup)
+            if shape != "default":
+                h.set_tuning(k, [w if shape == "wide" and w else 256 for w in wide])
+        (V, g), sizes = _traced(lambda: (h.vpot()[0], h.forces(s.dm)), tmp_path / "trace.json")
+        for k in KINDS[precision]:
+            t = h.tuning(k)["threads"]
+            for c, n in enumerate(h.info["n_prim_pairs_class"]):
+                assert n == 0 or sizes[KERNELS[k], c] == {t[c]}, (k, c)
+            assert shape != "wide" or any(x > 256 for x in t)
+    finally:
+        h.close()
     tol = TOL_FP64 if precision == 0 else TOL_MIXED
-    check_V(g["V"], ref["V"], precision)
-    for key in ("dE_dRqm", "dE_dRmm", "dE_dq"):
-        assert grad_err(g[key], ref, key, precision == 1) < tol, key
-
-
-def test_default_blocks_of_a_large_sweep():
-    import paper_2408_03273_gb300 as q
-    h = q.Handle(workloads.config2_active_site())
-    try:
-        for k in range(4):
-            assert h.sweep_threads(k) == _sizes(h, k, 256)
-        with pytest.raises(q.QMMMError):
-            h.sweep_threads(4)
-    finally:
-        h.close()
-
-
-def test_plan_of_another_shape_replaces_the_installed_one(small):
-    # an installed shape holds until it is replaced; the autotuner starts from the default again
-    import paper_2408_03273_gb300 as q
-    h = q.Handle(small[0])
-    try:
-        h.set_tuning(0, [256] * 10)
-        assert h.sweep_threads(0) == _sizes(h, 0, 256)
-        h.autotune(q.QMMM_TUNE_V)
-        t = h.tuning(0)
-        got = h.sweep_threads(0)
-        for c, n in enumerate(h.info["n_prim_pairs_class"]):
-            assert got[c] == (0 if not n else 128 if t["threads"][c] == 256 else t["wide"][c]), c
-        assert np.all(np.isfinite(h.vpot()[0]))
-    finally:
-        h.close()
+    check_V(V, ref["V"], precision)
+    for got, key in zip(g, ("dE_dRqm", "dE_dRmm", "dE_dq")):
+        assert grad_err(got, ref, key, precision == 1) < tol, key
