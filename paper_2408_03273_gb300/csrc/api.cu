@@ -647,11 +647,10 @@ int tile_cap(const qmmm_handle *h, int kind, int cls, int variant)
 }
 
 // Grid caps of the class kernels that the autotuner times alone, and the shares that qmmm_get_tuning
-// reports: shares of the SMs in proportion to each class's
-// SM-time (primitive pairs x cost), but never more blocks than the class has warps' worth of
-// 32-pair tiles for (times maxsl, when a class may split its charges over maxsl block rows);
-// what a capped class cannot use goes to the others.  Returns false when no class has work.
-bool split_sms(const qmmm_handle *h, int kind, const int *variant, int *share, int maxsl = 1)
+// reports: shares of the SMs in proportion to each class's SM-time (primitive pairs x cost), but never
+// more blocks than the class has warps' worth of 32-pair tiles for; what a capped class cannot use
+// goes to the others.  Returns false when no class has work.
+bool split_sms(const qmmm_handle *h, int kind, const int *variant, int *share)
 {
     double w[NCLASS];
     int cap[NCLASS];
@@ -663,7 +662,7 @@ bool split_sms(const qmmm_handle *h, int kind, const int *variant, int *share, i
         cap[c] = 0;
         w[c] = 0.0;
         if (!open[c]) continue;
-        cap[c] = tile_cap(h, kind, c, variant[c]) * maxsl;
+        cap[c] = tile_cap(h, kind, c, variant[c]);
         w[c] = npp * std::max(h->cls_cost[kind][c], 1e-30);
         ++nopen;
     }

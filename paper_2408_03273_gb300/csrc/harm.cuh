@@ -460,38 +460,6 @@ __host__ __device__ __forceinline__ void harm_eval(const double (&M)[nherm(L)], 
     ez = fma(-Z, w, ez);
 }
 
-// Hermite coefficients D -> harmonic coefficients M (constants of the radial factors included)
-template <int L>
-__device__ __forceinline__ void harm_fold(const double (&D)[nherm(L)], double (&M)[nherm(L)])
-{
-    double out[nherm(L)];
-    for (int i = 0; i < nherm(L); ++i) out[i] = 0.0;
-#pragma unroll 1
-    for (int i = 0; i < HT.tend[L]; ++i) {
-        const HarmEntry &t = HT.t[i];
-        out[harm_off(L, t.k) + t.lm] += t.c * D[t.herm];
-    }
-#pragma unroll
-    for (int i = 0; i < nherm(L); ++i) M[i] = out[i];
-}
-// harmonic sums -> Hermite sums W_tuv = sum_C q R_tuv
-template <int L>
-__device__ __forceinline__ void harm_unfold(const double (&S)[nherm(L)], double (&W)[nherm(L)])
-{
-    double in[nherm(L)], out[nherm(L)];
-#pragma unroll
-    for (int i = 0; i < nherm(L); ++i) {
-        in[i] = S[i];
-        out[i] = 0.0;
-    }
-#pragma unroll 1
-    for (int i = 0; i < HT.tend[L]; ++i) {
-        const HarmEntry &t = HT.t[i];
-        out[t.herm] += t.c * in[harm_off(L, t.k) + t.lm];
-    }
-#pragma unroll
-    for (int i = 0; i < nherm(L); ++i) W[i] = out[i];
-}
 // gradient coefficients: sum_lm M_klm d Y_lm / da = sum N^a_k,lm1 Y_lm1
 template <int L>
 __device__ __forceinline__ void harm_grad(const double (&M)[nherm(L)], double (&Nx)[nhgrad(L) + 1],

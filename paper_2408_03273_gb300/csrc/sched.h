@@ -7,6 +7,9 @@
 
 namespace qmmm {
 
+// Two rules of the share-capped sweeps that fine_slices replaced, vpot_max_slices and class_slices; only
+// tests/test_sched.py calls them.
+//
 // Most charge slices per V class: at least 128 charges each, at most 8, and the partial
 // matrices (one per slice, each V element written by one class and slice, summed in a fixed
 // order) within 512 MB.

@@ -1,5 +1,5 @@
 // tc_digits.cuh -- exact BF16 digit planes of fixed-point numbers for the tensor-core sums
-// (recip_tc.cu, mmrecip_tc.cu), and 2^61 fixed-point complex arithmetic on 32-bit halves.
+// (recip_tc.cu, mmrecip_tc.cu), and 2^61 fixed-point arithmetic on 32-bit halves.
 //
 // A 48-bit fixed-point value v (|v| <= 2^48) is written as seven balanced planes, a leading one
 // and six base-128 digits: v 2^-48 = 2^-6 sum_{s<7} p_s with p_0 in [-64, 64] and
@@ -44,27 +44,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
-// 2^61 fixed point split into 32-bit halves: x = h 2^31 + l, l in [0, 2^31), |h| <= 2^30; an int4
-// holds (re h, re l, im h, im l)
-__device__ __forceinline__ int4 split61(long long re, long long im)
-{
-    return make_int4((int)(re >> 31), (int)(re & 0x7fffffff), (int)(im >> 31), (int)(im & 0x7fffffff));
-}
+// 2^61 fixed point split into 32-bit halves: x = h 2^31 + l, l in [0, 2^31), |h| <= 2^30
 __device__ __forceinline__ long long join61(int h, int l) { return (long long)h * 2147483648ll + l; }
 // (x y) / 2^62 for 2^61 values, within 1 unit: the low x low term is dropped
 __device__ __forceinline__ long long mul61(long long x, long long y)
 {
     const int xh = (int)(x >> 31), xl = (int)(x & 0x7fffffff), yh = (int)(y >> 31), yl = (int)(y & 0x7fffffff);
     return (long long)xh * yh + (((long long)xh * yl + (long long)xl * yh) >> 31);
-}
-// complex product of two split 2^61 values at 2^60 scale, within 2 units (six 32 x 32 -> 64
-// products and four for the cross terms)
-__device__ __forceinline__ void cmul61(const int4 x, const int4 y, long long &re, long long &im)
-{
-    const long long mr = (long long)x.x * y.y + (long long)x.y * y.x - (long long)x.z * y.w - (long long)x.w * y.z;
-    const long long mi = (long long)x.x * y.w + (long long)x.y * y.z + (long long)x.z * y.y + (long long)x.w * y.x;
-    re = (long long)x.x * y.x - (long long)x.z * y.z + (mr >> 31);
-    im = (long long)x.x * y.z + (long long)x.z * y.x + (mi >> 31);
 }
 // a real split value, and the product of two at 2^60 scale, within 1 unit
 __device__ __forceinline__ int2 split61r(long long x) { return make_int2((int)(x >> 31), (int)(x & 0x7fffffff)); }
