@@ -159,7 +159,9 @@ int qmmm_set_positions(qmmm_handle *h, const double *qm_xyz, const double *mm_xy
 
 /* Region-I one-electron matrix V[nao*nao] of Eq. 9 (symmetric) and, if E_nuc_mm != NULL, the
  * region-I nuclear-MM energy sum_j sum_{i in I} Z_j q_i erf(r/sigma_i)/r.  V stays cached in
- * the handle for qmmm_energy. */
+ * the handle for qmmm_energy.  Scratch, kept by the handle: FP64, C(L+3,3) doubles per primitive pair
+ * and charge slice, L = l_A + l_B (1 slice on large systems, up to 16 on small ones; shared with
+ * qmmm_forces); mixed, the slices' partial V, at most 512 MB. */
 int qmmm_vpot(qmmm_handle *h, double *V, double *E_nuc_mm);
 
 /* Multipole part at density dm[nao*nao] (symmetric): E_II (scalar), optionally the Mulliken
@@ -180,7 +182,8 @@ int qmmm_density_gradient(qmmm_handle *h, const double *dm, double *G);
 
 /* Gradient of E_QM-MM at fixed dm (region-I integral derivatives, nuclear-MM term, tensor
  * derivatives, and the multipole Pulay term of Eq. 15): dE_dRqm[natm*3], dE_dRmm[nmm*3],
- * dE_dq[nmm].  Any output may be NULL. */
+ * dE_dq[nmm].  Any output may be NULL.  Scratch, kept by the handle: FP64, 2 C(L+3,3) + 3 doubles per
+ * primitive pair (1.4 KB for (f,f); 150 atoms with f shells, 650 000 pairs: 171 MB). */
 int qmmm_forces(qmmm_handle *h, const double *dm, double *dE_dRqm, double *dE_dRmm, double *dE_dq);
 
 /* Plan counts. */

@@ -379,9 +379,14 @@ int copy_out(qmmm_handle *h, double *dst, const double *src, size_t n)
 }
 
 // The reciprocal-sum method in effect; allocates the tensor-core scratch the first time it is
-// needed.  QMMM_RECIP_AUTO: the tensor cores once the reciprocal work is large enough to outweigh
-// the five extra launches of each tensor-core sum (the CUDA-core kernels win below ~4e7 dense G
-// entries x charges: on the 645-charge water workload, 1.2e6, by 0.14 ms per mixed step).
+// needed.  QMMM_RECIP_AUTO: the tensor cores once the reciprocal work (dense G entries x charges)
+// outweighs the launches that each of their sums adds.  Positions and forces of a 3-atom system, CUDA
+// cores / tensor cores, ms:
+//   mixed: 0.545 / 0.613 at 1.1e6 (kmax 7, 591 charges), 0.642 / 0.636 at 1.6e7 (9, 4491), 0.838 / 0.654 at
+//          3.6e7 (11, 5697), 1.025 / 0.665 at 6.3e7 (11, 9897);
+//   FP64:  0.923 / 0.859, 1.244 / 0.900, 2.037 / 0.907, 2.821 / 0.932.
+// The line is the one measured for the sums over complex phases, which took twice as long; for the
+// present ones it lies above the crossover.
 constexpr double RECIP_TC_MIN_WORK = 4e7;
 int select_recip(qmmm_handle *h)
 {
@@ -394,7 +399,8 @@ int select_recip(qmmm_handle *h)
         const TcShape &sh = h->ew.tcs;
         int rc;
         if ((rc = h->tc_phase.ensure(sh.phase_bytes)) || (rc = h->tc_bpl.ensure(sh.bplane_words)) ||
-            (rc = h->tc_real.ensure(sh.real_sums)) || (rc = h->tc_bmax.ensure(sh.nbmax)) || (rc = h->tc_part.ensure(sh.part_ints)))
+            (rc = h->tc_real.ensure(sh.real_sums)) || (rc = h->tc_bmax.ensure(sh.nbmax)) ||
+            (rc = h->tc_part.ensure(sh.part_ints)))
             return rc;
         // the padding beyond the last charge is copied but never used; keep it defined
         CUDA_TRY(cudaMemset(h->tc_phase.p, 0, sh.phase_bytes));
@@ -677,12 +683,13 @@ bool split_sms(const qmmm_handle *h, int kind, const int *variant, int *share)
 // Most charge slices of a class sweep.
 constexpr int MAX_SLICES = 16;
 
-// Per-pair work of a sweep outside its charge loop, in charges of loop work: the Hermite and
-// density algebra, FP64 in both precisions (against an FP32 charge loop on the mixed path).
+// Per-pair work of a sweep outside its charge loop, in charges of loop work, which every charge slice
+// repeats: on the mixed path the Hermite algebra, FP64 against an FP32 charge loop; in the FP64 sweeps,
+// whose pair algebra has kernels of its own, the pair's geometry and in the adjoint the gradient
+// coefficients (harm_grad).
 double setup_charges(int kind)
 {
-    if (kind_is_mixed(kind)) return 64.0;
-    return 3.0;  // (the FP64 sweeps' pair algebra has kernels of its own)
+    return kind_is_mixed(kind) ? 64.0 : 3.0;
 }
 
 // How the classes of a sweep over nch charges are cut into blocks: charge slices per class, launch
@@ -1421,7 +1428,7 @@ static int compute_multipoles(qmmm_handle *h, const double *ddm, double *F, int 
     CUDA_TRY(cudaMemcpyAsync(h->mult.p, h->mult_init.p, 10 * (size_t)h->natm * sizeof(double), cudaMemcpyDeviceToDevice, st));
     const BasisDev b = h->basis();
     const int mode = MOM_MULT | (F ? MOM_FOCK : 0) | extra_mode;
-    // the classes are small kernels (one lane per primitive pair): run them concurrently
+    // the classes are small kernels (a block per 32 primitive pairs): run them concurrently
     return fork_classes(h, [&](int cls, int p0, int p1, cudaStream_t cs) {
         return launch_moments(b, cls, p0, p1, ddm, h->phi.p, h->mult.p, F, h->gqm.p, mode, cs);
     });
@@ -1572,9 +1579,9 @@ int qmmm_forces(qmmm_handle *h, const double *dmat, double *dE_dRqm, double *dE_
         if ((rc = join_classes(h, h->tstream))) return rc;
         CUDA_TRY(cudaEventRecord(h->ev[1], h->tstream));
     }
-    // The rest follows the sweep: run beside it, it delayed the FP64 classes, which hold their
-    // shares of the SMs for the whole sweep (large site: FP64 step 461 -> 496 ms), and on the mixed
-    // path it saved 2.6 of 49.6 ms but left the sweep's own duration unmeasurable
+    // The rest follows the sweep.  Beside it, each of its blocks that took an SM would keep an FP64 sweep
+    // block, which needs a whole one, waiting; measured when the classes still held fixed shares of the
+    // SMs: large site, FP64 step 461 -> 496 ms, mixed 49.6 -> 47.0 ms with the sweep's own duration lost
     if ((rc = join_classes(h, h->stream))) return rc;
     if ((rc = forces_rest(h, ddm))) return rc;
     if ((rc = forces_end(h, dE_dRqm, dE_dRmm, dE_dq))) return rc;
@@ -1621,8 +1628,8 @@ int qmmm_qm_images(qmmm_handle *h, const double *dmat, double *E, double *dE_dRq
     const double *ddm;
     const size_t n2 = (size_t)h->nao * h->nao, na = (size_t)h->natm;
     if ((rc = stage_input(h, dmat, n2, h->dm, &ddm))) return rc;
-    if ((rc = h->qmq_ws.ensure(qm_images_scratch(h->ewald(), h->nsm))) || (rc = h->qmq_u.ensure(na * 20)) || (rc = h->qmq_g.ensure(na * 3)) ||
-        (rc = h->qmq_E.ensure(1)))
+    if ((rc = h->qmq_ws.ensure(qm_images_scratch(h->ewald(), h->nsm))) || (rc = h->qmq_u.ensure(na * 20)) ||
+        (rc = h->qmq_g.ensure(na * 3)) || (rc = h->qmq_E.ensure(1)))
         return rc;
     double *Fd = nullptr;
     if (F) {
@@ -1632,7 +1639,8 @@ int qmmm_qm_images(qmmm_handle *h, const double *dmat, double *E, double *dE_dRq
     }
     // Mulliken multipoles at this density, then the image tensors, energy, potentials, gradient
     if ((rc = compute_multipoles(h, ddm, nullptr, 0))) return rc;
-    CUDA_TRY(launch_qm_images(h->ewald(), h->gfac.p, h->mult.p, h->qmq_ws.p, h->nsm, h->qmq_E.p, h->qmq_u.p, h->qmq_g.p, st));
+    CUDA_TRY(launch_qm_images(h->ewald(), h->gfac.p, h->mult.p, h->qmq_ws.p, h->nsm, h->qmq_E.p, h->qmq_u.p,
+                              h->qmq_g.p, st));
     // the multipoles move with the basis (Pulay) and depend on gamma (Fock): the moment kernels
     // with the image potential in place of the MM one
     const BasisDev b = h->basis();

@@ -922,7 +922,8 @@ __device__ __forceinline__ void multipole_field(const double *M, double x, doubl
 {
     const double tx = M[4] * x + M[5] * y + M[6] * z, ty = M[5] * x + M[7] * y + M[8] * z,
                  tz = M[6] * x + M[8] * y + M[9] * z;
-    const double mu = M[1] * x + M[2] * y + M[3] * z, tr = 0.5 * (M[4] + M[7] + M[9]), xx = 0.5 * (tx * x + ty * y + tz * z);
+    const double mu = M[1] * x + M[2] * y + M[3] * z, tr = 0.5 * (M[4] + M[7] + M[9]);
+    const double xx = 0.5 * (tx * x + ty * y + tz * z);
     pot += s * (M[0] * f + (mu + tr) * g1 + xx * g2);
     const double w = s * (M[0] * g1 + (mu + tr) * g2 + xx * g3), h1 = s * g1, h2 = s * g2;
     fld[0] += w * x + h1 * M[1] + h2 * tx;

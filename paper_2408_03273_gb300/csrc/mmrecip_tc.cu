@@ -16,7 +16,8 @@
 // Over complex phases K was twice as long and an entry cost two multiplications.  Sum of a 150-atom
 // site (kmax 24, 200 001 charges), mixed path: 4.36 -> 2.64 ms with the real functions, -> 2.02 ms with the
 // z rows resident in shared memory and the y rows of a chunk in one copy; FP64 path 14.9 -> 8.0 ms.
-// Bound: the producers' integer work and barrier round trips per chunk (tensor pipe a third busy).
+// Bound: the producers' integer work and barrier round trips per chunk (FP64 path, 60-atom site: 0.97 ms,
+// tensor pipe 22% busy, issue slots 35%).
 //
 // A operand (M = 128 charges x K): the products of the charges' real phases, digitised on chip from
 // fixed-point phase rows staged by TMA; B operand (N = 112 rows (k, n_x, re/im) x K): B_k divided
@@ -28,8 +29,9 @@
 // merged: the merged sum's FP32 rounding is about 2^-31 of level 0's scale), so 160 rows per tile
 // and the three channels of kx <= 25 take a single N tile: the A operand is digitised once and no
 // N row beyond the 6 (kx + 1) in use is computed.  Against the double-float CUDA-core kernel the
-// mixed path's sum differs by 3e-9 (active site, kmax 16) and 1.3e-8 (large site, kmax 24) of the
-// largest MM gradient component, a tenth or less of the mixed path's error against FP64.  Level 0
+// mixed path's sum differs by 9e-10 (dE/dq: 1.6e-9; active site, kmax 16) and 5.5e-9 (7.3e-9; large site,
+// kmax 24) of the largest MM gradient component, a tenth or less of the mixed path's error against
+// FP64; the FP64 sum from the CUDA cores' by 1.7e-13 (3.4e-13) and 1.1e-12 (1.6e-12).  Level 0
 // is exact for any input while 4096 N_y N_z < 2^24 (kmax <= 31) and beyond that unless the
 // row-normalised coefficients, which decay as exp(-G^2/4 alpha^2), sum to more than 2^11 in
 // magnitude; levels 1 to 3 are sums of random-sign digit products, typically 2^17 or less.  The epilogue
@@ -547,8 +549,8 @@ void tc_mmr_shape(const EwaldDev &e, int nacc, int np, MmrShape &sh)
 
 template <int NP>
 static cudaError_t mm_recip_np(const EwaldDev &e, const MmrShape &sh, const MmrBuf &b, const double2 *A,
-                               const double2 *Az, const unsigned char *Yt, const unsigned char *Zt, double *dq, double *dR, int *err,
-                               cudaStream_t st);
+                               const double2 *Az, const unsigned char *Yt, const unsigned char *Zt, double *dq,
+                               double *dR, int *err, cudaStream_t st);
 
 cudaError_t launch_mm_recip_tc(const EwaldDev &e, const MmrShape &sh, const MmrBuf &b, const double2 *A,
                                const double2 *Az, double *dq, double *dR, int *err, cudaStream_t st)
@@ -569,8 +571,8 @@ cudaError_t launch_mm_recip_tc(const EwaldDev &e, const MmrShape &sh, const MmrB
 // B planes and the MMA kernel with NP planes per operand
 template <int NP>
 static cudaError_t mm_recip_np(const EwaldDev &e, const MmrShape &sh, const MmrBuf &b, const double2 *A,
-                               const double2 *Az, const unsigned char *Yt, const unsigned char *Zt, double *dq, double *dR, int *err,
-                               cudaStream_t st)
+                               const double2 *Az, const unsigned char *Yt, const unsigned char *Zt, double *dq,
+                               double *dR, int *err, cudaStream_t st)
 {
     cudaError_t rc;
     const int NX = e.kmax[0] + 1, NY = 2 * e.kmax[1] + 1, NZ = 2 * e.kmax[2] + 1;

@@ -33,7 +33,10 @@ __host__ __device__ constexpr int op_y(int c) { return c == 2 ? 1 : c == 7 ? 2 :
 __host__ __device__ constexpr int op_z(int c) { return c == 3 ? 1 : c == 9 ? 2 : (c == 6 || c == 8) ? 1 : 0; }
 // Exponents of the octupole components xxx, xxy, xxz, xyy, xyz, xzz, yyy, yyz, yzz, zzz
 __host__ __device__ constexpr int o3_x(int c) { return c == 0 ? 3 : c <= 2 ? 2 : c <= 5 ? 1 : 0; }
-__host__ __device__ constexpr int o3_z(int c) { return c == 9 ? 3 : (c == 5 || c == 8) ? 2 : (c == 2 || c == 4 || c == 7) ? 1 : 0; }
+__host__ __device__ constexpr int o3_z(int c)
+{
+    return c == 9 ? 3 : (c == 5 || c == 8) ? 2 : (c == 2 || c == 4 || c == 7) ? 1 : 0;
+}
 __host__ __device__ constexpr int o3_y(int c) { return 3 - o3_x(c) - o3_z(c); }
 
 // 1-D moments M^e_t about a centre at distance X from P

@@ -207,16 +207,19 @@ enum SweepKind { SW_VPOT_F64 = 0, SW_VPOT_F32 = 1, SW_VGRAD_F64 = 2, SW_VGRAD_F3
 // Threads per block of the wide variant of a sweep kernel (0: none).  All warps of a block share
 // one staged chunk of charges, and that chunk's shared memory allows one block per SM, so the
 // block size sets the warps per SM.  A block of NT threads launched with __launch_bounds__(NT, 1)
-// may use 65536 / NT registers per thread, rounded down to a multiple of 8; NT is the widest block
-// whose cap stays at or above the kernel's register count at 256 threads, so the wide variant
-// holds more warps per SM without spilling.  Classes at 255 registers have no wide variant.
+// may use 65536 / NT registers per thread, rounded down to a multiple of 8.  The sizes were chosen as
+// the widest whose cap covered the register counts of the Hermite-recursion kernels; saved
+// configurations name them (qmmm_set_tuning), so they stay.  Counts of the present kernels at 256
+// threads beside them (ptxas): no FP64 kernel spills in its wide block, and V (p,s) (p,p) (d,p) (f,s) (f,p),
+// adjoint (p,s) (p,p) (d,s) would have room for a wider one; the mixed V of (s,s) (p,s) (d,p) spills 20, 88
+// and 68 bytes in its.
 __host__ __device__ constexpr int sweep_wide_threads(int kind, int cls)
 {
     // class order: (0,0) (1,0) (1,1) (2,0) (2,1) (2,2) (3,0) (3,1) (3,2) (3,3)
     constexpr int T[SW_NKIND][10] = {
-        {1024, 640, 512, 640, 384, 384, 512, 0, 0, 0},  // vpot_f64 : 64 87 105 96 150 158 120 regs
-        {896, 768, 512, 512, 384, 0, 384, 0, 0, 0},     // vpot_f32 : 68 80 106 102 154 - 136
-        {640, 512, 0, 0, 0, 0, 0, 0, 0, 0},             // vgrad_f64: 93 117
+        {1024, 640, 512, 640, 384, 384, 512, 0, 0, 0},  // vpot_f64 : 64 80 96 96 118 150 118 150 206 254
+        {896, 768, 512, 512, 384, 0, 384, 0, 0, 0},     // vpot_f32 : 95 112 135 127 177 242 167 255 255 255
+        {640, 512, 0, 0, 0, 0, 0, 0, 0, 0},             // vgrad_f64: 90 112 162 162 238 255 238 255 255 255
         {256, 256, 256, 256, 256, 256, 256, 256, 0, 0}, // vgrad_f32: charge lanes, variant 1 as
                                                         // cl_variant (256 threads either way)
     };

@@ -48,8 +48,9 @@ struct qmmm_handle_impl;
 // Region-I sweeps.  A launch has `nblk` blocks of `threads` threads per charge slice (at most 256, or
 // the class's wide block, sweep_wide_threads, where one exists); its warps take the class's tiles in
 // turn.  `nslice` splits the charge chunk over that many block rows, the mixed V kernels then writing
-// slice s into V + s * vstride (FP64: slices of the pairs' sums, added before the contraction).  The mixed adjoint (launch_vgrad_f32) sizes its own grid; `variant`
-// picks its charges per lane (cl_variant).
+// slice s into V + s * vstride (FP64: slices of the pairs' sums, added before the contraction).  The
+// mixed adjoint (launch_vgrad_f32) sizes its own grid from nsm, the SMs; `variant` picks its charges
+// per lane (cl_variant).
 // dst[k] = sum_s src[s*n + k], s < nslice, in order (the V slices)
 cudaError_t launch_sum_slices_d(const double *src, int nslice, size_t n, double *dst, cudaStream_t st);
 // sums: scratch of the class, nslice x the Hermite sums of every primitive pair

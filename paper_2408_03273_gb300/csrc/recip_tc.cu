@@ -11,10 +11,11 @@
 // with signs (k_sf_tc_combine).  Over complex phases both operands had re and im rows per charge:
 // twice the products, two N tiles (and so twice the digitising) beyond kz = 19 and two
 // multiplications per entry of A.  k_sf_tc on a 150-atom site (kmax 24, 200 001 charges): 4.07 -> 2.01 ms;
-// the producers' integer work is the bound (tensor pipe 30% busy).
+// the producers' integer work is the bound (60-atom site: 0.31 ms, tensor pipe 29% busy, issue slots 42%).
 //
-// The product is D[line, rz] = sum_k A[line, k] B[rz, k], k the charge.  The tensor cores multiply BF16 operands exactly and accumulate in FP32, so
-// the FP64-class product is built from exact pieces (an Ozaki-type split): every operand element,
+// The product is D[line, rz] = sum_k A[line, k] B[rz, k], k the charge.  The tensor cores multiply BF16
+// operands exactly and accumulate in FP32, so the FP64-class product is built from exact pieces (an
+// Ozaki-type split): every operand element,
 // a 48-bit fixed-point number v (|v| <= 2^48, scaled by 1/max|q| for A), is written as seven
 // balanced digit planes, a leading one and six of base 128,
 //     v 2^-48 = 2^-6 sum_{s<7} p_s,   p_0 in [-64, 64],  p_s in [-64, 63] 2^-7s (s >= 1),

@@ -20,14 +20,15 @@
 // of small systems.  Sweep of a QM water 0.53 -> 0.34 ms, of 17 atoms with f shells 4.31 -> 2.05 ms; of the
 // 60- and the 150-atom site, which hide the chain, unchanged (45 and 194 ms).
 //
-// Bound: the FP64 pipe, 2 lanes per clock and SM, 85-91% busy, with 7-8% of the issue slots used: the
-// kernel's time is its count of FP64 instructions.  So the tensors R are never formed: D0 and W are
-// kept as solid-harmonic components (harm.cuh), per charge one recursion of (L+1)^2 harmonics, one
-// multiply-add per harmonic for the value, the charge sum and each gradient component (these with
-// the coefficients N of the differentiated harmonics, one order lower).  FP64 instructions per
-// (warp, charge) on a 60-atom active site, setup included: (s,s) 30, (p,p) 77, (d,s) 87, (d,p) 140,
-// (d,d) 241.  Coefficients and sums of the high classes spill to local memory ((f,f): 2.9 KB
-// stores), which the idle load pipe carries.  Adjoint sweep against the Hermite recursion with its
+// Bound: the FP64 pipe, 2 lanes per clock and SM, 88-90% busy on the SMs that hold a block and 85-86% over
+// a whole sweep, with 7-8% of the issue slots used: the kernel's time is its count of FP64
+// instructions.  So the tensors R are never formed: D0 and W are kept as solid-harmonic components
+// (harm.cuh), per charge one recursion of (L+1)^2 harmonics, one multiply-add per harmonic for the
+// value, the charge sum and each gradient component (these with the coefficients N of the
+// differentiated harmonics, one order lower).  FP64 instructions per (warp, charge) for L = 0..6, setup
+// included: 31, 46, 83, 138, 214, 310, 423 (150-atom site with f shells; a 60-atom site within 1.5%).
+// Coefficients and sums of the high classes spill to local memory ((f,f): 2.9 KB stores), which the
+// idle load pipe carries.  Adjoint sweep against the Hermite recursion with its
 // contractions: active site 78.3 -> 60.9 ms, a 150-atom site with f shells 412 -> 242 ms, a QM
 // water 1.35 -> 0.82 ms (untuned handles).
 //

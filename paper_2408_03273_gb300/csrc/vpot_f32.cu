@@ -182,7 +182,7 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
         if (e != cudaSuccess) return e;
         attr = true;
     }
-        VJob one{};
+    VJob one{};
     one.bd = bd;
     one.rg = rg;
     one.V = V;
@@ -192,8 +192,8 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
     one.ch_end = ch_end;
     one.gx = nblk;
     one.ns = nslice;
-    k_vpot_f32<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(one, nullptr, 0, boys + (size_t)(LA + LB) * BOYS_TAB_F,
-                                                                 tb, vstride, err);
+    k_vpot_f32<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(
+        one, nullptr, 0, boys + (size_t)(LA + LB) * BOYS_TAB_F, tb, vstride, err);
     return cudaGetLastError();
 }
 
@@ -229,7 +229,8 @@ cudaError_t VpotF32<LA, LB>::run(const BasisDev &bd, const RegionDev &rg, int pp
         if (threads == W)
             return launch_nt<LA, LB, W>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice,
                                         vstride, st);
-    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice, vstride, st);
+    return launch_nt<LA, LB, 256>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys, V, err, nblk, threads, nslice,
+                                  vstride, st);
 }
 
 template <int LA, int LB>

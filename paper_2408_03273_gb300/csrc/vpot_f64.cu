@@ -7,10 +7,10 @@
 // charges (x, y, z, q) into shared memory with one TMA bulk copy, every lane sweeps all of them
 // (shared-memory broadcast) and accumulates W_tuv = sum_C q_C s_C R_tuv in registers, as
 // solid-harmonic components (harm.cuh).  The bound is the FP64 pipe (90% busy, 8% of the issue
-// slots used), so the kernel's time is its count of FP64 instructions: per (warp, charge) 13 for
-// (s,s), 38 (d,s), 106 (d,d) on a 60-atom active site.  V sweep against the Hermite recursion:
-// active site 33.5 -> 24.4 ms, a 150-atom site with f shells 147 -> 104 ms, a QM water 0.43 ->
-// 0.33 ms (untuned handles).  Charges are grouped by Gaussian width so that rho is formed once per
+// slots used), so the kernel's time is its count of FP64 instructions: per (warp, charge) 13, 21,
+// 37, 61, 94, 135, 182 for L = 0..6, setup included (150-atom site with f shells; a 60-atom site within
+// 1.5%).  V sweep against the Hermite recursion: active site 33.5 -> 24.4 ms, a 150-atom site with f
+// shells 147 -> 104 ms, a QM water 0.43 -> 0.33 ms (untuned handles).  Charges are grouped by Gaussian width so that rho is formed once per
 // (primitive pair, width class).
 //
 // The sweep leaves the sums of every pair and charge slice; k_pair_V adds the slices in a fixed order
@@ -179,8 +179,8 @@ static cudaError_t launch_nt(const BasisDev &bd, const RegionDev &rg, int pp_beg
         if (e != cudaSuccess) return e;
         attr = true;
     }
-        k_vpot_f64<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end, boys,
-                                                                      sums, err);
+    k_vpot_f64<LA, LB, NT><<<dim3(nblk, nslice), threads, smem, st>>>(bd, rg, pp_begin, pp_end, ch_begin, ch_end,
+                                                                      boys, sums, err);
     return cudaGetLastError();
 }
 

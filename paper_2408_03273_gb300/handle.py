@@ -32,7 +32,7 @@ class Handle:
 
     def set_recip_method(self, method: int):
         """QMMM_RECIP_CUDA_CORES, QMMM_RECIP_TENSOR (structure factor on the tensor cores) or
-        QMMM_RECIP_AUTO (tensor cores for the mixed path)."""
+        QMMM_RECIP_AUTO (tensor cores for large reciprocal sums)."""
         L.qmmm_set_recip_method(self.h, method)
 
     def set_positions(self, qm_xyz, mm_xyz, mm_q=None):
