@@ -63,20 +63,46 @@ def flops_adjoint(L):
 
 
 def flops_fp64(L, adjoint):
-    """The same for the FP64 sweeps, which work in solid harmonics: (L+1)^2 harmonics with one radial
-    factor per l, and per harmonic a multiply-add for the charge sum (the adjoint: the value, the charge
-    sum and the gradient).  Two FLOPs per executed FP64 instruction, by a fit to their counts:
-    10 + 3.1 (L+1)^2 for V, 23 + 7.1 (L+1)^2 for the adjoint."""
-    return 2 * (23 + 7.1 * (L + 1) ** 2 if adjoint else 10 + 3.1 * (L + 1) ** 2)
+    """The same for the FP64 sweeps, which work in solid harmonics, for a distant charge (csrc/harm.cuh;
+    the Gaussian terms of near charges are not counted): displacement and r^2 8, reciprocal root 8,
+    radial factors, the harmonics' recursion, 2 per harmonic for the charge sum, and in the adjoint 2
+    more for the value and 6 per differentiated harmonic for the gradient, 10 per order to join
+    them, and the sums over the pairs."""
+    n = (L + 1) ** 2
+    walk = 0
+    for m in range(L + 1):
+        walk += 6 if m > 1 else 0
+        for l in range(m, L):  # noqa: E741
+            if l == m:
+                walk += 2 if m else 0
+            else:
+                walk += 1 + (2 if (l == 1 and m == 0) else 3) + (3 if m else 0)
+    if not adjoint:
+        return 16 + (2 if L else 1) + L + walk + 2 * n
+    return 17 + 2 * L + 1 + walk + 4 * n - 3 + (6 * (L * L - 1) if L else 0) + 10 * L + 20
 
 
 CLASS_L = [la + lb for la in range(4) for lb in range(la + 1)]  # class index la(la+1)/2 + lb
+
+# FP64 instructions that the FP64 sweeps execute per (warp of 32 primitive pairs, charge), by class, the
+# pairs' setup and the near charges included: smsp__inst_executed_pipe_fp64 of one step on the large
+# site (those of the active site, without f shells, differ by at most 1.5%).
+FP64_INST = {False: [13.4, 21.1, 36.4, 37.0, 61.1, 94.5, 60.8, 92.8, 134.8, 181.7],
+             True: [31.1, 46.1, 82.9, 83.6, 138.6, 215.8, 138.1, 212.4, 309.9, 422.5]}
+
+
+def fp64_pipe(info, adjoint, ms):
+    """Share of the FP64 pipes' time (2 lanes per clock and SM, 152 SMs, 2070 MHz) that a sweep of `ms`
+    keeps them busy, from its count of FP64 instructions."""
+    n = sum(-(-p // 32) * info["n_region1"] * FP64_INST[adjoint][c] for c, p in enumerate(info["n_prim_pairs_class"]))
+    return {"warp_instructions": n, "busy": n * 32 / (2 * 152 * 2.070e9) / (ms * 1e-3)}
+
 
 # DRAM bytes (read + write) of one adjoint sweep (all angular-class kernels of one call, the mixed
 # path's pair records and pair gradients included), per (workload, precision), from one ncu
 # capture of the current kernels (dram__bytes_read.sum + dram__bytes_write.sum); a workload or
 # precision without a capture of the current kernels reports None.
-SWEEP_TRAFFIC = {("c4", "mixed"): 364_729_600}
+SWEEP_TRAFFIC = {("c4", "mixed"): 364_729_600, ("c4", "fp64"): 558_068_480}
 
 
 def sweep_flops(info, adjoint, fp64):
@@ -568,6 +594,8 @@ def main():
             "peak_note": ("FP64 plain-ALU peak from the unit counts at 2070 MHz (152 SMs x 2 DFMA/clk)"
                           if prec == q.QMMM_FP64 else "FP32 plain-ALU peak at 2070 MHz (152 SMs x 128 FFMA/clk)"),
             "flops_per_launch": fl}
+    if prec == q.QMMM_FP64:
+        roof["fp64_pipe"] = fp64_pipe(info, dom_adj, roof["kernel_ms"])
 
     # launches of our kernels per step (a claim; the ncu launch list of this command confirms the
     # composition).  Per call:
