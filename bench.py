@@ -604,8 +604,8 @@ def main():
     #     double-float g(G) S(G) table),
     #     plus the structure factor (tensor cores: max|q|, phases, B planes, MMA, reduction, combination = 6;
     #     CUDA cores: kernel + slice sum = 2)
-    #   vpot: one kernel per class and charge chunk (FP64: and the contraction of its pair sums) +
-    #     nuclear-MM term and its sum
+    #   vpot: one kernel per class and charge chunk (FP64: and the contraction of its pair sums), the sum of
+    #     V's slices with its mirror image + nuclear-MM term and its sum
     #   ewald: one moments kernel per class + the energy terms
     #   forces: one moments kernel per class (Pulay) + the adjoint per class and chunk: density fold (mixed
     #     path: pair records), sweep, pair gradients = 3
@@ -613,12 +613,9 @@ def main():
     #     gradient, scatter, unpermute) + the MM-side reciprocal sum (tensor cores: atom phases,
     #     multipole structure factor, phases, scales, B planes per N tile, MMA = 5 + tiles; CUDA
     #     cores: 3)
-    # The mixed vpot adds one V slice-sum kernel when its classes split their charges (128 or more
-    # region-I charges and room for two partial matrices in 512 MB).
     def launches_per_step(precision):
         ncls = sum(1 for n in info["n_prim_pairs_class"] if n > 0)
         nI = info["n_region1"]
-        v_maxsl = min(min(nI, 4096) // 64, (512 << 20) // max(1, 8 * s.nao * s.nao))
         ch_f = math.ceil(nI / 4096) if nI else 0
         ch_g = math.ceil(nI / 2560) if nI else 0
         tensor = recip_in_effect(precision).startswith("tensor cores")
@@ -630,7 +627,7 @@ def main():
         mm_tc = tensor and (2 * cpt * kx + 15) // 16 * 16 <= lim and 2 * s.kmax[2] + 1 >= 8
         mm_tiles = -(-3 // cpt)
         mixed = precision == q.QMMM_MIXED
-        vpot = ncls * ch_f + (1 if v_maxsl > 1 else 0) if mixed else 2 * ncls * ch_f
+        vpot = (1 if mixed else 2) * ncls * ch_f + (1 if nI else 0)
         return (10 + (1 if mixed else 0) + (6 if tensor else 2)) + (vpot + 2) + (ncls + 1) + \
             (ncls + 3 * ncls * ch_g + 8 + ((5 + mm_tiles) if mm_tc else 3))
 

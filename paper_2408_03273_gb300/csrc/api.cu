@@ -1347,8 +1347,8 @@ static int ensure_vslices(qmmm_handle *h, int *nbuf)
 
 // qmmm_vpot in parts (a batch runs the mixed V sweeps of all its frames together):
 // vpot_prep clears V, or the per-slice partial matrices when slices is set (then *Vdst points at
-// them and *nbuf is their count); vpot_sweep runs the class sweeps; vpot_end sums the slices, adds
-// the nuclear-MM energy and copies out.
+// them and *nbuf is their count); vpot_sweep runs the class sweeps over the lower triangle; vpot_end sums
+// the slices, mirrors V, adds the nuclear-MM energy and copies out.
 static int vpot_prep(qmmm_handle *h, bool slices, double **Vdst, int *nbuf)
 {
     cudaStream_t st = h->stream;
@@ -1395,7 +1395,7 @@ static int vpot_end(qmmm_handle *h, int nbuf, double *Vout, double *E_nuc_mm, bo
     cudaStream_t st = h->stream;
     int rc;
     const size_t n2 = (size_t)h->nao * h->nao;
-    if (nbuf > 1) CUDA_TRY(launch_sum_slices_d(h->Vslices.p, nbuf, n2, h->V.p, st));
+    if (h->nI > 0) CUDA_TRY(launch_sum_mirror(nbuf > 1 ? h->Vslices.p : h->V.p, nbuf, h->nao, h->V.p, st));
     CUDA_TRY(mark(h, 1));
     if (enuc) {
         CUDA_TRY(launch_enucmm(h->qm.p, h->Zd.p, h->natm, h->rI.p, h->rI_idx.p, h->nI, h->mm_beta.p, h->Epart.p,

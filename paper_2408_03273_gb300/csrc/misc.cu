@@ -117,20 +117,38 @@ cudaError_t launch_unpermute(const double *dq_int, const double *dR_int, const i
     return cudaGetLastError();
 }
 
-__global__ void k_sum_slices_d(const double *src, int nslice, size_t n, double *dst)
+// dst = sum over the slices of src (lower triangles, in order), mirrored: a block per 32 x 32 tile of the
+// lower triangle, transposed through shared memory.  src == dst (one slice): only the upper is written.
+constexpr int SM_T = 32;
+__global__ void __launch_bounds__(256) k_sum_mirror(const double *src, int nslice, int n, double *dst)
 {
-    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int sl = 0; sl < nslice; ++sl) s += src[(size_t)sl * n + k];
-        dst[k] = s;
+    __shared__ double t[SM_T][SM_T + 1];
+    int bi = (int)((sqrtf(8.0f * blockIdx.x + 1.0f) - 1.0f) * 0.5f);  // tile row, blockIdx.x = bi (bi + 1) / 2 + bj
+    while ((long long)bi * (bi + 1) / 2 > blockIdx.x) --bi;
+    while ((long long)(bi + 1) * (bi + 2) / 2 <= blockIdx.x) ++bi;
+    const int bj = (int)(blockIdx.x - (long long)bi * (bi + 1) / 2), x = threadIdx.x & 31;
+    const size_t n2 = (size_t)n * n;
+    for (int y = threadIdx.x >> 5; y < SM_T; y += 8) {
+        const int r = bi * SM_T + y, c = bj * SM_T + x;
+        if (r >= n || c > r) continue;
+        const size_t k = (size_t)r * n + c;
+        double s = src[k];
+        for (int sl = 1; sl < nslice; ++sl) s += src[sl * n2 + k];
+        if (src != dst) dst[k] = s;
+        t[y][x] = s;
+    }
+    __syncthreads();
+    for (int y = threadIdx.x >> 5; y < SM_T; y += 8) {
+        const int r = bj * SM_T + y, c = bi * SM_T + x;  // upper triangle
+        if (c < n && r < c) dst[(size_t)r * n + c] = t[x][y];
     }
 }
 
-cudaError_t launch_sum_slices_d(const double *src, int nslice, size_t n, double *dst, cudaStream_t st)
+cudaError_t launch_sum_mirror(const double *src, int nslice, int n, double *dst, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    const int grid = (int)std::min<size_t>((n + 255) / 256, 8192);
-    k_sum_slices_d<<<grid, 256, 0, st>>>(src, nslice, n, dst);
+    const long long nt = (n + SM_T - 1) / SM_T;
+    k_sum_mirror<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, st>>>(src, nslice, n, dst);
     return cudaGetLastError();
 }
 

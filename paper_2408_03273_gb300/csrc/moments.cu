@@ -277,7 +277,7 @@ k_moments(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ dm, 
             }
             if constexpr (FOCK) {
                 const double v = seg_reduce(-0.5 * coef * f, take);
-                // a shell with itself: one triangle and its mirror, so that F is symmetric bit for bit
+                // a shell with itself: one triangle and its mirror, equal bit for bit
                 if (head && active && (mirror || ia <= ib)) {
                     atomicAdd(F + r * bd.nao + c, v);
                     if (mirror || ia < ib) atomicAdd(F + c * bd.nao + r, v);

@@ -62,6 +62,12 @@ __device__ __forceinline__ double pair_density(const PPLane &pl, const BasisDev 
     return g * (TWO_PI * pl.ip * pl.cab);
 }
 
+// Where an element of V is summed: both of its triangles' elements meet in the lower one, which
+// k_sum_mirror copies to the upper.  Added to each triangle by itself, the contributions of a shell
+// pair that spans three tiles, or of several charge chunks, came in any order and the two elements
+// could differ in the last bit.
+__device__ __forceinline__ size_t lower_index(size_t r, size_t c, int n) { return r >= c ? r * n + c : c * n + r; }
+
 // The centre-A derivative coefficients Da_tuv = sum_ab g_ab E'^a_{tuv}, E'^a the product of Hermite
 // coefficients with the factor of direction a replaced by
 //   E'^{ij}_t = dE^{ij}_t / dX_AB = 2a E^{i+1,j}_t - i E^{i-1,j}_t - (a/p) E^{ij}_{t-1}

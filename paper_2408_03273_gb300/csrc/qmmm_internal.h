@@ -51,8 +51,8 @@ struct qmmm_handle_impl;
 // slice s into V + s * vstride (FP64: slices of the pairs' sums, added before the contraction).  The
 // mixed adjoint (launch_vgrad_f32) sizes its own grid from nsm, the SMs; `variant` picks its charges
 // per lane (cl_variant).
-// dst[k] = sum_s src[s*n + k], s < nslice, in order (the V slices)
-cudaError_t launch_sum_slices_d(const double *src, int nslice, size_t n, double *dst, cudaStream_t st);
+// V (n x n) from the lower triangles of its slices, added in order, and mirrored (src may be dst)
+cudaError_t launch_sum_mirror(const double *src, int nslice, int n, double *dst, cudaStream_t st);
 // sums: scratch of the class, nslice x the Hermite sums of every primitive pair
 cudaError_t launch_vpot_f64(const BasisDev &b, const RegionDev &r, int cls, int pp_begin, int pp_end,
                             int ch_begin, int ch_end, const double *boys, double *V, int *err, int nblk, int threads,

@@ -137,7 +137,7 @@ k_vpot_f32(VJob one, const VJob *__restrict__ jobs, int njob, const float *__res
 
         bool take[5], head;
         seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-        const bool mirror = pl.sp.shA != pl.sp.shB;
+        const bool self = pl.sp.shA == pl.sp.shB;  // a shell with itself: one triangle
 #pragma unroll
         for (int ia = 0; ia < NA; ++ia) {
 #pragma unroll
@@ -154,11 +154,8 @@ k_vpot_f32(VJob one, const VJob *__restrict__ jobs, int njob, const float *__res
                         for (int w = 0; w <= az + bz; ++w) v += exy * Ez[az][bz][w] * W[hidx(t, u, w)];
                     }
                 v = seg_reduce(coef * v, take);
-                if (head && pl.active) {
-                    const size_t r = pl.sp.aoA + ia, c = pl.sp.aoB + ib;
-                    atomicAdd(V + r * bd.nao + c, v);
-                    if (mirror) atomicAdd(V + c * bd.nao + r, v);
-                }
+                if (head && pl.active && (!self || ia <= ib))
+                    atomicAdd(V + lower_index(pl.sp.aoA + ia, pl.sp.aoB + ib, bd.nao), v);
             }
         }
     }

@@ -19,8 +19,9 @@
 // once per slice, into one partial V per slice: sweep of 17 atoms with f shells 1.18 -> 0.70 ms, of a QM
 // water 0.205 -> 0.138 ms, of the 60-atom site 19.8 -> 19.7 ms).  Primitive pairs of a
 // shell pair are summed by a segmented warp-shuffle reduction and the head lane adds the block into
-// V (and its mirror).  A shell pair spans at most two tiles when it has at most 32 primitive pairs,
-// so at most two additions reach any element: the result does not depend on scheduling.
+// the lower triangle of V (mirrored at the end).  A shell pair spans at most two tiles when it has at most
+// 32 primitive pairs, so at most two additions per chunk of charges reach any element: with one chunk the
+// result does not depend on scheduling.
 #include <algorithm>
 
 #include "harm.cuh"
@@ -129,7 +130,7 @@ k_pair_V(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ sums,
     const double coef = -TWO_PI * pl.ip * pl.cab * HALF_SQRT_PI * sqrt(pl.ip);
     bool take[5], head;
     seg_setup(pl.active ? pl.s : -1 - lane, lane, take, head);
-    const bool mirror = pl.sp.shA != pl.sp.shB;
+    const bool self = pl.sp.shA == pl.sp.shB;  // a shell with itself: one triangle
 #pragma unroll 1
     for (int ib = 0; ib < NB; ++ib) {
         int b3[3] = {0, 0, 0};
@@ -156,12 +157,8 @@ k_pair_V(BasisDev bd, int pp_begin, int pp_end, const double *__restrict__ sums,
             v = fma(row[0][t][lane], h, v);
         }
         v = seg_reduce(coef * v, take);
-        // a shell with itself: one triangle and its mirror, so that V is symmetric bit for bit
-        if (head && pl.active && (mirror || ia <= ib)) {
-            const size_t r = pl.sp.aoA + ia, c = pl.sp.aoB + ib;
-            atomicAdd(V + r * bd.nao + c, v);
-            if (mirror || ia < ib) atomicAdd(V + c * bd.nao + r, v);
-        }
+        if (head && pl.active && (!self || ia <= ib))
+            atomicAdd(V + lower_index(pl.sp.aoA + ia, pl.sp.aoB + ib, bd.nao), v);
     }
 }
 
