@@ -57,6 +57,8 @@ def test_launched_block_sizes(small, precision, shape, tmp_path):
             if shape != "default":
                 h.set_tuning(k, [w if shape == "wide" and w else 256 for w in wide])
         (V, g), sizes = _traced(lambda: (h.vpot()[0], h.forces(s.dm)), tmp_path / "trace.json")
+        if not sizes:
+            pytest.skip("no kernel trace (another tool holds the tracer)")
         for k in KINDS[precision]:
             t = h.tuning(k)["threads"]
             for c, n in enumerate(h.info["n_prim_pairs_class"]):
